@@ -225,7 +225,7 @@ rh_status rh_hessvec(rh_grid *grid, const double *W, int64_t ldw, int32_t N,
  * requests on grids of different sizes, computed by ONE kernel launch on
  * `stream` (asynchronous).  Items are independent; item i gets
  * ceil(N_i / width) CTAs (width = target directions per CTA, the right-hand-
- * side interleave width; 0 picks the rh_hessvec default per item).  Up to 32
+ * side interleave width; 0 spreads the items so that they end together).  Up to 32
  * items per launch; larger batches take several launches.
  *   grid    adjoint-ready grid (rh_adjoint for its current state); all items
  *           must be on the same device
@@ -252,7 +252,8 @@ rh_status rh_batch_hessvec(int32_t n_items, const rh_hv_item *items, int32_t wid
 /*
  * Launch configuration of a batched launch (Algorithm 2's level tiles):
  *   width        target directions per CTA (the right-hand-side interleave
- *                width); 0 spreads each item over the SMs' CTA slots
+ *                width); 0 gives each item the directions per CTA with which all
+ *                items' CTAs fit the SMs' slots at once and end together
  *   threads      CTA size, one of the compiled shapes 128, 192, 256, 384,
  *                resident at 6, 4, 3, 2 CTAs per SM (768 threads an SM each);
  *                0 takes 384.  A CTA's level of a sweep is one barrier: small

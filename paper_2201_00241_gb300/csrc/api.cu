@@ -637,6 +637,53 @@ __global__ void k_rto_apply(int n_p, int n_bus, const int* info, const double* p
 
 int nblk(int n, int t) { return (n + t - 1) / t; }
 
+// CTAs of each item of a batched launch whose width is left to the library.  A CTA with D
+// directions of a grid takes about
+//   t(D) = kLevelUs x (levels of the four sweeps) + kFlopUs x (flops of a direction) x D,
+// with the SM's CTA slots occupied (fitted on GB300: the 9241-bus grid takes 2.0 ms at
+// D = 1 and 5.6 ms at D = 10, the 1354-bus grid 0.40 ms at D = 4).  The items run side by
+// side, so the launch ends with its slowest CTA: the least T is taken for which every
+// item, at the most directions per CTA that end by T, gets all its CTAs into the slots at
+// once.  One CTA a direction instead, whatever the batch, puts a batch of many
+// directions through the slots in several waves of the latency-bound sweeps: a round of
+// 15 requests (118 to 9241 buses, 1920 directions) took 5.6 ms, 8 x 64 directions on the
+// 1354-bus grid 0.92 ms.
+void spread_batch(const rh_hv_item* items, int n, int slots, int* G) {
+    constexpr double kLevelUs = 4.5, kFlopUs = 0.27e-3;
+    std::vector<double> a(n), b(n);
+    std::vector<int> cap(n);
+    double lo = 0.0, hi = 0.0;
+    for (int k = 0; k < n; k++) {
+        const auto& S = items[k].grid->S;
+        const int T = S.n_x - S.t0;
+        const double flops = 4.0 * (double)S.jp_col.size() + 4.0 * (S.nnz_l + S.nnz_u - S.n_x) +
+                             8.0 * (double)S.yj.size();
+        a[k] = kLevelUs * (2.0 * S.n_flev + 2.0 * S.n_blev);
+        b[k] = kFlopUs * flops;
+        // at most 256 directions, and the dense tail's rows in shared memory
+        cap[k] = T > 1 ? std::max(1, rh::dirs_tail_cap() / T) : 256;
+        cap[k] = std::min(std::min(cap[k], 256), std::max(1, items[k].N));
+        lo = std::max(lo, items[k].N > 0 ? a[k] + b[k] : 0.0);
+        hi = std::max(hi, a[k] + b[k] * cap[k]);
+    }
+    auto ctas = [&](double t) {
+        int64_t sum = 0;
+        for (int k = 0; k < n; k++) {
+            const int D = std::max(1, (int)std::min((double)cap[k], std::floor((t - a[k]) / b[k])));
+            // the fewest CTAs with at most D directions
+            G[k] = items[k].N > 0 ? (items[k].N + D - 1) / D : 0;
+            sum += G[k];
+        }
+        return sum;
+    };
+    if (ctas(lo) <= slots) return;
+    for (int it = 0; it < 40; it++) {
+        const double mid = 0.5 * (lo + hi);
+        (ctas(mid) <= slots ? hi : lo) = mid;
+    }
+    ctas(hi);
+}
+
 }  // namespace
 
 extern "C" {
@@ -1673,13 +1720,15 @@ rh_status rh_batch_hessvec_cfg(int32_t n_items, const rh_hv_item* items, const r
     std::unique_ptr<rh::DirBatch> B(new rh::DirBatch());
     for (int first = 0; first < n_items; first += rh::kMaxBatch) {
         int n = std::min(rh::kMaxBatch, n_items - first);
+        int spread[rh::kMaxBatch];
+        if (width == 0) spread_batch(items + first, n, rh::dirs_batch_slots(threads), spread);
         B->n_items = 0;
         B->cta_ptr[0] = 0;
         for (int k = 0; k < n; k++) {
             const rh_hv_item& it = items[first + k];
             if (it.N == 0) continue;
             rh_grid* g = it.grid;
-            int G = width > 0 ? (it.N + width - 1) / width : rh::dirs_ctas_for(it.N, rh::dirs_batch_slots(threads));
+            int G = width > 0 ? (it.N + width - 1) / width : spread[k];
             G = std::max(G, (it.N + 255) / 256);
             rh::DirLaunch& L = B->l[B->n_items];
             L.N = it.N;

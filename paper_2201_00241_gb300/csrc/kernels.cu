@@ -2284,6 +2284,8 @@ int dirs_ctas_for(int N, int slots) {
 
 int dirs_default_ctas(int N) { return dirs_ctas_for(N, kDirCtasPerSm * num_sms()); }
 
+int dirs_tail_cap() { return kPartCap; }
+
 bool dirs_tail_fits(int T, int N, int n_cta) {
     if (T <= 1 || n_cta <= 0) return false;
     int dmax = (N + n_cta - 1) / n_cta;

@@ -292,6 +292,7 @@ void launch_dirs(const DirGrid& g, const DirLaunch& L, cudaStream_t st);
 // raise the dynamic shared-memory limits of the kernels that need it (once per grid)
 cudaError_t prepare_kernels();
 bool dirs_tail_fits(int T, int N, int n_cta);
+int dirs_tail_cap();       // dense-tail rows x directions a CTA can hold
 // dense tail triangles of the current factors (pos: T*T map to A, -1 where structurally zero)
 // x[r][c] *= s[r] for r < n, c < N
 void launch_scale_rows(int n, int N, const double* s, double* x, int64_t ld, cudaStream_t st);

@@ -44,7 +44,7 @@ class _Desc(C.Structure):
 
 
 class HvConfig(C.Structure):
-    """rh_hv_config: width (directions per CTA, 0 = spread over the SMs), threads
+    """rh_hv_config: width (directions per CTA, 0 = items spread to end together), threads
     (CTA shape 128, 192, 256 or 384; 0 = 384), split_lanes (narrow-level k-split
     cap, a power of two <= 32; 0 = 32)."""
     _fields_ = [("width", C.c_int32), ("threads", C.c_int32), ("split_lanes", C.c_int32)]
