@@ -74,11 +74,16 @@ struct rh_grid {
     int *sbr_ptr = nullptr, *sbr_maxext = nullptr;
     int4* sbr_slot = nullptr;
     int n_sbr = 0;
+    // k_solve1's schedules (LineSched) and line arrays; n_line < 0: its descriptors do not fit
+    int4 *line_up = nullptr, *line_down = nullptr;
+    int *line_col = nullptr, *line_map = nullptr;
+    double *line_val = nullptr, *line_tval = nullptr;
+    int n_line_up = 0, n_line_down = 0, n_line = -1;
+    int line_off[3] = {0, 0, 0};                  // first entries of bwd, fwd's vt and bwd's vt
     int* tail_pos = nullptr;
     int *qtheta = nullptr, *bparent = nullptr;
     int *jp_rows = nullptr, *jp_zero_rows = nullptr;
     int n_jp_rows = 0, n_jp_zero = 0;
-    double *triL = nullptr, *triU = nullptr, *triUt = nullptr, *triLt = nullptr;
     // unit-diagonal factors of the direction kernel (J_x = D L'' U')
     double *Ad = nullptr, *Atd = nullptr, *jptvd = nullptr;
     int* arow = nullptr;   // row of every position of A
@@ -104,7 +109,7 @@ struct rh_grid {
 
     // --- device: state ----------------------------------------------------
     double *vm = nullptr, *va = nullptr, *pg = nullptr, *pd = nullptr, *qd = nullptr, *P = nullptr, *Q = nullptr;
-    double *A = nullptr, *At = nullptr, *invdiag = nullptr, *jpv = nullptr, *jptv = nullptr;
+    double *A = nullptr, *invdiag = nullptr, *jpv = nullptr, *jptv = nullptr;
     double *gres = nullptr, *lam = nullptr, *grad = nullptr, *v1 = nullptr;
     double4_32a* inc_coef = nullptr;
     double *d2 = nullptr, *asum = nullptr, *csum = nullptr, *pg_curv = nullptr, *gref_th = nullptr,
@@ -215,7 +220,7 @@ struct rh_grid {
         rh::DirGrid g;
         g.n_x = S.n_x; g.n_p = S.n_p; g.zero_row = S.n_x + S.n_p;
         g.nnz = (int)S.col.size();
-        g.col = col; g.A = A; g.At = At; g.invdiag = invdiag;
+        g.col = col; g.invdiag = invdiag;
         g.lf = {S.n_flev, flev_ptr, fslot, flev_maxext};
         g.lb = {S.n_blev, blev_ptr, bslot, blev_maxext};
         g.sf = {n_sf, sf_ptr, sf_slot, sf_maxext};
@@ -224,7 +229,6 @@ struct rh_grid {
         g.ef = {n_ef, ef_ptr, ef_slot, ef_maxext};
         g.t0 = S.t0; g.T = S.n_x - S.t0;
         g.ks_cap = 32;
-        g.triL = triL; g.triU = triU; g.triUt = triUt; g.triLt = triLt;
         g.Ad = Ad; g.Atd = Atd; g.jptvd = jptvd;
         g.triLd = triLd; g.triUd = triUd; g.triUtd = triUtd; g.triLtd = triLtd;
         g.qtheta = qtheta; g.bparent = bparent;
@@ -236,6 +240,21 @@ struct rh_grid {
         g.d2 = d2; g.asum = asum; g.csum = csum; g.has_gref = has_gref; g.gref_th = gref_th; g.gref_v = gref_v;
         g.n_gref = n_gref; g.gref_row = gref_row; g.gref_val = gref_val; g.c2ref = dscal + 1;
         g.pg_row = pg_row; g.pg_curv = pg_curv;
+        return g;
+    }
+    rh::LineGrid s1() const {
+        rh::LineGrid g;
+        g.n_x = S.n_x; g.t0 = S.t0; g.T = S.n_x - S.t0;
+        const double *v = line_val, *t = line_tval;
+        const int *up = line_col, *down = line_col + line_off[0];
+        g.up = {n_line_up, line_up, up, v, v + line_off[1]};
+        g.down = {n_line_down, line_down, down, v + line_off[0], v + line_off[2]};
+        g.tup = {n_line_up, line_up, up, t, t + line_off[1]};
+        g.tdown = {n_line_down, line_down, down, t + line_off[0], t + line_off[2]};
+        g.n_line = n_line; g.map = line_map; g.arow = arow; g.col = col; g.tpos = tpos; g.diagpos = diagpos;
+        g.line = line_val; g.tline = line_tval;
+        g.A = A; g.invdiag = invdiag;
+        g.triLd = triLd; g.triUd = triUd; g.triUtd = triUtd; g.triLtd = triLtd;
         return g;
     }
     rh::RfGrid rf() const {
@@ -291,6 +310,118 @@ std::vector<int> tree_column_order(const rh::Symbolic& S) {
     }
     std::stable_sort(cm.begin(), cm.end(), [&](int a, int b) { return anchor[a] < anchor[b]; });
     return cm;
+}
+
+// The steps of a sweep over the levels ptr[l] .. ptr[l + 1] of `slots`, for CTAs of NT
+// threads: the buses of a level by descending number of lanes, side by side (a group
+// starts at a multiple of its size), in rounds of NT, or on one half of the warps and the
+// other in turn where they fit; the level's last round ends in a barrier.  A level's groups are those that cost its busiest sub-partition, or its longest
+// warp, the fewest FP64 instructions (64 cycles each; a shuffle takes as long): at most m
+// entries a lane, for m = 1, 2, 4, ...  False: a row is too long for the descriptors.
+struct LineHost {
+    std::vector<int4> steps;
+    std::vector<int> map, col, vt;       // entries' positions in A (-1: a pad) and columns; buses' own entries
+};
+bool line_steps(const std::vector<int>& ptr, const std::vector<int4>& slots, const std::vector<int>& col, bool up,
+                int flags, int NT, LineHost& L) {
+    struct Bus {
+        int lg, t;
+        bool two;
+    };
+    std::vector<Bus> best, cur;
+    bool half = false;           // the last level took the first half of the warps
+    for (size_t l = 0; l + 1 < ptr.size(); l++) {
+        if (ptr[l + 1] == ptr[l]) continue;
+        double least = 0.0;
+        best.clear();
+        for (int m = 1; m <= 64; m *= 2) {
+            cur.clear();
+            for (int t = ptr[l]; t < ptr[l + 1]; t++) {
+                const bool two = slots[t].w >= 0;
+                int lg = 0;
+                while (lg < (two ? 4 : 5) && (m << lg) < slots[t].y) lg++;
+                cur.push_back({lg, t, two});
+            }
+            std::stable_sort(cur.begin(), cur.end(),
+                             [](const Bus& x, const Bus& y) { return x.lg + x.two > y.lg + y.two; });
+            double pipe[4] = {0, 0, 0, 0}, longest = 0.0;
+            int lane = 0, warp = 0, e = 0, lg = 0;
+            auto close = [&] {
+                const double fp = e + std::max(0, e - rh::kLinePre) + lg + 1;
+                pipe[(warp % (NT / 32)) & 3] += fp;
+                longest = std::max(longest, fp + lg);
+                warp++;
+                lane = e = lg = 0;
+            };
+            for (const Bus& b : cur) {
+                const int size = 1 << (b.lg + b.two);
+                if (lane + size > 32) close();
+                lane += size;
+                e = std::max(e, (slots[b.t].y + (1 << b.lg) - 1) >> b.lg);
+                lg = std::max(lg, b.lg);
+            }
+            if (lane) close();
+            const double cost = std::max(longest, std::max(std::max(pipe[0], pipe[1]), std::max(pipe[2], pipe[3])));
+            if (best.empty() || cost < least) {
+                least = cost;
+                best.swap(cur);
+            }
+        }
+        // lanes of the level: the bus and its row's first position, then the warps' blocks
+        struct Lane {
+            int slot, lg, li, r0;      // slot -1: idle
+            bool lead;
+        };
+        std::vector<Lane> lanes;
+        for (const Bus& b : best) {
+            const int4 s = slots[b.t];
+            for (int r = 0; r < (b.two ? 2 : 1); r++)
+                for (int li = 0; li < (1 << b.lg); li++)
+                    lanes.push_back({b.t, b.lg, li, r ? s.w : s.z, r == 0 && li == 0});
+        }
+        const Lane idle = {-1, 0, 0, 0, false};
+        while (lanes.size() % 32) lanes.push_back(idle);
+        // a level that fits half the warps takes the half that the step before left idle
+        if (lanes.size() <= (size_t)NT / 2 && half) lanes.insert(lanes.begin(), NT / 2, idle);
+        half = lanes.size() <= (size_t)NT / 2;
+        while (lanes.size() % NT) lanes.push_back(idle);
+        for (size_t k = 0; k < lanes.size(); k += 32) {
+            int lg = 0, cnt = 0, on = 0;
+            for (size_t i = k; i < k + 32; i++) {
+                if (lanes[i].slot < 0) continue;
+                const int l = lanes[i].lg;
+                lg = std::max(lg, l);
+                cnt = std::max(cnt, (slots[lanes[i].slot].y + (1 << l) - 1) >> l);
+                on = rh::kLineActive;
+            }
+            if (cnt > rh::kLineCntMask) return false;
+            const int base = (int)L.map.size();
+            const int w0 = flags | on | cnt | (lg << rh::kLineWlg) | (k + NT >= lanes.size() ? rh::kLineSync : 0);
+            for (int e = 0; e < cnt; e++)
+                for (size_t i = k; i < k + 32; i++) {
+                    const Lane& ln = lanes[i];
+                    const int at = ln.slot < 0 ? 0 : ln.li + (e << ln.lg);
+                    const bool in = ln.slot >= 0 && at < slots[ln.slot].y;
+                    L.map.push_back(in ? ln.r0 + at : -1);
+                    L.col.push_back(in ? col[ln.r0 + at] : 0);
+                }
+            for (size_t i = k; i < k + 32; i++) {
+                const Lane& ln = lanes[i];
+                int4 d = make_int4(-1, base, -1, w0);
+                if (ln.slot >= 0) {
+                    const int4 s = slots[ln.slot];
+                    d.x = s.x;
+                    d.w |= (ln.lg << rh::kLineLg) | (s.w >= 0 ? rh::kLineSplit : 0);
+                    if (ln.lead && s.w >= 0 && !(flags & rh::kLineExt)) {
+                        d.z = (int)L.vt.size();
+                        L.vt.push_back(up ? s.w + s.y : s.z - 1);
+                    }
+                }
+                L.steps.push_back(d);
+            }
+        }
+    }
+    return true;
 }
 
 rh_status set_device(const rh_grid* g) {
@@ -373,15 +504,17 @@ rh_status assemble(rh_grid* g, int method, double* gres, cudaStream_t s) {
     return RH_OK;
 }
 
-// Transposed values, the direction kernel's unit-diagonal factors and the dense
-// tail's triangles from the current LU (enqueue only).
-void enqueue_factor_copies(rh_grid* g, cudaStream_t s) {
+// From the current LU: the direction kernel's unit-diagonal factors and J_p, the dense
+// tail's triangles, and the single solves' line arrays (enqueue only).  newton: only what a
+// Newton step reads.
+void enqueue_factor_copies(rh_grid* g, cudaStream_t s, bool newton = false) {
     const auto& S = g->S;
-    rh::launch_transpose_values((int)S.col.size(), g->tpos, g->arow, g->col, g->diagpos, g->A, g->invdiag, g->At,
-                                g->Ad, g->Atd, (int)S.jp_col.size(), g->jpt_src, g->jpt_row, g->jpv, g->jptv,
-                                g->jptvd, s);
-    rh::launch_build_tail(S.n_x - S.t0, S.t0, g->tail_pos, g->A, g->invdiag, g->triL, g->triU, g->triUt, g->triLt,
-                          g->triLd, g->triUd, g->triUtd, g->triLtd, s);
+    const bool line = g->n_line >= 0;
+    if (!newton || !line)
+        rh::launch_transpose_values((int)S.col.size(), g->tpos, g->arow, g->col, g->diagpos, g->A, g->invdiag, g->Ad,
+                                    g->Atd, (int)S.jp_col.size(), g->jpt_src, g->jpt_row, g->jpv, g->jptv, g->jptvd, s);
+    if (line) rh::launch_line_values(g->s1(), !newton, s);
+    rh::launch_build_tail(S.n_x - S.t0, S.t0, g->tail_pos, g->A, g->invdiag, g->triLd, g->triUd, g->triUtd, g->triLtd, s);
 }
 
 // L2 prefetch of the refactorisation's level data, read level by level after
@@ -576,9 +709,9 @@ rh_status dirs(rh_grid* g, int N, int64_t ld, double* V, double* T, const double
 // fewer CTAs than the device holds leaves free (k_solve1's shared-memory x
 // needs a shared-memory carveout that an SM running k_dirs does not have).
 rh_status solve_one(rh_grid* g, unsigned phases, cudaStream_t s, bool beside_dirs = false) {
-    const int mode = beside_dirs ? 0 : rh::solve1_mode(g->S.n_x, g->S.n_x - g->S.t0);
+    const int mode = beside_dirs || g->n_line < 0 ? 0 : rh::solve1_mode(g->S.n_x, g->S.n_x - g->S.t0);
     if (mode > 0) {
-        RH_CUDA(rh::launch_solve1(g->dir(), g->v1, phases, mode == 2, s));
+        RH_CUDA(rh::launch_solve1(g->s1(), g->v1, (phases & rh::PH_LT) != 0, mode == 2, s));
         return RH_OK;
     }
     // through k_dirs, whose factors are unit-diagonal (J_x = D L'' U'): the right-hand
@@ -896,6 +1029,37 @@ rh_status rh_grid_create(const rh_grid_desc* d, int32_t device, rh_grid** out) {
         RH_CUDA(g->upload(g->sb_ptr, sbp));
         RH_CUDA(g->upload(g->sb_slot, sbs));
         RH_CUDA(g->upload(g->sb_maxext, sbm));
+        {
+            // the single solves sweep the sparse part and solve the dense tail, or, where
+            // the tail's triangle does not fit in shared memory, sweep every level
+            const int mode = rh::solve1_mode(S.n_x, S.n_x - S.t0), NT = rh::line_threads(S.n_x);
+            LineHost up, down;
+            bool ok = mode > 0;
+            if (mode == 2) {
+                ok = line_steps(sfp, sfs, S.col, true, 0, NT, up) &&
+                     line_steps(efp, efs, S.col, true, rh::kLineExt, NT, up) &&
+                     line_steps(sbp, sbs, S.col, false, 0, NT, down);
+            } else if (mode == 1) {
+                ok = line_steps(S.flev_ptr, fs, S.col, true, 0, NT, up) &&
+                     line_steps(S.blev_ptr, bs, S.col, false, 0, NT, down);
+            }
+            if (ok) {
+                g->n_line_up = (int)(up.steps.size() / NT);
+                g->n_line_down = (int)(down.steps.size() / NT);
+                g->line_off[0] = (int)up.map.size();
+                g->line_off[1] = g->line_off[0] + (int)down.map.size();
+                g->line_off[2] = g->line_off[1] + (int)up.vt.size();
+                for (const std::vector<int>* v : {&down.map, &up.vt, &down.vt}) up.map.insert(up.map.end(), v->begin(), v->end());
+                up.col.insert(up.col.end(), down.col.begin(), down.col.end());
+                g->n_line = (int)up.map.size();
+                RH_CUDA(g->upload(g->line_up, up.steps));
+                RH_CUDA(g->upload(g->line_down, down.steps));
+                RH_CUDA(g->upload(g->line_col, up.col));
+                RH_CUDA(g->upload(g->line_map, up.map));
+                RH_CUDA(g->alloc(g->line_val, up.map.size()));
+                RH_CUDA(g->alloc(g->line_tval, up.map.size()));
+            }
+        }
         RH_CUDA(g->upload(g->ef_ptr, efp));
         RH_CUDA(g->upload(g->ef_slot, efs));
         RH_CUDA(g->upload(g->ef_maxext, efm));
@@ -919,10 +1083,6 @@ rh_status rh_grid_create(const rh_grid_desc* d, int32_t device, rh_grid** out) {
         RH_CUDA(g->upload(g->qtheta, qth));
         RH_CUDA(g->upload(g->bparent, bpar));
         size_t ntri = T > 1 ? (size_t)T * (T - 1) / 2 : 1;
-        RH_CUDA(g->alloc(g->triL, ntri));
-        RH_CUDA(g->alloc(g->triU, ntri));
-        RH_CUDA(g->alloc(g->triUt, ntri));
-        RH_CUDA(g->alloc(g->triLt, ntri));
         RH_CUDA(g->alloc(g->triLd, ntri));
         RH_CUDA(g->alloc(g->triUd, ntri));
         RH_CUDA(g->alloc(g->triUtd, ntri));
@@ -981,7 +1141,6 @@ rh_status rh_grid_create(const rh_grid_desc* d, int32_t device, rh_grid** out) {
     RH_CUDA(g->alloc(g->P, nb));
     RH_CUDA(g->alloc(g->Q, nb));
     RH_CUDA(g->alloc(g->A, S.col.size()));
-    RH_CUDA(g->alloc(g->At, S.col.size()));
     RH_CUDA(g->alloc(g->Ad, S.col.size()));
     RH_CUDA(g->alloc(g->Atd, S.col.size()));
     RH_CUDA(g->alloc(g->invdiag, nx));
@@ -1111,7 +1270,7 @@ rh_status rh_powerflow(rh_grid* g, const double* x0, double tol, int32_t max_ite
             [&]() -> rh_status {
                 RH_CUDA(rh::launch_refactor(g->rf(), S.rf_lev_ptr.data(), S.rf_tgt_lev_ptr.data(),
                                             S.rf_piv_lev_ptr.data(), S.rf_n_lev, g->stream));
-                enqueue_factor_copies(g, g->stream);
+                enqueue_factor_copies(g, g->stream, true);
                 RH_CUDA(cudaGetLastError());
                 return RH_OK;
             },
@@ -1305,7 +1464,7 @@ rh_status enqueue_batch_newton(rh_grid* const* items, int n, uint32_t mask, int 
     for (int k = 0; k < B->n; k++) R->g[k] = act[k]->rf();
     RH_CUDA(rh::launch_refactor_batch(*R, S.rf_lev_ptr.data(), S.rf_tgt_lev_ptr.data(), S.rf_piv_lev_ptr.data(), S.rf_n_lev, s));
     const int T = S.n_x - S.t0;
-    const int mode = rh::solve1_mode(S.n_x, T);
+    const int mode = g0->n_line < 0 ? 0 : rh::solve1_mode(S.n_x, T);
     if (mode == 2) {
         std::unique_ptr<rh::TriBatch> tb(new rh::TriBatch());
         tb->n = B->n;
@@ -1315,8 +1474,8 @@ rh_status enqueue_batch_newton(rh_grid* const* items, int n, uint32_t mask, int 
             tb->pos[k] = act[k]->tail_pos;
             tb->A[k] = act[k]->A;
             tb->invdiag[k] = act[k]->invdiag;
-            tb->triL[k] = act[k]->triL;
-            tb->triU[k] = act[k]->triU;
+            tb->triLd[k] = act[k]->triLd;
+            tb->triUd[k] = act[k]->triUd;
         }
         rh::launch_tail_tri_batch(*tb, s);
     }
@@ -1324,10 +1483,10 @@ rh_status enqueue_batch_newton(rh_grid* const* items, int n, uint32_t mask, int 
         std::unique_ptr<rh::Solve1Batch> sb(new rh::Solve1Batch());
         sb->n = B->n;
         for (int k = 0; k < B->n; k++) {
-            sb->g[k] = act[k]->dir();
+            sb->g[k] = act[k]->s1();
             sb->x[k] = act[k]->v1;
         }
-        RH_CUDA(rh::launch_solve1_batch(*sb, rh::PH_L | rh::PH_U, mode == 2, S.n_x, T, s));
+        RH_CUDA(rh::launch_solve1_batch(*sb, mode == 2, S.n_x, T, s));
     } else {
         // x does not fit in one CTA's shared memory: the direction kernel solves each item
         for (rh_grid* g : act) {

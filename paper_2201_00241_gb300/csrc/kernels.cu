@@ -837,7 +837,7 @@ __device__ __forceinline__ double unit_scale(const double* A, const int* diagpos
 __global__ void k_transpose_values(int nnz, const int* __restrict__ tpos, const int* __restrict__ arow,
                                    const int* __restrict__ col, const int* __restrict__ diagpos,
                                    const double* __restrict__ A, const double* __restrict__ invdiag,
-                                   double* __restrict__ At, double* __restrict__ Ad, double* __restrict__ Atd,
+                                   double* __restrict__ Ad, double* __restrict__ Atd,
                                    int nnz_jp, const int* __restrict__ jpt_src, const int* __restrict__ jpt_row,
                                    const double* __restrict__ jpv, double* __restrict__ jptv,
                                    double* __restrict__ jptvd) {
@@ -845,7 +845,6 @@ __global__ void k_transpose_values(int nnz, const int* __restrict__ tpos, const 
     if (i < nnz) {
         const int r = arow[i], c = col[i];
         const double at = A[tpos[i]];
-        At[i] = at;
         Ad[i] = r == c ? 1.0 : A[i] * unit_scale(A, diagpos, invdiag, r, c);
         Atd[i] = r == c ? 1.0 : at * unit_scale(A, diagpos, invdiag, c, r);
     }
@@ -866,11 +865,10 @@ __global__ void k_scale_rows(int n, int N, const double* __restrict__ s, double*
     x[(int64_t)r * ld + c] *= s[r];
 }
 
-// The dense tail's triangles: for the single solves (columns of U scaled by
-// 1/u_jj), and of the unit-diagonal factors L'', U' for the direction kernel.
-__device__ __forceinline__ void k_build_tail_body(int T, int t0, const int* __restrict__ pos, const double* __restrict__ A,
-                             const double* __restrict__ invdiag, double* triL, double* triU, double* triUt,
-                             double* triLt, double* triLd, double* triUd, double* triUtd, double* triLtd) {
+// The dense tail's triangles of the unit-diagonal factors L'', U' and their transposes.
+__global__ void k_build_tail(int T, int t0, const int* __restrict__ pos, const double* __restrict__ A,
+                             const double* __restrict__ invdiag, double* triLd, double* triUd, double* triUtd,
+                             double* triLtd) {
     int idx = blockIdx.x * blockDim.x + threadIdx.x;
     if (idx >= T * T) return;
     int i = idx / T, j = idx - i * T;
@@ -880,21 +878,14 @@ __device__ __forceinline__ void k_build_tail_body(int T, int t0, const int* __re
     const double ii = invdiag[t0 + i], ij = invdiag[t0 + j];
     if (i > j) {
         int o = j * (T - 1) - j * (j - 1) / 2 + (i - j - 1);
-        triL[o] = aij;                              // L_ij
-        triUt[o] = aji * ij;                        // (U^T)_ij = U_ji, scaled by 1/u_jj
         triLd[o] = aij * A[pos[j * T + j]] * ii;    // L''_ij
         triUtd[o] = aji * ij;                       // (U'^T)_ij = U'_ji
     } else {
         int o = j * (j - 1) / 2 + i;
-        triU[o] = aij * ij;                         // U_ij scaled by 1/u_jj
-        triLt[o] = aji;                             // (L^T)_ij = L_ji
         triUd[o] = aij * ii;                        // U'_ij
         triLtd[o] = aji * A[pos[i * T + i]] * ij;   // (L''^T)_ij = L''_ji
     }
 }
-__global__ void k_build_tail(int T, int t0, const int* __restrict__ pos, const double* __restrict__ A,
-                             const double* __restrict__ invdiag, double* triL, double* triU, double* triUt,
-                             double* triLt, double* triLd, double* triUd, double* triUtd, double* triLtd) { k_build_tail_body(T, t0, pos, A, invdiag, triL, triU, triUt, triLt, triLd, triUd, triUtd, triLtd); }
 
 // ---------------------------------------------------------------------------
 // the direction kernel: Algorithm 2 for a slice of directions per CTA
@@ -1221,8 +1212,8 @@ constexpr int kTailB = 16;
 __device__ __forceinline__ double tri_l(const double* src, int T, int i, int j) { return src[lpack_off(j, T) + (i - j - 1)]; }
 __device__ __forceinline__ double tri_u(const double* src, int i, int j) { return src[upack_off(j) + i]; }
 
-template <bool SCALE>
-__device__ void tail_fwd(const DirGrid& g, const double* __restrict__ tri_g, double* X, int64_t ld, int c0, int D,
+template <bool SCALE, class Grid>
+__device__ void tail_fwd(const Grid& g, const double* __restrict__ tri_g, double* X, int64_t ld, int c0, int D,
                          double* xt, double* tri) {
     const int T = g.T, t0 = g.t0;
     const int ntri = T * (T - 1) / 2;
@@ -1273,8 +1264,8 @@ __device__ void tail_fwd(const DirGrid& g, const double* __restrict__ tri_g, dou
     __syncthreads();
 }
 
-template <bool SCALE>
-__device__ void tail_bwd(const DirGrid& g, const double* __restrict__ tri_g, double* X, int64_t ld, int c0, int D,
+template <bool SCALE, class Grid>
+__device__ void tail_bwd(const Grid& g, const double* __restrict__ tri_g, double* X, int64_t ld, int c0, int D,
                          double* xt, double* tri) {
     const int T = g.T, t0 = g.t0;
     const int ntri = T * (T - 1) / 2;
@@ -1641,211 +1632,139 @@ __global__ void __launch_bounds__(NT, MINB) k_dirs_batch(DirBatch B) {
     dirs_body(sg, sl, (int)blockIdx.x - B.cta_ptr[item], part, sref, nullptr);
 }
 
-// Sweeps of a single right-hand side held in shared memory (k_solve1).  There
-// is nothing to coalesce, so each bus block of a level takes a group of G
-// lanes (G a power of two, G * nb <= blockDim): the lanes stride over the row
-// and combine their sums with warp shuffles in log2(G) steps, and lane 0 of the
-// group finishes the block.  One barrier per level.  (Spreading a level over a
-// thread-block cluster with x replicated through distributed shared memory was
-// slower: a level's cost is its chain of dependent loads, which more CTAs do not
-// shorten, and a cluster barrier costs more than a CTA barrier.)
-__device__ __forceinline__ int group_size(int nb, int maxext, int threads) {
-    int G = 1;
-    while (G < 32 && 2 * G * nb <= threads && G < maxext) G *= 2;
-    return G;
-}
-
-// s0 -= sum v0[e] x[col[e]], s1 likewise, over e = e0, e0 + G, ... < n; unrolled by
-// 4 so that four independent index/value loads (L2: read once per solve) are in
-// flight per lane.
-__device__ __forceinline__ void row1_sub(const int* __restrict__ col, const double* __restrict__ vals, int r0, int r1,
-                                         int e0, int n, int G, const double* X, bool two, double& s0, double& s1) {
-    int e = e0;
-    for (; e + 3 * G < n; e += 4 * G) {
-        const int i0 = col[r0 + e], i1 = col[r0 + e + G], i2 = col[r0 + e + 2 * G], i3 = col[r0 + e + 3 * G];
-        const double u0 = vals[r0 + e], u1 = vals[r0 + e + G], u2 = vals[r0 + e + 2 * G], u3 = vals[r0 + e + 3 * G];
-        double w0 = 0.0, w1 = 0.0, w2 = 0.0, w3 = 0.0;
-        if (two) {
-            w0 = vals[r1 + e];
-            w1 = vals[r1 + e + G];
-            w2 = vals[r1 + e + 2 * G];
-            w3 = vals[r1 + e + 3 * G];
-        }
-        const double x0 = X[i0], x1 = X[i1], x2 = X[i2], x3 = X[i3];
-        s0 = fma(-u0, x0, s0);
-        s0 = fma(-u1, x1, s0);
-        s0 = fma(-u2, x2, s0);
-        s0 = fma(-u3, x3, s0);
-        if (two) {
-            s1 = fma(-w0, x0, s1);
-            s1 = fma(-w1, x1, s1);
-            s1 = fma(-w2, x2, s1);
-            s1 = fma(-w3, x3, s1);
-        }
-    }
-    for (; e < n; e += G) {
-        const double xv = X[col[r0 + e]];
-        s0 = fma(-vals[r0 + e], xv, s0);
-        if (two) s1 = fma(-vals[r1 + e], xv, s1);
-    }
-}
-
-// sum of s over the G lanes of a group (G <= 32; groups are whole and aligned in
-// the warp)
-__device__ __forceinline__ void group_sum(int it, int items, int G, double& s0, double& s1) {
-    if (G == 1) return;
-    const int live = items - (it - (int)(threadIdx.x & 31));      // lanes of this warp holding an item
-    const unsigned m = live >= 32 ? 0xffffffffu : ((1u << live) - 1u);
-    for (int off = G / 2; off > 0; off >>= 1) {
-        s0 += __shfl_down_sync(m, s0, off, G);
-        s1 += __shfl_down_sync(m, s1, off, G);
-    }
-}
-
-// The first item of a level for one thread, with everything it needs that does
-// not depend on x: its slot, the first four (column, value) pairs of its share
-// of the row and the finishing data.  Loaded for the next level before the
-// barrier that ends the current one, so that after the barrier only the
-// shared-memory reads of x and the FMAs remain on the critical path (for rows
-// whose share is longer than four entries the rest is loaded as before).
-struct Pf1 {
-    int4 sl;
-    int i[4];
-    double u[4], w[4];
-    double inv0, inv1, vt;
-    bool valid;
+// Sweeps of a right-hand side held in shared memory.  There is nothing to coalesce, so
+// each row takes a group of G adjacent lanes (a power of two, at most 16 for the two rows
+// of a bus, 32 for one): the lanes stride over the row and combine their sums with warp
+// shuffles in log2(G) steps, and the first lane of the bus finishes it.
+//
+// The schedule is laid out on the host (line_steps in api.cu) as steps of one descriptor
+// per thread, {q, base, b, w}: theta row of the bus (-1: idle lane), the warp's first entry
+// in the line arrays, the bus's place in the schedule, and w (see LineBits).  Entry k of the
+// warp's lane l is at base + 32 k + l of the column indices and of the values, which
+// k_line_values copies there from the factors (negated) before the solve: every load of a
+// warp is one contiguous run.  Read from the factors' rows instead, a warp's load touches a
+// 32-byte sector per row for 8 bytes, and one SM's L2 path bounds the solve: 1.25 M cycles for
+// the two sweeps of the 9241-bus grid.
+//
+// A descriptor's address depends on the step's number alone, so the descriptors are read
+// three steps ahead and the row data one step ahead, while a step is reduced and finished;
+// between two barriers a level reads x from shared memory, multiplies, shuffles and
+// finishes.  A lone warp issues an instruction every 4-5 cycles, so a narrow level is given
+// to one half of the warps and the next to the other half: a half loads its row data while
+// the other computes.  Wide levels take all warps for as many rounds as they need.  FP64
+// instructions hold a sub-partition's pipe 64 cycles whatever their lanes do, so line_steps
+// counts those of each level's busiest sub-partition and longest warp for each group size
+// and takes the least.
+// (Spreading a level over a thread-block cluster with x replicated through distributed
+// shared memory was slower: more CTAs do not shorten a level's chain, and a cluster
+// barrier costs more than a CTA barrier.)
+struct LineAhead {
+    int i[kLinePre];
+    double u[kLinePre];
+    double vt;                 // the bus's own off-diagonal entry
 };
 
-template <bool FWD, bool SCALE, bool FIN>
-__device__ __forceinline__ void pf1_load(const DirGrid& g, const int4* __restrict__ slots,
-                                         const double* __restrict__ vals, int b0, int nb, int G, int it, Pf1& p) {
-    p.valid = it < nb * G;
-    if (!p.valid) return;
-    const int bi = it / G, li = it - bi * G;
-    p.sl = slots[b0 + bi];
-    const int n = p.sl.y, r0 = p.sl.z;
-    const bool two = p.sl.w >= 0;
-    const int r1 = two ? p.sl.w : r0;
+__device__ __forceinline__ void line_ahead(const LineSched& sc, const int4 d, LineAhead& p) {
+    const int cnt = d.w & kLineCntMask;                    // the same for the whole warp
+    const int at = d.y + (threadIdx.x & 31);
 #pragma unroll
-    for (int k = 0; k < 4; k++) {
-        const int e = li + k * G;
-        const bool in = e < n;
-        p.i[k] = in ? g.col[r0 + e] : -1;
-        p.u[k] = in ? vals[r0 + e] : 0.0;
-        p.w[k] = (in && two) ? vals[r1 + e] : 0.0;
-    }
-    if (FIN && li == 0) {
-        const int q = p.sl.x;
-        p.inv0 = SCALE ? g.invdiag[q] : 1.0;
-        p.inv1 = (SCALE && two) ? g.invdiag[q + 1] : 1.0;
-        p.vt = two ? vals[FWD ? r1 + n : r0 - 1] : 0.0;
-    }
+    for (int k = 0; k < kLinePre; k++)
+        if (k < cnt) {
+            p.i[k] = sc.col[at + 32 * k];
+            p.u[k] = sc.val[at + 32 * k];
+        }
+    if (d.z >= 0) p.vt = sc.vt[d.z];
 }
 
-// row share of one item: the prefetched first chunk, then the rest of the row
-__device__ __forceinline__ void pf1_sum(const DirGrid& g, const double* __restrict__ vals, const Pf1& p, int li,
-                                        int G, const double* X, double& s0, double& s1) {
-    const int n = p.sl.y, r0 = p.sl.z;
-    const bool two = p.sl.w >= 0;
-    const int r1 = two ? p.sl.w : r0;
+// x_q = b_q - sum v_qc x_c over the schedule's levels; in a bus of two rows the theta row
+// is solved first (FWD) or the v row.
+template <bool FWD, int NT>
+__device__ void line_sweep(const LineSched& sc, double* X) {
+    const int n_steps = sc.n;
+    if (n_steps <= 0) return;
+    const int4* my = sc.steps + threadIdx.x;
+    auto desc = [&](int st) { return st < n_steps ? my[st * NT] : make_int4(-1, 0, -1, 0); };
+    int4 d = desc(0), d1 = desc(1), d2 = desc(2);
+    LineAhead p;
 #pragma unroll
-    for (int k = 0; k < 4; k++) {
-        if (p.i[k] >= 0) {
-            const double xv = X[p.i[k]];
-            s0 = fma(-p.u[k], xv, s0);
-            if (two) s1 = fma(-p.w[k], xv, s1);
-        }
+    for (int k = 0; k < kLinePre; k++) {
+        p.i[k] = 0;
+        p.u[k] = 0.0;
     }
-    row1_sub(g.col, vals, r0, r1, li + 4 * G, n, G, X, two, s0, s1);
-}
-
-template <bool SCALE, bool EXT>
-__device__ void sweep1_fwd(const DirGrid& g, const LevelSet& ls, const double* __restrict__ vals, double* X) {
-    const int TT = (int)blockDim.x, gt = (int)threadIdx.x;
-    if (ls.n_lev <= 0) return;
-    int b0 = ls.ptr[0], nb = ls.ptr[1] - b0, G = group_size(nb, ls.maxext[0], TT);
-    Pf1 cur;
-    pf1_load<true, SCALE, !EXT>(g, ls.slots, vals, b0, nb, G, gt, cur);
-    for (int lev = 0; lev < ls.n_lev; lev++) {
-        int b0n = 0, nbn = 0, Gn = 1;
-        if (lev + 1 < ls.n_lev) {
-            b0n = ls.ptr[lev + 1];
-            nbn = ls.ptr[lev + 2] - b0n;
-            Gn = group_size(nbn, ls.maxext[lev + 1], TT);
-        }
-        for (int it = gt; it < nb * G; it += TT) {
-            Pf1 p = cur;
-            if (it != gt) pf1_load<true, SCALE, !EXT>(g, ls.slots, vals, b0, nb, G, it, p);
-            const int li = it - (it / G) * G;
-            const int q = p.sl.x;
-            const bool two = p.sl.w >= 0;
-            double s0 = 0.0, s1 = 0.0;
-            pf1_sum(g, vals, p, li, G, X, s0, s1);
-            group_sum(it, nb * G, G, s0, s1);
-            if (li == 0) {
-                const double a0 = X[q] + s0;
-                double a1 = two ? X[q + 1] + s1 : 0.0;
-                if (EXT) {
-                    X[q] = a0;
-                    if (two) X[q + 1] = a1;
+    p.vt = 0.0;
+    line_ahead(sc, d, p);
+    for (int st = 0; st < n_steps; st++) {
+        const int4 d3 = desc(st + 3);
+        const int w = d.w;
+        if (w & kLineActive) {                             // the same for the whole warp
+            const int q = d.x, lg = (w >> kLineLg) & 7, cnt = w & kLineCntMask, wlg = (w >> kLineWlg) & 7;
+            const int G = 1 << lg, row = (w & kLineSplit) && (threadIdx.x & G) ? 1 : 0;
+            // the first lane of a row starts from its right-hand side
+            double s = q >= 0 && (threadIdx.x & (G - 1)) == 0 ? X[q + row] : 0.0;
+            double xv[kLinePre];
+#pragma unroll
+            for (int k = 0; k < kLinePre; k++) xv[k] = X[p.i[k]];
+#pragma unroll
+            for (int k = 0; k < kLinePre; k++)
+                if (k < cnt) s = fma(p.u[k], xv[k], s);
+            for (int k = kLinePre; k < cnt; k += 4) {      // rows of more than kLinePre G entries
+                const int at = d.y + (threadIdx.x & 31) + 32 * k;
+                int c[4];
+                double u[4];
+#pragma unroll
+                for (int m = 0; m < 4; m++) {
+                    c[m] = k + m < cnt ? sc.col[at + 32 * m] : 0;
+                    u[m] = k + m < cnt ? sc.val[at + 32 * m] : 0.0;
+                }
+#pragma unroll
+                for (int m = 0; m < 4; m++)
+                    if (k + m < cnt) s = fma(u[m], X[c[m]], s);
+            }
+#pragma unroll
+            for (int o = 4; o >= 0; o--)
+                if (o < wlg) {
+                    const double t = __shfl_down_sync(0xffffffffu, s, 1 << o);
+                    if (o < lg) s += t;
+                }
+            const double s1 = __shfl_sync(0xffffffffu, s, (threadIdx.x + G) & 31);
+            if (q >= 0 && (threadIdx.x & ((w & kLineSplit ? 2 * G : G) - 1)) == 0) {
+                if (!(w & kLineSplit)) {
+                    X[q] = s;
+                } else if (w & kLineExt) {
+                    X[q] = s;
+                    X[q + 1] = s1;
                 } else {
-                    const double x0 = SCALE ? a0 * p.inv0 : a0;
-                    X[q] = x0;
-                    if (two) {
-                        a1 = fma(-p.vt, x0, a1);
-                        X[q + 1] = SCALE ? a1 * p.inv1 : a1;
-                    }
+                    X[FWD ? q : q + 1] = FWD ? s : s1;
+                    X[FWD ? q + 1 : q] = FWD ? fma(p.vt, s, s1) : fma(p.vt, s1, s);
                 }
             }
         }
-        if (lev + 1 < ls.n_lev) pf1_load<true, SCALE, !EXT>(g, ls.slots, vals, b0n, nbn, Gn, gt, cur);
-        __syncthreads();
-        b0 = b0n;
-        nb = nbn;
-        G = Gn;
+        if (d1.w & kLineActive) line_ahead(sc, d1, p);
+        if (w & kLineSync) __syncthreads();                // the same for every thread of the step
+        d = d1;
+        d1 = d2;
+        d2 = d3;
     }
 }
 
-template <bool SCALE>
-__device__ void sweep1_bwd(const DirGrid& g, const LevelSet& ls, const double* __restrict__ vals, double* X) {
-    const int TT = (int)blockDim.x, gt = (int)threadIdx.x;
-    if (ls.n_lev <= 0) return;
-    int b0 = ls.ptr[0], nb = ls.ptr[1] - b0, G = group_size(nb, ls.maxext[0], TT);
-    Pf1 cur;
-    pf1_load<false, SCALE, true>(g, ls.slots, vals, b0, nb, G, gt, cur);
-    for (int lev = 0; lev < ls.n_lev; lev++) {
-        int b0n = 0, nbn = 0, Gn = 1;
-        if (lev + 1 < ls.n_lev) {
-            b0n = ls.ptr[lev + 1];
-            nbn = ls.ptr[lev + 2] - b0n;
-            Gn = group_size(nbn, ls.maxext[lev + 1], TT);
-        }
-        for (int it = gt; it < nb * G; it += TT) {
-            Pf1 p = cur;
-            if (it != gt) pf1_load<false, SCALE, true>(g, ls.slots, vals, b0, nb, G, it, p);
-            const int li = it - (it / G) * G;
-            const int q = p.sl.x;
-            const bool two = p.sl.w >= 0;
-            double s0 = 0.0, s1 = 0.0;
-            pf1_sum(g, vals, p, li, G, X, s0, s1);
-            group_sum(it, nb * G, G, s0, s1);
-            if (li == 0) {
-                double a0 = X[q] + s0;
-                if (two) {
-                    const double a1 = X[q + 1] + s1;
-                    const double x1 = SCALE ? a1 * p.inv1 : a1;
-                    X[q + 1] = x1;
-                    a0 = fma(-p.vt, x1, a0);
-                }
-                X[q] = SCALE ? a0 * p.inv0 : a0;
-            }
-        }
-        if (lev + 1 < ls.n_lev) pf1_load<false, SCALE, true>(g, ls.slots, vals, b0n, nbn, Gn, gt, cur);
-        __syncthreads();
-        b0 = b0n;
-        nb = nbn;
-        G = Gn;
+// The line arrays' values from the factors: entry i is minus the entry of the unit-diagonal
+// factors L'', U' (see k_transpose_values) at position map[i], or (trans) of their transpose
+// there; 0 for a pad.
+__device__ __forceinline__ void line_values_body(const LineGrid& g, bool trans, double* __restrict__ out) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= g.n_line) return;
+    const int m = g.map[i];
+    double v = 0.0;
+    if (m >= 0) {
+        const int r = g.arow[m], c = g.col[m];
+        v = trans ? -(g.A[g.tpos[m]] * unit_scale(g.A, g.diagpos, g.invdiag, c, r))
+                  : -(g.A[m] * unit_scale(g.A, g.diagpos, g.invdiag, r, c));
     }
+    out[i] = v;
+}
+// blockIdx.y 0: of the factors into `line`, 1: of their transpose into `tline`
+__global__ void k_line_values(const __grid_constant__ LineGrid g) {
+    line_values_body(g, blockIdx.y != 0, blockIdx.y ? g.tline : g.line);
 }
 
 // One right-hand side, one CTA, x held in shared memory for the whole sweep
@@ -1855,42 +1774,29 @@ __device__ void sweep1_bwd(const DirGrid& g, const LevelSet& ls, const double* _
 // column by column in shared memory, as in k_dirs, instead of as one sparse
 // level per variable.
 constexpr int kSolve1Part = 2048;
-constexpr int kSolve1Threads = 768;   // 85 registers per thread: room for the prefetched level data
-__device__ __forceinline__ void k_solve1_body(DirGrid g, double* x, unsigned phases, int use_tail) {
+template <int NT>
+__device__ __forceinline__ void k_solve1_body(const LineGrid& g, double* x, bool trans, int use_tail) {
     extern __shared__ double X[];
     double* tri = X + g.n_x;
     double* part = tri + (use_tail ? (size_t)g.T * (g.T - 1) / 2 : 0);
-    for (int q = threadIdx.x; q < g.n_x; q += blockDim.x) X[q] = x[q];
+    // J_x = D L'' U': the right-hand side of J_x z = b enters as D^-1 b, and the solution
+    // D psi of J_x^T leaves as psi
+    for (int q = threadIdx.x; q < g.n_x; q += NT) X[q] = trans ? x[q] : x[q] * g.invdiag[q];
     __syncthreads();
+    line_sweep<true, NT>(trans ? g.tup : g.up, X);
     if (use_tail) {
-        if (phases & PH_L) {
-            sweep1_fwd<false, false>(g, g.sf, g.A, X);
-            sweep1_fwd<false, true>(g, g.ef, g.A, X);
-            tail_fwd<false>(g, g.triL, X, 1, 0, 1, part, tri);
-        }
-        if (phases & PH_U) {
-            tail_bwd<true>(g, g.triU, X, 1, 0, 1, part, tri);
-            sweep1_bwd<true>(g, g.sb, g.A, X);
-        }
-        if (phases & PH_UT) {
-            sweep1_fwd<true, false>(g, g.sf, g.At, X);
-            sweep1_fwd<true, true>(g, g.ef, g.At, X);
-            tail_fwd<true>(g, g.triUt, X, 1, 0, 1, part, tri);
-        }
-        if (phases & PH_LT) {
-            tail_bwd<false>(g, g.triLt, X, 1, 0, 1, part, tri);
-            sweep1_bwd<false>(g, g.sb, g.At, X);
-        }
-    } else {
-        if (phases & PH_L) sweep1_fwd<false, false>(g, g.lf, g.A, X);
-        if (phases & PH_U) sweep1_bwd<true>(g, g.lb, g.A, X);
-        if (phases & PH_UT) sweep1_fwd<true, false>(g, g.lf, g.At, X);
-        if (phases & PH_LT) sweep1_bwd<false>(g, g.lb, g.At, X);
+        tail_fwd<false>(g, trans ? g.triUtd : g.triLd, X, 1, 0, 1, part, tri);
+        tail_bwd<false>(g, trans ? g.triLtd : g.triUd, X, 1, 0, 1, part, tri);
     }
+    line_sweep<false, NT>(trans ? g.tdown : g.down, X);
     __syncthreads();
-    for (int q = threadIdx.x; q < g.n_x; q += blockDim.x) x[q] = X[q];
+    for (int q = threadIdx.x; q < g.n_x; q += NT) x[q] = trans ? X[q] * g.invdiag[q] : X[q];
 }
-__global__ void __launch_bounds__(kSolve1Threads, 1) k_solve1(DirGrid g, double* x, unsigned phases, int use_tail) { k_solve1_body(g, x, phases, use_tail); }
+template <int NT>
+__global__ void __launch_bounds__(NT, kLineRegs / NT)
+    k_solve1(const __grid_constant__ LineGrid g, double* x, int trans, int use_tail) {
+    k_solve1_body<NT>(g, x, trans, use_tail);
+}
 
 // ---------------------------------------------------------------------------
 // adjoint (eq. 7) and the per-state second-order coefficients
@@ -2091,7 +1997,7 @@ __global__ void k_tail_scatter_batch(RfBatch B) {
     k_tail_scatter_body(B.g[blockIdx.y]);
 }
 
-// the single solves' tail triangles: L (unit lower) and U with column j scaled by 1/u_jj
+// the single solves' tail triangles, of the unit-diagonal factors L'' and U'
 __global__ void k_tail_tri_batch(TriBatch B) {
     const int i = blockIdx.y, T = B.T;
     const int idx = blockIdx.x * blockDim.x + threadIdx.x;
@@ -2099,13 +2005,19 @@ __global__ void k_tail_tri_batch(TriBatch B) {
     const int r = idx / T, c = idx - r * T;
     if (r == c) return;
     const int p = B.pos[i][idx];
-    const double a = p >= 0 ? B.A[i][p] : 0.0;
-    if (r > c) B.triL[i][c * (T - 1) - c * (c - 1) / 2 + (r - c - 1)] = a;
-    else B.triU[i][c * (c - 1) / 2 + r] = a * B.invdiag[i][B.t0 + c];
+    const double a = p >= 0 ? B.A[i][p] : 0.0, ir = B.invdiag[i][B.t0 + r];     // as k_build_tail, bit for bit
+    if (r > c) B.triLd[i][c * (T - 1) - c * (c - 1) / 2 + (r - c - 1)] = a * B.A[i][B.pos[i][c * T + c]] * ir;
+    else B.triUd[i][c * (c - 1) / 2 + r] = a * ir;
 }
 
-__global__ void __launch_bounds__(kSolve1Threads, 1) k_solve1_batch(Solve1Batch B, unsigned phases, int use_tail) {
-    k_solve1_body(B.g[blockIdx.x], B.x[blockIdx.x], phases, use_tail);
+__global__ void k_line_values_batch(const __grid_constant__ Solve1Batch B) {
+    line_values_body(B.g[blockIdx.y], false, B.g[blockIdx.y].line);
+}
+
+template <int NT>
+__global__ void __launch_bounds__(NT, kLineRegs / NT)
+    k_solve1_batch(const __grid_constant__ Solve1Batch B, int use_tail) {
+    k_solve1_body<NT>(B.g[blockIdx.x], B.x[blockIdx.x], false, use_tail);
 }
 
 }  // namespace
@@ -2231,7 +2143,8 @@ cudaError_t prepare_kernels() {
     if (g_prepared[dev]) return cudaSuccess;
     e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
     if (e != cudaSuccess) return e;
-    const void* fns[3] = {(const void*)k_dirs, (const void*)k_solve1, (const void*)k_solve1_batch};
+    const void* fns[5] = {(const void*)k_dirs, (const void*)k_solve1<256>, (const void*)k_solve1<512>,
+                          (const void*)k_solve1_batch<256>, (const void*)k_solve1_batch<512>};
     for (const void* f : fns) {
         cudaFuncAttributes fa;
         e = cudaFuncGetAttributes(&fa, f);
@@ -2252,13 +2165,13 @@ cudaError_t prepare_kernels() {
 }
 
 void launch_transpose_values(int nnz, const int* tpos, const int* arow, const int* col, const int* diagpos,
-                             const double* A, const double* invdiag, double* At, double* Ad, double* Atd, int nnz_jp,
+                             const double* A, const double* invdiag, double* Ad, double* Atd, int nnz_jp,
                              const int* jpt_src, const int* jpt_row, const double* jpv, double* jptv, double* jptvd,
                              cudaStream_t st) {
     int n = nnz > nnz_jp ? nnz : nnz_jp;
     if (n > 0)
-        k_transpose_values<<<blocks_for(n, 256), 256, 0, st>>>(nnz, tpos, arow, col, diagpos, A, invdiag, At, Ad, Atd,
-                                                               nnz_jp, jpt_src, jpt_row, jpv, jptv, jptvd);
+        k_transpose_values<<<blocks_for(n, 256), 256, 0, st>>>(nnz, tpos, arow, col, diagpos, A, invdiag, Ad, Atd, nnz_jp,
+                                                               jpt_src, jpt_row, jpv, jptv, jptvd);
 }
 
 // SMs of the current device (1 if the query fails)
@@ -2329,18 +2242,26 @@ void launch_scale_rows(int n, int N, const double* s, double* x, int64_t ld, cud
     if ((int64_t)n * N > 0) k_scale_rows<<<blocks_for((int64_t)n * N, 256), 256, 0, st>>>(n, N, s, x, ld);
 }
 
-void launch_build_tail(int T, int t0, const int* pos, const double* A, const double* invdiag, double* triL,
-                       double* triU, double* triUt, double* triLt, double* triLd, double* triUd, double* triUtd,
-                       double* triLtd, cudaStream_t st) {
+void launch_build_tail(int T, int t0, const int* pos, const double* A, const double* invdiag, double* triLd,
+                       double* triUd, double* triUtd, double* triLtd, cudaStream_t st) {
     if (T > 1)
-        k_build_tail<<<blocks_for((int64_t)T * T, 256), 256, 0, st>>>(T, t0, pos, A, invdiag, triL, triU, triUt, triLt,
-                                                                      triLd, triUd, triUtd, triLtd);
+        k_build_tail<<<blocks_for((int64_t)T * T, 256), 256, 0, st>>>(T, t0, pos, A, invdiag, triLd, triUd, triUtd,
+                                                                      triLtd);
+}
+
+void launch_line_values(const LineGrid& g, bool transposed_too, cudaStream_t st) {
+    if (g.n_line > 0)
+        k_line_values<<<dim3((unsigned)blocks_for(g.n_line, 256), transposed_too ? 2u : 1u), 256, 0, st>>>(g);
 }
 
 void launch_adjoint_rhs(const PfGrid& g, const PfState& s, const AdjData& a, cudaStream_t st) {
     k_adjoint_rhs<<<1, 32, 0, st>>>(g, s, a);
     k_objective<<<1, 256, 0, st>>>(g, s, a.F);
 }
+
+// Small grids take CTAs of 256 threads: their levels do not fill more warps, and idle
+// warps cost issue slots and barrier time at every step.
+int line_threads(int n_x) { return n_x <= 1024 ? 256 : 512; }
 
 static size_t solve1_smem(int n_x, int T, bool tail) {
     return ((size_t)n_x + (tail ? (size_t)T * (T - 1) / 2 : 0) + kSolve1Part) * sizeof(double);
@@ -2352,8 +2273,10 @@ int solve1_mode(int n_x, int T) {
     return solve1_smem(n_x, T, false) <= cap ? 1 : 0;
 }
 
-cudaError_t launch_solve1(const DirGrid& g, double* x, unsigned phases, bool use_tail, cudaStream_t st) {
-    k_solve1<<<1, kSolve1Threads, solve1_smem(g.n_x, g.T, use_tail), st>>>(g, x, phases, use_tail ? 1 : 0);
+cudaError_t launch_solve1(const LineGrid& g, double* x, bool trans, bool use_tail, cudaStream_t st) {
+    const size_t smem = solve1_smem(g.n_x, g.T, use_tail);
+    if (line_threads(g.n_x) == 256) k_solve1<256><<<1, 256, smem, st>>>(g, x, trans, use_tail ? 1 : 0);
+    else k_solve1<512><<<1, 512, smem, st>>>(g, x, trans, use_tail ? 1 : 0);
     return cudaGetLastError();
 }
 
@@ -2443,10 +2366,13 @@ void launch_tail_tri_batch(const TriBatch& B, cudaStream_t st) {
         k_tail_tri_batch<<<dim3((unsigned)blocks_for((int64_t)B.T * B.T, 256), (unsigned)B.n), 256, 0, st>>>(B);
 }
 
-cudaError_t launch_solve1_batch(const Solve1Batch& B, unsigned phases, bool use_tail, int n_x, int T,
-                                cudaStream_t st) {
+cudaError_t launch_solve1_batch(const Solve1Batch& B, bool use_tail, int n_x, int T, cudaStream_t st) {
     if (B.n <= 0) return cudaSuccess;
-    k_solve1_batch<<<B.n, kSolve1Threads, solve1_smem(n_x, T, use_tail), st>>>(B, phases, use_tail ? 1 : 0);
+    const int nl = B.g[0].n_line;      // one topology: the same for every item
+    if (nl > 0) k_line_values_batch<<<dim3((unsigned)blocks_for(nl, 256), (unsigned)B.n), 256, 0, st>>>(B);
+    const size_t smem = solve1_smem(n_x, T, use_tail);
+    if (line_threads(n_x) == 256) k_solve1_batch<256><<<B.n, 256, smem, st>>>(B, use_tail ? 1 : 0);
+    else k_solve1_batch<512><<<B.n, 512, smem, st>>>(B, use_tail ? 1 : 0);
     return cudaGetLastError();
 }
 

@@ -37,17 +37,13 @@ struct DirGrid {
     int n_x, n_p;
     int nnz;                                   // positions of the pattern of A (index checks)
     int zero_row;                              // n_x + n_p: a row of zeros in V
-    // filled matrix A = L + U (CSR), its transposed values and 1/diagonal
+    // columns of the filled matrix A = L + U (CSR) and 1/diagonal
     const int *col;
-    const double *A, *At, *invdiag;
+    const double *invdiag;
     LevelSet lf, lb;                           // full forward / backward schedules
     LevelSet sf, sb, ef;                       // sparse part only, and the tail's external phase
     LevelSet sbr;                              // sb restricted to the rows of J_p and their ancestors
-    // dense trailing block [t0, t0 + T): packed strictly-triangular columns
-    //   triL  (L,  lower, unit)            triU  (U,  upper, column j scaled by 1/u_jj)
-    //   triUt (U^T, lower, column j scaled) triLt (L^T, upper, unit)
-    int t0, T;
-    const double *triL, *triU, *triUt, *triLt;
+    int t0, T;                                 // dense trailing block [t0, t0 + T)
     // Unit-diagonal factors used by k_dirs (J_x = D L'' U', D = diag(U)): values of
     // L'' and U' in A's pattern and transposed, the dense tail's triangles of L'',
     // U', U'^T, L''^T, and D^-1 J_p by p index (jptvd)
@@ -282,10 +278,10 @@ void launch_prefetch_l2(const PrefetchList& L, cudaStream_t st);
 // at the front), the pivot steps of every sparse bus, then the dense tail's LU.
 cudaError_t launch_refactor(const RfGrid& g, const int* lev_ptr_host, const int64_t* tgt_lev_ptr_host,
                             const int* piv_lev_ptr_host, int n_lev, cudaStream_t st);
-// At (transposed values), Ad / Atd (the unit-diagonal factors L'', U' of J_x = D L'' U'
-// and their transpose), jptv (J_p by p index) and jptvd (D^-1 J_p by p index)
+// Ad / Atd (the unit-diagonal factors L'', U' of J_x = D L'' U' and their transpose), jptv
+// (J_p by p index) and jptvd (D^-1 J_p by p index)
 void launch_transpose_values(int nnz, const int* tpos, const int* arow, const int* col, const int* diagpos,
-                             const double* A, const double* invdiag, double* At, double* Ad, double* Atd, int nnz_jp,
+                             const double* A, const double* invdiag, double* Ad, double* Atd, int nnz_jp,
                              const int* jpt_src, const int* jpt_row, const double* jpv, double* jptv, double* jptvd,
                              cudaStream_t st);
 void launch_dirs(const DirGrid& g, const DirLaunch& L, cudaStream_t st);
@@ -296,15 +292,42 @@ int dirs_tail_cap();       // dense-tail rows x directions a CTA can hold
 // dense tail triangles of the current factors (pos: T*T map to A, -1 where structurally zero)
 // x[r][c] *= s[r] for r < n, c < N
 void launch_scale_rows(int n, int N, const double* s, double* x, int64_t ld, cudaStream_t st);
-// triangles of the single solves (triL .. triLt) and of the unit-diagonal factors (triLd .. triLtd)
-void launch_build_tail(int T, int t0, const int* pos, const double* A, const double* invdiag, double* triL,
-                       double* triU, double* triUt, double* triLt, double* triLd, double* triUd, double* triUtd,
-                       double* triLtd, cudaStream_t st);
+void launch_build_tail(int T, int t0, const int* pos, const double* A, const double* invdiag, double* triLd,
+                       double* triUd, double* triUtd, double* triLtd, cudaStream_t st);
 // One right-hand side in one CTA with x in shared memory: mode 2 also keeps the
 // dense tail triangle there (needs the tail triangles built), 1 without it,
 // 0 when x does not fit (use the direction kernel instead).
 int solve1_mode(int n_x, int T);
-cudaError_t launch_solve1(const DirGrid& g, double* x, unsigned phases, bool use_tail, cudaStream_t st);
+// Its schedule: steps of line_threads(n_x) descriptors {q, base, b, w} each, built by
+// line_steps from the level lists (kernels.cu explains the descriptor).
+constexpr int kLineRegs = 512;        // threads an SM holds at 128 registers
+constexpr int kLinePre = 8;           // entries a lane holds ahead
+// LineBits, the fields of a descriptor's w: the warp's entries per lane, log2(G), the warp's
+// largest log2(G), and the flags
+constexpr int kLineCntMask = 0xff, kLineLg = 8, kLineWlg = 11;
+constexpr int kLineExt = 1 << 26;     // rows of the dense tail, subtract only
+constexpr int kLineSync = 1 << 27;    // barrier after the step (its level ends)
+constexpr int kLineSplit = 1 << 28;   // a bus of two rows: a group of lanes for each, side by side
+constexpr int kLineActive = 1 << 30;  // the warp has a bus in this step
+struct LineSched {
+    int n;                            // steps
+    const int4* steps;
+    const int* col;                   // line arrays: column of each entry (0: a pad),
+    const double* val;                //   its value negated (0: a pad), and each bus's own
+    const double* vt;                 //   off-diagonal entry negated
+};
+struct LineGrid {
+    int n_x, t0, T;
+    LineSched up, down, tup, tdown;   // with L'', U', and with U'^T, L''^T
+    int n_line;                       // entries of the line arrays [up | down | up's vt | down's vt]
+    const int *map, *arow, *col, *tpos, *diagpos;   // their positions in A (-1: a pad); A's rows, columns, ...
+    double *line, *tline;             // their values, of the factors and of their transpose
+    const double *A, *invdiag;
+    const double *triLd, *triUd, *triUtd, *triLtd;
+};
+void launch_line_values(const LineGrid& g, bool transposed_too, cudaStream_t st);
+int line_threads(int n_x);
+cudaError_t launch_solve1(const LineGrid& g, double* x, bool trans, bool use_tail, cudaStream_t st);
 
 // Dense Cholesky of the tracking step (dense.cu).  A, L, B, work, y and info
 // are device pointers; column-major.  info receives 0 or the 1-based column of
@@ -336,11 +359,11 @@ struct TriBatch {
     int n, T, t0;
     const int* pos[kMaxPfBatch];
     const double *A[kMaxPfBatch], *invdiag[kMaxPfBatch];
-    double *triL[kMaxPfBatch], *triU[kMaxPfBatch];
+    double *triLd[kMaxPfBatch], *triUd[kMaxPfBatch];
 };
 struct Solve1Batch {
     int n;
-    DirGrid g[kMaxPfBatch];
+    LineGrid g[kMaxPfBatch];
     double* x[kMaxPfBatch];
 };
 // residual and Jacobian of every item (after launch_pf_prep_batch)
@@ -353,7 +376,7 @@ cudaError_t launch_refactor_batch(const RfBatch& B, const int* lev_ptr_host, con
                                   const int* piv_lev_ptr_host, int n_lev, cudaStream_t st);
 // the dense tail's triangles of the single solves (L, and U with columns scaled by 1/u_jj)
 void launch_tail_tri_batch(const TriBatch& B, cudaStream_t st);
-cudaError_t launch_solve1_batch(const Solve1Batch& B, unsigned phases, bool use_tail, int n_x, int T, cudaStream_t st);
+cudaError_t launch_solve1_batch(const Solve1Batch& B, bool use_tail, int n_x, int T, cudaStream_t st);
 void launch_newton_update_batch(const PfBatch& B, cudaStream_t st);
 
 int dense_tile(int n);
