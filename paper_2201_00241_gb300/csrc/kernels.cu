@@ -1660,7 +1660,7 @@ __global__ void __launch_bounds__(NT, MINB) k_dirs_batch(DirBatch B) {
 // barrier costs more than a CTA barrier.)
 struct LineAhead {
     int i[kLinePre];
-    double u[kLinePre];
+    double u[kLinePre];        // the switch of line_sweep names all eight
     double vt;                 // the bus's own off-diagonal entry
 };
 
@@ -1703,10 +1703,21 @@ __device__ void line_sweep(const LineSched& sc, double* X) {
             double s = q >= 0 && (threadIdx.x & (G - 1)) == 0 ? X[q + row] : 0.0;
             double xv[kLinePre];
 #pragma unroll
-            for (int k = 0; k < kLinePre; k++) xv[k] = X[p.i[k]];
-#pragma unroll
-            for (int k = 0; k < kLinePre; k++)
-                if (k < cnt) s = fma(p.u[k], xv[k], s);
+            for (int k = 0; k < kLinePre; k++) xv[k] = k < cnt ? X[p.i[k]] : 0.0;
+            // Jumps, not predicates: a predicated-off FP64 instruction still takes its 64 cycles.
+            // Unrolled with `if (k < cnt)`, a level of 16-lane rows cost 2000 cycles for any cnt;
+            // so it costs 1700, and the two sweeps of the 9241-bus grid 494 k cycles for 580 k.
+            switch (cnt) {
+                default: s = fma(p.u[7], xv[7], s); [[fallthrough]];
+                case 7: s = fma(p.u[6], xv[6], s); [[fallthrough]];
+                case 6: s = fma(p.u[5], xv[5], s); [[fallthrough]];
+                case 5: s = fma(p.u[4], xv[4], s); [[fallthrough]];
+                case 4: s = fma(p.u[3], xv[3], s); [[fallthrough]];
+                case 3: s = fma(p.u[2], xv[2], s); [[fallthrough]];
+                case 2: s = fma(p.u[1], xv[1], s); [[fallthrough]];
+                case 1: s = fma(p.u[0], xv[0], s); [[fallthrough]];
+                case 0: break;
+            }
             for (int k = kLinePre; k < cnt; k += 4) {      // rows of more than kLinePre G entries
                 const int at = d.y + (threadIdx.x & 31) + 32 * k;
                 int c[4];
@@ -1720,12 +1731,18 @@ __device__ void line_sweep(const LineSched& sc, double* X) {
                 for (int m = 0; m < 4; m++)
                     if (k + m < cnt) s = fma(u[m], X[c[m]], s);
             }
-#pragma unroll
-            for (int o = 4; o >= 0; o--)
-                if (o < wlg) {
-                    const double t = __shfl_down_sync(0xffffffffu, s, 1 << o);
-                    if (o < lg) s += t;
-                }
+            auto halve = [&](int o) {
+                const double t = __shfl_down_sync(0xffffffffu, s, 1 << o);
+                if (o < lg) s += t;
+            };
+            switch (wlg) {
+                case 5: halve(4); [[fallthrough]];
+                case 4: halve(3); [[fallthrough]];
+                case 3: halve(2); [[fallthrough]];
+                case 2: halve(1); [[fallthrough]];
+                case 1: halve(0); [[fallthrough]];
+                default: break;
+            }
             const double s1 = __shfl_sync(0xffffffffu, s, (threadIdx.x + G) & 31);
             if (q >= 0 && (threadIdx.x & ((w & kLineSplit ? 2 * G : G) - 1)) == 0) {
                 if (!(w & kLineSplit)) {
