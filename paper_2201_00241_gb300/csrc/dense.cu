@@ -21,10 +21,11 @@
 // factorisation, triangular solve).  No launch reads a tile that another of
 // its CTAs writes.
 //
-// The solves run one launch per tile: the forward sweep L y = b writes y into a
-// workspace while the other CTAs of the launch subtract L_ik y_k from the
-// right-hand side below it, and the backward sweep L^T x = y writes x back into
-// B while its other CTAs update the workspace above.
+// The solves run one launch per tile, or per panel of 96 columns where there are few
+// right-hand sides: the forward sweep L y = b writes y into a workspace while the other
+// CTAs of the launch subtract L_ik y_k from the right-hand side below it, and the
+// backward sweep L^T x = y writes x back into B while its other CTAs update the
+// workspace above.
 //
 // The diagonal tile is eliminated without divisions: step j replaces every
 // trailing entry by 2^-e_j (d_j a_rc - a_rj a_cj), with d_j the current pivot and
@@ -567,6 +568,160 @@ __global__ void __launch_bounds__(kDenseThreads)
     }
 }
 
+// Solves with few right-hand sides: panels of kPN columns, one launch per panel.  A solve
+// is a chain (one column after the other), so what counts is how little stands between two
+// columns.  One launch per 16-column tile spends more on the launch and on the loads behind
+// it (5.3 us a tile, 2.4 us of them the chain) than on the chain; a panel of 96 columns has
+// both once per 96.  The panel's triangle is staged folded (column c beside column
+// kPN - 1 - c) in static shared memory: 37.6 KB, several CTAs to an SM.
+//
+// CTA (b, j) works for right-hand side j: it solves the panel (each CTA for itself, as all
+// of them need it), CTA b = 0 stores it, and b > 0 takes it off RB further rows.  Warp w < 6
+// owns rows 16 w .. 16 w + 15 of the panel, two lanes a row: the warp of the next 16 rows
+// adds its lanes' shares and substitutes with shuffles, writes the result to shared memory,
+// and after one barrier the other warps take it off their rows.
+//
+// Everything read from L is loaded before the wait for the previous launch: that launch
+// waited for the writer of L and writes right-hand sides only.  It lets the next launch
+// start as soon as its own wait is over, so the loads of a panel run beside the chain of
+// the panel before.
+constexpr int kPN = 96;
+constexpr int kPStride = kPN + 2;
+__device__ __forceinline__ int fold(int r, int c) {         // r >= c
+    return c < kPN / 2 ? c * kPStride + (r - c) : (kPN - 1 - c) * kPStride + r + 1;
+}
+
+// Loads the panel's triangle and 1 / l_rr; the 16 x 16 blocks on its diagonal become the
+// multipliers l_rc / l_cc (FWD) or l_rc / l_rr of the unscaled substitutions.
+template <bool FWD>
+__device__ __forceinline__ void panel_load(double* S, double* Inv, const double* __restrict__ L, int64_t ldl, int p0,
+                                           int pb) {
+    const int t = threadIdx.x;
+    if (t < kPN) Inv[t] = t < pb ? 1.0 / L[(p0 + t) + (int64_t)(p0 + t) * ldl] : 0.0;
+    for (int e = t; e < kPN * kPN; e += kDenseThreads) {
+        const int r = e % kPN, c = e / kPN;
+        if (r >= c) S[fold(r, c)] = r < pb ? L[(p0 + r) + (int64_t)(p0 + c) * ldl] : 0.0;
+    }
+    __syncthreads();
+    for (int e = t; e < kPN / 16 * 256; e += kDenseThreads) {
+        const int b = e / 256, r = 16 * b + e % 16, c = 16 * b + e / 16 % 16;
+        if (r > c) S[fold(r, c)] *= Inv[FWD ? c : r];
+    }
+    __syncthreads();
+}
+
+// Solves the panel with right-hand side z (this lane's share of row 16 w + lane % 16) into Y.
+template <bool FWD>
+__device__ __forceinline__ void panel_solve(const double* S, const double* Inv, double* Y, double z) {
+    const int w = threadIdx.x / 32, r = threadIdx.x % 16, half = threadIdx.x / 16 % 2, row = 16 * w + r;
+    for (int s = 0; s < kPN / 16; s++) {
+        const int b = FWD ? s : kPN / 16 - 1 - s;
+        if (w == b) {
+            double m[16];
+#pragma unroll
+            for (int j = 0; j < 16; j++) {
+                const int q = 16 * b + j;
+                m[j] = FWD ? (r > j ? S[fold(row, q)] : 0.0) : (r < j ? S[fold(q, row)] : 0.0);
+            }
+            z += __shfl_xor_sync(0xffffffffu, z, 16);
+#pragma unroll
+            for (int i = 0; i < 15; i++) {
+                const int j = FWD ? i : 15 - i;
+                const double zj = __shfl_sync(0xffffffffu, z, j, 16);
+                if (FWD ? r > j : r < j) z = fma(-m[j], zj, z);
+            }
+            if (half == 0) Y[row] = z * Inv[row];
+        }
+        __syncthreads();
+        if (w < kPN / 16 && (FWD ? w > b : w < b)) {
+            const int q0 = 16 * b + 8 * half;
+#pragma unroll
+            for (int j = 0; j < 8; j++)
+                z = fma(-(FWD ? S[fold(row, q0 + j)] : S[fold(q0 + j, row)]), Y[q0 + j], z);
+        }
+    }
+}
+
+template <bool FWD, int RB>
+__global__ void __launch_bounds__(kDenseThreads)
+    k_chol_panel(int n, const double* __restrict__ L, int64_t ldl, double* __restrict__ B, int64_t ldb,
+                 double* __restrict__ W, int p) {
+    constexpr int KG = FWD ? kDenseThreads / RB : 32;       // lanes that share a row of the strip
+    constexpr int KN = kPN / KG;                            // panel columns per lane
+    constexpr int RW = FWD ? 1 : RB / (kDenseThreads / 32); // strip rows per lane
+    __shared__ double S[kPN / 2 * kPStride];
+    __shared__ double Inv[kPN], Y[kPN], part[kDenseThreads / 32][RB];
+    const int t = threadIdx.x, lane = t % 32, w = t / 32;
+    const int p0 = p * kPN, pb = min(kPN, n - p0), b = blockIdx.x;
+    double* rhs = FWD ? B + (int64_t)blockIdx.y * ldb : W + (int64_t)blockIdx.y * n;
+    double* out = FWD ? W + (int64_t)blockIdx.y * n : B + (int64_t)blockIdx.y * ldb;
+    // the strip: RB rows below the panel (FWD) or RB rows above it, of the transpose
+    const int i0 = FWD ? p0 + kPN + (b - 1) * RB : (b - 1) * RB;
+    const int ib = b ? min(RB, (FWD ? n : p0) - i0) : 0;
+    double M[RW][KN];
+#pragma unroll
+    for (int q = 0; q < RW; q++)
+#pragma unroll
+        for (int m = 0; m < KN; m++) {
+            const int i = FWD ? t % RB : w * RW + q, k = FWD ? t / RB + KG * m : lane + 32 * m;
+            M[q][m] = i < ib && k < pb ? (FWD ? L[(i0 + i) + (int64_t)(p0 + k) * ldl]
+                                              : L[(p0 + k) + (int64_t)(i0 + i) * ldl])
+                                       : 0.0;
+        }
+    panel_load<FWD>(S, Inv, L, ldl, p0, pb);
+    pdl_wait();
+    pdl_trigger();
+    const int row = 16 * w + lane % 16;
+    double old = 0.0;
+    if (t < ib) old = rhs[i0 + t];
+    panel_solve<FWD>(S, Inv, Y, row < pb && lane < 16 ? rhs[p0 + row] : 0.0);
+    if (b == 0) {
+        if (t < pb) out[p0 + t] = Y[t];
+        return;
+    }
+    double a[RW];
+#pragma unroll
+    for (int q = 0; q < RW; q++) {
+        a[q] = 0.0;
+#pragma unroll
+        for (int m = 0; m < KN; m++) a[q] = fma(M[q][m], Y[FWD ? t / RB + KG * m : lane + 32 * m], a[q]);
+    }
+    if constexpr (FWD) {
+        // lanes t, t + RB, ... share a row: first inside the warp, then over the warps
+#pragma unroll
+        for (int o = 16; o >= RB; o >>= 1) a[0] += __shfl_xor_sync(0xffffffffu, a[0], o);
+        if (lane < RB) part[w][lane] = a[0];
+        __syncthreads();
+        if (t < ib) {
+            double s0 = part[0][t], s1 = part[1][t];
+#pragma unroll
+            for (int v = 2; v < kDenseThreads / 32; v += 2) {
+                s0 += part[v][t];
+                s1 += part[v + 1][t];
+            }
+            rhs[i0 + t] = old - (s0 + s1);
+        }
+    } else {
+        // the warp's RW sums over its lanes: halve the sums a lane carries while there are several
+        int q = 0, o = 16;
+#pragma unroll
+        for (int h = RW / 2; h > 0; h >>= 1, o >>= 1) {
+            const bool up = lane & o;
+#pragma unroll
+            for (int v = 0; v < h; v++) {
+                const double give = up ? a[v] : a[v + h], keep = up ? a[v + h] : a[v];
+                a[v] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+            }
+            if (up) q += h;
+        }
+#pragma unroll
+        for (; o > 0; o >>= 1) a[0] += __shfl_xor_sync(0xffffffffu, a[0], o);
+        if ((lane & (32 / RW - 1)) == 0) part[0][w * RW + q] = a[0];
+        __syncthreads();
+        if (t < ib) rhs[i0 + t] = old - part[0][t];
+    }
+}
+
 // Launches of at most 4.5 x (SM count) CTAs request enough dynamic shared
 // memory (unused) that every CTA has an SM to itself: the panel CTAs, first in
 // the grid, then run their latency-bound chain without trailing CTAs beside them
@@ -635,6 +790,34 @@ cudaError_t potrf_tiles(int n, double* A, int64_t lda, int* info, double* y, cud
     return cudaGetLastError();
 }
 
+// A panel launch has (1 + strips) CTAs per right-hand side; strips of 8 rows end sooner,
+// strips of 32 need fewer CTAs.
+constexpr int kSolveCtas = 152;
+
+// Every CTA of a panel launch solves its panel, so the panels lose where right-hand sides
+// already fill the GPU, and for orders of one or two panels.  Measured, tiles -> panels, us
+// for both sweeps: 1019 x 1 403 -> 252, x 3 408 -> 277, x 16 505 -> 405, x 32 511 -> 657;
+// 519 x 1 211 -> 144, x 16 264 -> 177; 2400 x 1 871 -> 594, x 4 886 -> 736, x 8 1072 -> 1052,
+// x 16 1083 -> 1685; 107 x 1 55 -> 60.
+bool by_panels(int n, int nrhs) { return n > 128 && nrhs <= 16 && (int64_t)n * nrhs <= 16384; }
+
+template <bool FWD>
+cudaError_t panel_sweep(int n, const double* L, int64_t ldl, double* B, int64_t ldb, int nrhs, double* W, bool pdl,
+                        cudaStream_t s) {
+    const int np = (n + kPN - 1) / kPN;
+    for (int i = 0; i < np; i++) {
+        const int p = FWD ? i : np - 1 - i;
+        const int rows = FWD ? (n > (p + 1) * kPN ? n - (p + 1) * kPN : 0) : p * kPN;
+        const bool narrow = (int64_t)(1 + (rows + 7) / 8) * nrhs <= kSolveCtas;
+        const dim3 grid(1 + (narrow ? (rows + 7) / 8 : (rows + 31) / 32), (unsigned)nrhs);
+        const cudaError_t e = launch_pdl(pdl, narrow ? k_chol_panel<FWD, 8> : k_chol_panel<FWD, 32>, grid,
+                                         dim3(kDenseThreads), 0, s, n, L, ldl, B, ldb, W, p);
+        if (e != cudaSuccess) return e;
+        pdl = true;
+    }
+    return cudaGetLastError();
+}
+
 template <int TB>
 cudaError_t potrs_tiles(int n, const double* L, int64_t ldl, double* B, int64_t ldb, int nrhs, double* Y,
                         bool forward, cudaStream_t s) {
@@ -671,6 +854,13 @@ cudaError_t launch_potrf(int n, double* A, int64_t lda, int* info, double* y, cu
 cudaError_t launch_potrs(int n, const double* L, int64_t ldl, double* B, int64_t ldb, int nrhs, double* work,
                          bool forward, cudaStream_t s) {
     if (n == 0 || nrhs == 0) return cudaSuccess;
+    if (by_panels(n, nrhs)) {
+        if (forward) {
+            const cudaError_t e = panel_sweep<true>(n, L, ldl, B, ldb, nrhs, work, false, s);
+            if (e != cudaSuccess) return e;
+        }
+        return panel_sweep<false>(n, L, ldl, B, ldb, nrhs, work, forward, s);
+    }
     return dense_tile(n) == 16 ? potrs_tiles<16>(n, L, ldl, B, ldb, nrhs, work, forward, s)
                                : potrs_tiles<32>(n, L, ldl, B, ldb, nrhs, work, forward, s);
 }

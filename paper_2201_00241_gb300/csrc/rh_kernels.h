@@ -172,6 +172,9 @@ struct PfState {
 // so it is fully ordered after whatever precedes it (copies, event waits).
 #ifdef __CUDACC__
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// Lets the next kernel's CTAs start (up to their own pdl_wait) once every CTA of this one
+// is here; without it they start as this kernel's CTAs exit.
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 // ---- division-free elimination of dense tiles -----------------------------------
 // The diagonal tiles of the dense factorisations (the refactorisation's dense
