@@ -420,15 +420,26 @@ __global__ void __launch_bounds__(128) k_jac_ad(PfGrid g, PfState s, const int* 
 // x's block, the others one entry j each (positions a_tj, a_vj, a_jt, a_jv).
 __device__ __forceinline__ void k_rf_pivot_body(const RfGrid& g) {
     const int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (x < g.n_piv) {
-        const int k = (int)x;
-        const int qt = g.q0[k];
-        const int dt = g.diagpos[qt];
+    const int64_t e = x - g.n_piv;
+    int k = 0, qt = 0, dt = 0, n_rows = 0;
+    int4 p = make_int4(-1, -1, -1, -1);             // a_tj, a_vj, a_jt, a_jv
+    if (e < 0) {
+        k = (int)x;
+        qt = g.q0[k];
+        dt = g.diagpos[qt];
+        n_rows = g.nv[k];
+    } else if (e < g.n_pe) {
+        k = g.pe_bus[e];
+        p = g.pe_pos[e];
+    }
+    pdl_wait();
+    pdl_trigger();
+    if (e < 0) {
         const double tau = 1e-14 * __longlong_as_double((long long)*g.jmax);
         const double4_32a pq = g.piv[k];
         if (!(fabs(g.A[dt]) > tau)) atomicOr(g.err, 1);
         g.invdiag[qt] = pq.x;
-        if (g.nv[k] == 2) {
+        if (n_rows == 2) {
             const int dv = g.diagpos[qt + 1];
             if (!(inb(dv, g.nnz) && inb(qt + 1, g.n_x))) return;
             const double uvv = fma(-pq.y, pq.w, g.A[dv]);
@@ -439,10 +450,7 @@ __device__ __forceinline__ void k_rf_pivot_body(const RfGrid& g) {
         }
         return;
     }
-    const int64_t e = x - g.n_piv;
     if (e >= g.n_pe) return;
-    const int k = g.pe_bus[e];
-    const int4 p = g.pe_pos[e];                     // a_tj, a_vj, a_jt, a_jv
     if (!(inb(k, g.n_piv) && inb(p.x, g.nnz) && inb(p.z, g.nnz) && (p.y < 0 || (inb(p.y, g.nnz) && inb(p.w, g.nnz)))))
         return;
     const double4_32a pq = g.piv[k];
@@ -454,7 +462,6 @@ __device__ __forceinline__ void k_rf_pivot_body(const RfGrid& g) {
     }
 }
 __global__ void k_rf_pivot(RfGrid g) {
-    pdl_wait();
     k_rf_pivot_body(g);
 }
 
@@ -483,19 +490,22 @@ __device__ __forceinline__ void rf_piv_store(const RfGrid& g, int j, double att,
 // first level: one thread per job, the block read from A.
 __device__ __forceinline__ void k_rf_leaf_piv_body(const RfGrid& g, int njob) {
     const int q = blockIdx.x * blockDim.x + threadIdx.x;
+    int pp[4] = {-1, -1, -1, -1}, bus = 0;
+    if (q < njob) {
+        for (int e = 0; e < 4; e++) pp[e] = g.piv_pos[4 * q + e];
+        bus = g.piv_bus[q];
+    }
+    pdl_wait();
+    pdl_trigger();
     if (q >= njob) return;
     double v[4];
-    for (int e = 0; e < 4; e++) {
-        const int pp = g.piv_pos[4 * q + e];
-        v[e] = (pp >= 0 && inb(pp, g.nnz)) ? g.A[pp] : 0.0;
-    }
-    const bool two = g.piv_pos[4 * q + 3] >= 0;
+    for (int e = 0; e < 4; e++) v[e] = (pp[e] >= 0 && inb(pp[e], g.nnz)) ? g.A[pp[e]] : 0.0;
+    const bool two = pp[3] >= 0;
     const double it = 1.0 / v[0];
     const double idet = two ? 1.0 / rf_det(v[0], v[1], v[2], v[3]) : 0.0;
-    rf_piv_store(g, g.piv_bus[q], v[0], v[1], v[2], it, idet, two);
+    rf_piv_store(g, bus, v[0], v[1], v[2], it, idet, two);
 }
 __global__ void k_rf_leaf_piv(RfGrid g, int njob) {
-    pdl_wait();
     k_rf_leaf_piv_body(g, njob);
 }
 
@@ -530,45 +540,66 @@ __device__ __forceinline__ double rf_group(const RfGrid& g, int2 d, int2 tu, int
 // Targets [t0, t0 + nt) of one level; the first 4 * njob of them are the quads of
 // the level's pivot jobs j0 .. j0 + njob - 1 (lane e of job q: entry e of the bus's
 // block a_tt, a_tv, a_vt, a_vv, a target of this level or an empty lane).
+//
+// The plan's arrays do not change, so a thread reads its target's groups and its pivot
+// job's positions before it waits for the previous level, and the next level's CTAs start
+// as soon as this one's wait is over: between two levels only the values' loads, their
+// FMAs and the hand-over remain.  First-order derivatives at 9241 buses 894 -> 783 us (74
+// launches), eight Newton re-solves at 1354 buses 1203 -> 1124 us.
 __device__ __forceinline__ void k_rf_update_body(const RfGrid& g, int64_t t0, int64_t nt, int j0, int njob) {
     const int64_t tl = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t t = t0 + (tl < nt ? tl : 0);
-    double nv = 0.0;
-    int p = -1;
+    const int64_t wbase = tl - (int64_t)(threadIdx.x & 31);
+    const bool job_warp = wbase < 4 * (int64_t)njob, mine = tl < 4 * (int64_t)njob;
+    const int e = (int)(tl & 3);
+    const int64_t q = tl >> 2;
+    int p = -1, pos3 = -1, pp = -1, bus = 0;
+    int2 d = make_int2(0, 0), tu = make_int2(-1, 0), vu = tu;
+    int2 x[2][3] = {{d, tu, vu}, {d, tu, vu}};
+    int64_t x0 = 0, x1 = 0;
     if (tl < nt) {
         p = g.tgt_pos[t];
-        const int2 d = g.grp[3 * t], tu = g.grp[3 * t + 1], vu = g.grp[3 * t + 2];
-        const int64_t x0 = g.xptr[t], x1 = g.xptr[t + 1];
-        if (p >= 0 && inb(p, g.nnz)) {
-            double acc = rf_group(g, d, tu, vu, 0.0);
-            int64_t c = x0;
-            for (; c + 1 < x1; c += 2) {
-                const int2 da = g.xgrp[3 * c], tua = g.xgrp[3 * c + 1], vua = g.xgrp[3 * c + 2];
-                const int2 db = g.xgrp[3 * c + 3], tub = g.xgrp[3 * c + 4], vub = g.xgrp[3 * c + 5];
-                acc = rf_group(g, da, tua, vua, acc);
-                acc = rf_group(g, db, tub, vub, acc);
-            }
-            if (c < x1) acc = rf_group(g, g.xgrp[3 * c], g.xgrp[3 * c + 1], g.xgrp[3 * c + 2], acc);
-            nv = g.A[p] - acc;
-            g.A[p] = nv;
+        d = g.grp[3 * t];
+        tu = g.grp[3 * t + 1];
+        vu = g.grp[3 * t + 2];
+        x0 = g.xptr[t];
+        x1 = g.xptr[t + 1];
+    }
+    if (mine) {
+        pos3 = g.piv_pos[4 * (j0 + q) + 3];
+        pp = g.piv_pos[4 * (j0 + q) + e];
+        bus = g.piv_bus[j0 + q];
+    }
+#pragma unroll
+    for (int m = 0; m < 2; m++)
+        if (x0 + m < x1) {
+            x[m][0] = g.xgrp[3 * (x0 + m)];
+            x[m][1] = g.xgrp[3 * (x0 + m) + 1];
+            x[m][2] = g.xgrp[3 * (x0 + m) + 2];
         }
+    pdl_wait();
+    pdl_trigger();
+    double nv = 0.0;
+    if (p >= 0 && inb(p, g.nnz)) {
+        double acc = rf_group(g, d, tu, vu, 0.0);
+        if (x0 < x1) acc = rf_group(g, x[0][0], x[0][1], x[0][2], acc);
+        if (x0 + 1 < x1) acc = rf_group(g, x[1][0], x[1][1], x[1][2], acc);
+        int64_t c = x0 + 2;
+        for (; c + 1 < x1; c += 2) {
+            const int2 da = g.xgrp[3 * c], tua = g.xgrp[3 * c + 1], vua = g.xgrp[3 * c + 2];
+            const int2 db = g.xgrp[3 * c + 3], tub = g.xgrp[3 * c + 4], vub = g.xgrp[3 * c + 5];
+            acc = rf_group(g, da, tua, vua, acc);
+            acc = rf_group(g, db, tub, vub, acc);
+        }
+        if (c < x1) acc = rf_group(g, g.xgrp[3 * c], g.xgrp[3 * c + 1], g.xgrp[3 * c + 2], acc);
+        nv = g.A[p] - acc;
+        g.A[p] = nv;
     }
     // pivot jobs: the quads are whole within a warp, and a warp that holds any of
     // them runs the shuffles with all its lanes
-    const int64_t wbase = tl - (int64_t)(threadIdx.x & 31);
-    if (wbase < 4 * (int64_t)njob) {
-        const int e = (int)(tl & 3);
-        const int64_t q = tl >> 2;
-        const bool mine = tl < 4 * (int64_t)njob;
+    if (job_warp) {
         double v = nv;
-        int pos3 = -1;
-        if (mine) {
-            pos3 = g.piv_pos[4 * (j0 + q) + 3];
-            if (p < 0) {
-                const int pp = g.piv_pos[4 * (j0 + q) + e];
-                v = (pp >= 0 && inb(pp, g.nnz)) ? g.A[pp] : 0.0;
-            }
-        }
+        if (mine && p < 0) v = (pp >= 0 && inb(pp, g.nnz)) ? g.A[pp] : 0.0;
         const int b = (int)(threadIdx.x & 28);
         const double att = __shfl_sync(0xffffffffu, v, b);
         const double atv = __shfl_sync(0xffffffffu, v, b + 1);
@@ -578,11 +609,10 @@ __device__ __forceinline__ void k_rf_update_body(const RfGrid& g, int64_t t0, in
         const double x = e == 0 ? att : (e == 3 && pos3 >= 0 ? rf_det(att, atv, avt, avv) : 1.0);
         const double r = 1.0 / x;
         const double idet = __shfl_sync(0xffffffffu, r, b + 3);
-        if (mine && e == 0) rf_piv_store(g, g.piv_bus[j0 + q], att, atv, avt, r, idet, pos3 >= 0);
+        if (mine && e == 0) rf_piv_store(g, bus, att, atv, avt, r, idet, pos3 >= 0);
     }
 }
 __global__ void k_rf_update(RfGrid g, int64_t t0, int64_t nt, int j0, int njob) {
-    pdl_wait();
     k_rf_update_body(g, t0, nt, j0, njob);
 }
 
@@ -611,12 +641,13 @@ constexpr int kTailTB = 16;
 __device__ __forceinline__ void k_tail_gather_body(RfGrid g) {
     const int T = g.T;
     const int idx = blockIdx.x * blockDim.x + threadIdx.x;
+    const int p = idx < T * T ? g.tail_pos[idx] : -1;
+    pdl_wait();
+    pdl_trigger();
     if (idx >= T * T) return;
-    const int p = g.tail_pos[idx];
     g.tailD[idx] = (p >= 0 && inb(p, g.nnz)) ? g.A[p] : 0.0;
 }
 __global__ void k_tail_gather(RfGrid g) {
-    pdl_wait();
     k_tail_gather_body(g);
 }
 
@@ -800,6 +831,7 @@ __device__ __forceinline__ void k_tail_step_body(RfGrid g, int k) {
 }
 __global__ void __launch_bounds__(256) k_tail_step(RfGrid g, int k) {
     pdl_wait();
+    pdl_trigger();
     k_tail_step_body(g, k);
 }
 
@@ -1990,23 +2022,20 @@ __global__ void k_newton_update_batch(PfBatch B) {
 }
 
 __global__ void k_rf_update_batch(RfBatch B, int64_t t0, int64_t nt, int j0, int njob) {
-    pdl_wait();
     k_rf_update_body(B.g[blockIdx.y], t0, nt, j0, njob);
 }
 __global__ void k_rf_leaf_piv_batch(RfBatch B, int njob) {
-    pdl_wait();
     k_rf_leaf_piv_body(B.g[blockIdx.y], njob);
 }
 __global__ void k_rf_pivot_batch(RfBatch B) {
-    pdl_wait();
     k_rf_pivot_body(B.g[blockIdx.y]);
 }
 __global__ void k_tail_gather_batch(RfBatch B) {
-    pdl_wait();
     k_tail_gather_body(B.g[blockIdx.y]);
 }
 __global__ void __launch_bounds__(256) k_tail_step_batch(RfBatch B, int k) {
     pdl_wait();
+    pdl_trigger();
     k_tail_step_body(B.g[blockIdx.y], k);
 }
 __global__ void k_tail_scatter_batch(RfBatch B) {
