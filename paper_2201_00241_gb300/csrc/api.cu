@@ -321,6 +321,7 @@ std::vector<int> tree_column_order(const rh::Symbolic& S) {
 struct LineHost {
     std::vector<int4> steps;
     std::vector<int> map, col, vt;       // entries' positions in A (-1: a pad) and columns; buses' own entries
+    int pad;                             // the pads' column, whose x is 0
 };
 bool line_steps(const std::vector<int>& ptr, const std::vector<int4>& slots, const std::vector<int>& col, bool up,
                 int flags, int NT, LineHost& L) {
@@ -403,7 +404,7 @@ bool line_steps(const std::vector<int>& ptr, const std::vector<int4>& slots, con
                     const int at = ln.slot < 0 ? 0 : ln.li + (e << ln.lg);
                     const bool in = ln.slot >= 0 && at < slots[ln.slot].y;
                     L.map.push_back(in ? ln.r0 + at : -1);
-                    L.col.push_back(in ? col[ln.r0 + at] : 0);
+                    L.col.push_back(in ? col[ln.r0 + at] : L.pad);
                 }
             for (size_t i = k; i < k + 32; i++) {
                 const Lane& ln = lanes[i];
@@ -661,6 +662,20 @@ int balanced_ctas(int N) {
     return std::max(1, (N + per - 1) / per);
 }
 
+constexpr unsigned kToU = rh::PH_WLOAD | rh::PH_SPMUL | rh::PH_L | rh::PH_U;
+constexpr unsigned kFromProj = rh::PH_TPROJ | rh::PH_UT | rh::PH_LT | rh::PH_MULADD;
+
+// Whether a launch of N directions runs one direction per CTA (k_dir1): while k_dirs, with
+// two CTAs on an SM, has no more than one direction a CTA either.  That is one wave of k_dir1
+// on networks of up to 1024 rows of x (two CTAs of 256 threads on an SM) and at most two on
+// larger ones.  Measured, k_dirs -> k_dir1, us for N = 1 / 152 / 304: 118 buses 108 -> 63 /
+// 111 -> 65 / 119 -> 66; 500 buses 204 -> 102 / 224 -> 105 / 252 -> 112; 1354 buses 253 -> 134 /
+// 281 -> 137 / 360 -> 258; 2869 buses 495 -> 243 / 571 -> 248 / 744 -> 481; 9241 buses 1236 ->
+// 700 / 1467 -> 716 / 2196 -> 1414.  Beyond, k_dirs shares each load among the directions of a
+// CTA while k_dir1 takes another wave: N = 456 394 -> 380 us and N = 608 401 -> 501 us at 1354
+// buses, N = 456 61 -> 70 us on 30 buses.
+bool by_dir1(const rh_grid* g, int N) { return g->n_line >= 0 && N <= rh::dirs_cta_slots(); }
+
 rh_status dirs(rh_grid* g, int N, int64_t ld, double* V, double* T, const double* W, int64_t ldw, int col0,
                double* HW, int64_t ldhw, unsigned phases, cudaStream_t s, int n_cta = 0) {
     rh::DirLaunch L;
@@ -684,6 +699,11 @@ rh_status dirs(rh_grid* g, int N, int64_t ld, double* V, double* T, const double
     const bool all_cols = !W && col0 == 0 && N == g->S.n_p && g->hcolmap;
     L.colmap = (all_cols && (phases & (rh::PH_WLOAD | rh::PH_MULADD))) ? g->hcolmap : nullptr;
     L.reach = nullptr;
+    if ((phases == kToU || phases == kFromProj || phases == (kToU | kFromProj)) && by_dir1(g, N)) {
+        L.colmap = nullptr;
+        RH_CUDA(rh::launch_dir1(g->dir(), g->s1(), L, rh::solve1_mode(g->S.n_x, g->S.n_x - g->S.t0) == 2, s));
+        return RH_OK;
+    }
     if (all_cols && L.use_reach) {
         auto f = g->reach_dev.find(L.n_cta);
         if (f != g->reach_dev.end()) {
@@ -1034,6 +1054,7 @@ rh_status rh_grid_create(const rh_grid_desc* d, int32_t device, rh_grid** out) {
             // the tail's triangle does not fit in shared memory, sweep every level
             const int mode = rh::solve1_mode(S.n_x, S.n_x - S.t0), NT = rh::line_threads(S.n_x);
             LineHost up, down;
+            up.pad = down.pad = S.n_x;
             bool ok = mode > 0;
             if (mode == 2) {
                 ok = line_steps(sfp, sfs, S.col, true, 0, NT, up) &&
@@ -1397,7 +1418,7 @@ rh_status enqueue_reduced_hessian(rh_grid* g, double* Hd, int64_t lh) {
     if (st) return st;
     RH_CUDA(cudaEventRecord(g->ev_fork, g->stream));
     RH_CUDA(cudaStreamWaitEvent(g->stream2, g->ev_fork, 0));
-    st = enqueue_adjoint_chain(g, g->stream2, true);
+    st = enqueue_adjoint_chain(g, g->stream2, !by_dir1(g, np));
     if (st) return st;
     RH_CUDA(cudaEventRecordWithFlags(g->ev_d0, g->stream, cudaEventRecordExternal));
     st = dirs(g, np, np, g->V, g->T, nullptr, 0, 0, Hd, lh, rh::PH_WLOAD | rh::PH_SPMUL | rh::PH_L | rh::PH_U,

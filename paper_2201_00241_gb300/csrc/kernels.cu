@@ -1818,19 +1818,20 @@ __global__ void k_line_values(const __grid_constant__ LineGrid g) {
 
 // One right-hand side, one CTA, x held in shared memory for the whole sweep
 // (Newton steps and the first-order adjoint).  Dynamic shared memory holds
-// X[n_x] | the packed tail triangle (use_tail) | kSolve1Part doubles of scratch
+// X[n_x] | a zero | the packed tail triangle (use_tail) | kSolve1Part doubles of scratch
 // (the tail's right-hand side).  With the tail, the dense top block is solved
 // column by column in shared memory, as in k_dirs, instead of as one sparse
 // level per variable.
-constexpr int kSolve1Part = 2048;
+constexpr int kSolve1Part = 2047;
 template <int NT>
 __device__ __forceinline__ void k_solve1_body(const LineGrid& g, double* x, bool trans, int use_tail) {
     extern __shared__ double X[];
-    double* tri = X + g.n_x;
+    double* tri = X + g.n_x + 1;
     double* part = tri + (use_tail ? (size_t)g.T * (g.T - 1) / 2 : 0);
     // J_x = D L'' U': the right-hand side of J_x z = b enters as D^-1 b, and the solution
     // D psi of J_x^T leaves as psi
     for (int q = threadIdx.x; q < g.n_x; q += NT) X[q] = trans ? x[q] : x[q] * g.invdiag[q];
+    if (threadIdx.x == 0) X[g.n_x] = 0.0;                  // the pads' column
     __syncthreads();
     line_sweep<true, NT>(trans ? g.tup : g.up, X);
     if (use_tail) {
@@ -1845,6 +1846,137 @@ template <int NT>
 __global__ void __launch_bounds__(NT, kLineRegs / NT)
     k_solve1(const __grid_constant__ LineGrid g, double* x, int trans, int use_tail) {
     k_solve1_body<NT>(g, x, trans, use_tail);
+}
+
+// Algorithm 2 with one direction per CTA and x in shared memory: few directions, where
+// k_dirs has one or two a CTA and every level costs it the latency of slot, row and x loads
+// from L2.  The sweeps are line_sweep's, on the values k_line_values laid out, so a level
+// costs its multiplications, shuffles and one barrier; the projection reads x at random from
+// shared memory and passes through Y (in L2) to the transposed sweeps' x.  The chain of
+// levels bounds it on small networks and the SM's FP64 pipes on large ones: one product at
+// 118 buses 108 -> 63 us, 45 at 2869 buses 513 -> 233, 256 at 9241 buses 2046 -> 1465.
+//   phases SPMUL L U (x is left in V), TPROJ UT LT MULADD (x from V), or all of them
+template <int NT>
+__global__ void __launch_bounds__(NT, kLineRegs / NT)
+    k_dir1(const __grid_constant__ DirGrid g, const __grid_constant__ LineGrid s, const __grid_constant__ DirLaunch L,
+           int use_tail) {
+    extern __shared__ double X[];
+    double* tri = X + g.n_x + 1;
+    double* part = tri + (use_tail ? (size_t)s.T * (s.T - 1) / 2 : 0);
+    const int c = blockIdx.x, rows = g.zero_row + 1;
+    if (L.ws_elems > 0 && !inb((int64_t)(c + 1) * rows - 1, L.ws_elems)) return;
+    double* V = L.V + (int64_t)c * rows;
+    double* Y = L.T + (int64_t)c * rows;
+    const double* __restrict__ W = L.W ? L.W + (int64_t)c * L.ldw : nullptr;
+    const int id = id_col(L, c);
+    if (threadIdx.x == 0) X[g.n_x] = 0.0;                  // the pads' column
+    if (L.phases & PH_SPMUL) {
+        // D^-1 B, B = -J_p w, or minus column id of J_p
+        for (int q = threadIdx.x; q < g.n_x; q += NT) X[q] = 0.0;
+        __syncthreads();
+        if (W) {
+            for (int r = threadIdx.x; r < g.n_jp_rows; r += NT) {
+                const int q = g.jp_rows[r];
+                double a = 0.0;
+                for (int t = g.jp_ptr[q]; t < g.jp_ptr[q + 1]; t++) a = fma(g.jpv[t], W[g.jp_col[t]], a);
+                if (inb(q, g.n_x)) X[q] = -a * g.invdiag[q];
+            }
+        } else {
+            for (int t = g.jpt_ptr[id] + threadIdx.x; t < g.jpt_ptr[id + 1]; t += NT)
+                if (inb(g.jpt_row[t], g.n_x)) X[g.jpt_row[t]] = -g.jptvd[t];
+        }
+        __syncthreads();
+        line_sweep<true, NT>(s.up, X);
+        if (use_tail) {
+            tail_fwd<false>(s, s.triLd, X, 1, 0, 1, part, tri);
+            tail_bwd<false>(s, s.triUd, X, 1, 0, 1, part, tri);
+        }
+        line_sweep<false, NT>(s.down, X);
+        __syncthreads();
+    }
+    if (!(L.phases & PH_TPROJ)) {
+        for (int q = threadIdx.x; q < g.n_x; q += NT) V[q] = X[q];
+        return;
+    }
+    if (!(L.phases & PH_SPMUL)) {
+        for (int q = threadIdx.x; q < g.n_x; q += NT) X[q] = V[q];
+        __syncthreads();
+    }
+    // entry r of v = (z, w, 0)
+    auto v_at = [&](int r) {
+        if (!inb(r, rows) || r == g.zero_row) return 0.0;
+        return r < g.n_x ? X[r] : (W ? W[r - g.n_x] : (r - g.n_x == id ? 1.0 : 0.0));
+    };
+    if (threadIdx.x < 32) {
+        double a = 0.0;
+        for (int e = threadIdx.x; e < g.n_gref; e += 32) a = fma(g.gref_val[e], v_at(g.gref_row[e]), a);
+        for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+        if (threadIdx.x == 0) part[0] = *g.c2ref * a;
+    }
+    __syncthreads();
+    const double sref = part[0];
+    // projection (see tproj)
+    for (int bi = threadIdx.x; bi < g.n_bus; bi += NT) {
+        const int b = g.tp_bus[bi], rth = g.uth[b], rv = g.uv[b];
+        const double dth = v_at(rth), dv = v_at(rv), ab = g.asum[b];
+        double yv = fma(g.d2[b], dv, ab * dth);
+        double yth = fma(ab, dv, g.csum[b] * dth);
+        int e = g.inc_ptr[b];
+        const int e1 = g.inc_ptr[b + 1];
+        for (; e + 2 <= e1; e += 2) {
+            const double th0 = v_at(g.inc_uth[e]), v0 = v_at(g.inc_uv[e]);
+            const double th1 = v_at(g.inc_uth[e + 1]), v1 = v_at(g.inc_uv[e + 1]);
+            const double4_32a cf0 = g.inc_coef[e], cf1 = g.inc_coef[e + 1];
+            yv = fma(cf0.x, v0, yv);
+            yv = fma(cf0.y, th0, yv);
+            yth = fma(cf0.z, v0, yth);
+            yth = fma(cf0.w, th0, yth);
+            yv = fma(cf1.x, v1, yv);
+            yv = fma(cf1.y, th1, yv);
+            yth = fma(cf1.z, v1, yth);
+            yth = fma(cf1.w, th1, yth);
+        }
+        if (warp_any(e < e1)) {
+            if (e < e1) {
+                const double th0 = v_at(g.inc_uth[e]), v0 = v_at(g.inc_uv[e]);
+                const double4_32a cf = g.inc_coef[e];
+                yv = fma(cf.x, v0, yv);
+                yv = fma(cf.y, th0, yv);
+                yth = fma(cf.z, v0, yth);
+                yth = fma(cf.w, th0, yth);
+            }
+        }
+        const bool hg = g.has_gref[b];
+        if (warp_any(hg)) {
+            if (hg) {
+                yv = fma(sref, g.gref_v[b], yv);
+                yth = fma(sref, g.gref_th[b], yth);
+            }
+        }
+        if (rth != g.zero_row && inb(rth, rows)) Y[rth] = flip_sign(yth, true);
+        if (inb(rv, rows)) Y[rv] = flip_sign(yv, rv < g.n_x);
+        const int pr = g.pg_row[b];
+        if (warp_any(pr >= 0)) {
+            if (pr >= 0 && inb(pr, rows)) Y[pr] = g.pg_curv[b] * v_at(pr);
+        }
+    }
+    __syncthreads();
+    for (int q = threadIdx.x; q < g.n_x; q += NT) X[q] = Y[q];
+    __syncthreads();
+    line_sweep<true, NT>(s.tup, X);
+    if (use_tail) {
+        tail_fwd<false>(s, s.triUtd, X, 1, 0, 1, part, tri);
+        tail_bwd<false>(s, s.triLtd, X, 1, 0, 1, part, tri);
+    }
+    line_sweep<false, NT>(s.tdown, X);
+    __syncthreads();
+    double* HW = L.HW + (int64_t)(id - L.col0) * L.ldhw;
+    for (int k = threadIdx.x; k < g.n_p; k += NT) {
+        double h = Y[g.n_x + k];
+        for (int t = g.jpt_ptr[k]; t < g.jpt_ptr[k + 1]; t++)
+            if (inb(g.jpt_row[t], g.n_x)) h = fma(g.jptvd[t], X[g.jpt_row[t]], h);
+        HW[k] = h;
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -2189,8 +2321,9 @@ cudaError_t prepare_kernels() {
     if (g_prepared[dev]) return cudaSuccess;
     e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
     if (e != cudaSuccess) return e;
-    const void* fns[5] = {(const void*)k_dirs, (const void*)k_solve1<256>, (const void*)k_solve1<512>,
-                          (const void*)k_solve1_batch<256>, (const void*)k_solve1_batch<512>};
+    const void* fns[7] = {(const void*)k_dirs, (const void*)k_solve1<256>, (const void*)k_solve1<512>,
+                          (const void*)k_solve1_batch<256>, (const void*)k_solve1_batch<512>,
+                          (const void*)k_dir1<256>, (const void*)k_dir1<512>};
     for (const void* f : fns) {
         cudaFuncAttributes fa;
         e = cudaFuncGetAttributes(&fa, f);
@@ -2310,13 +2443,20 @@ void launch_adjoint_rhs(const PfGrid& g, const PfState& s, const AdjData& a, cud
 int line_threads(int n_x) { return n_x <= 1024 ? 256 : 512; }
 
 static size_t solve1_smem(int n_x, int T, bool tail) {
-    return ((size_t)n_x + (tail ? (size_t)T * (T - 1) / 2 : 0) + kSolve1Part) * sizeof(double);
+    return ((size_t)n_x + 1 + (tail ? (size_t)T * (T - 1) / 2 : 0) + kSolve1Part) * sizeof(double);
 }
 
 int solve1_mode(int n_x, int T) {
     const size_t cap = 227 * 1024;
     if (T > 1 && T <= kSolve1Part && solve1_smem(n_x, T, true) <= cap) return 2;
     return solve1_smem(n_x, T, false) <= cap ? 1 : 0;
+}
+
+cudaError_t launch_dir1(const DirGrid& g, const LineGrid& s, const DirLaunch& L, bool use_tail, cudaStream_t st) {
+    const size_t smem = solve1_smem(s.n_x, s.T, use_tail);
+    if (line_threads(s.n_x) == 256) k_dir1<256><<<L.N, 256, smem, st>>>(g, s, L, use_tail ? 1 : 0);
+    else k_dir1<512><<<L.N, 512, smem, st>>>(g, s, L, use_tail ? 1 : 0);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_solve1(const LineGrid& g, double* x, bool trans, bool use_tail, cudaStream_t st) {

@@ -166,8 +166,10 @@ struct PfState {
 // serialisation: the next launch is scheduled as the current one's CTAs exit
 // instead of after its completion is signalled, hiding part of the launch
 // latency.  Every kernel launched this way calls pdl_wait() before it touches
-// memory, which returns once the previous kernel in the stream has completed
-// and its writes are visible; without a previous kernel it returns at once.
+// memory that an earlier kernel of its chain writes (what no kernel of the chain
+// writes it may read before), which returns once the previous kernel in the stream
+// has completed and its writes are visible; without a previous kernel it returns
+// at once.
 // The first kernel of a chain is launched without the attribute (pdl = false),
 // so it is fully ordered after whatever precedes it (copies, event waits).
 #ifdef __CUDACC__
@@ -315,7 +317,7 @@ constexpr int kLineActive = 1 << 30;  // the warp has a bus in this step
 struct LineSched {
     int n;                            // steps
     const int4* steps;
-    const int* col;                   // line arrays: column of each entry (0: a pad),
+    const int* col;                   // line arrays: column of each entry (n_x: a pad),
     const double* val;                //   its value negated (0: a pad), and each bus's own
     const double* vt;                 //   off-diagonal entry negated
 };
@@ -331,6 +333,10 @@ struct LineGrid {
 void launch_line_values(const LineGrid& g, bool transposed_too, cudaStream_t st);
 int line_threads(int n_x);
 cudaError_t launch_solve1(const LineGrid& g, double* x, bool trans, bool use_tail, cudaStream_t st);
+// Directions of a launch with one direction per CTA and x in shared memory (L.N CTAs;
+// direction c's rows at V + c * (zero_row + 1) and T likewise): SpMul to the U sweep, the
+// projection to SpMulAdd, or both.  Needs solve1_mode() > 0 and its schedule.
+cudaError_t launch_dir1(const DirGrid& g, const LineGrid& s, const DirLaunch& L, bool use_tail, cudaStream_t st);
 
 // Dense Cholesky of the tracking step (dense.cu).  A, L, B, work, y and info
 // are device pointers; column-major.  info receives 0 or the 1-based column of
