@@ -101,7 +101,7 @@ struct rh_grid {
     int* hcolmap = nullptr;
     std::vector<int> colmap;                    // host copy
     std::map<int, rh::ReachSched*> reach_dev;   // device structs, keyed by the launch's CTA count
-    int *tp_bus = nullptr, *uth = nullptr, *uv = nullptr, *inc_ptr = nullptr, *inc_nb = nullptr;
+    int *tp_bus = nullptr, *uth = nullptr, *uv = nullptr, *inc_ptr = nullptr;
     int* tp_l0 = nullptr;   // per bus: position of (v, theta) in At for a PQ bus of forward level 0, else -1
     int *inc_uth = nullptr, *inc_uv = nullptr, *gref_row = nullptr, *pg_row = nullptr, *xmap = nullptr;
     uint8_t* has_gref = nullptr;
@@ -724,14 +724,14 @@ rh_status dirs(rh_grid* g, int N, int64_t ld, double* V, double* T, const double
     return RH_OK;
 }
 
-// single right-hand side in g->v1 (internal order), in place.  beside_dirs: as
+// single right-hand side in g->v1 (internal order), the solution in `out`.  beside_dirs: as
 // one CTA of the direction kernel, which fits in the slot a direction launch of
 // fewer CTAs than the device holds leaves free (k_solve1's shared-memory x
 // needs a shared-memory carveout that an SM running k_dirs does not have).
-rh_status solve_one(rh_grid* g, unsigned phases, cudaStream_t s, bool beside_dirs = false) {
+rh_status solve_one(rh_grid* g, unsigned phases, double* out, cudaStream_t s, bool beside_dirs = false) {
     const int mode = beside_dirs || g->n_line < 0 ? 0 : rh::solve1_mode(g->S.n_x, g->S.n_x - g->S.t0);
     if (mode > 0) {
-        RH_CUDA(rh::launch_solve1(g->s1(), g->v1, (phases & rh::PH_LT) != 0, mode == 2, s));
+        RH_CUDA(rh::launch_solve1(g->s1(), g->v1, out, (phases & rh::PH_LT) != 0, mode == 2, s));
         return RH_OK;
     }
     // through k_dirs, whose factors are unit-diagonal (J_x = D L'' U'): the right-hand
@@ -740,6 +740,7 @@ rh_status solve_one(rh_grid* g, unsigned phases, cudaStream_t s, bool beside_dir
     rh_status st = dirs(g, 1, 1, g->v1, g->v1, nullptr, 0, 0, nullptr, 0, phases, s);
     if (st) return st;
     if (phases & rh::PH_LT) rh::launch_scale_rows(g->S.n_x, 1, g->invdiag, g->v1, 1, s);
+    if (out != g->v1) RH_CUDA(cudaMemcpyAsync(out, g->v1, g->S.n_x * sizeof(double), cudaMemcpyDeviceToDevice, s));
     return RH_OK;
 }
 
@@ -894,7 +895,7 @@ rh_status rh_grid_create(const rh_grid_desc* d, int32_t device, rh_grid** out) {
     int zero_row = nx + np;
 
     // projection structure
-    std::vector<int> uth(nb), uv(nb), pg_row(nb, -1), inc_ptr(nb + 1, 0), inc_nb, inc_uth, inc_uv;
+    std::vector<int> uth(nb), uv(nb), pg_row(nb, -1), inc_ptr(nb + 1, 0), inc_uth, inc_uv;
     std::vector<uint8_t> has_gref(nb, 0);
     for (int i = 0; i < nb; i++) {
         uth[i] = S.qth[i] >= 0 ? S.qth[i] : zero_row;
@@ -905,15 +906,14 @@ rh_status rh_grid_create(const rh_grid_desc* d, int32_t device, rh_grid** out) {
         for (int t = S.yp[i]; t < S.yp[i + 1]; t++) {
             int j = S.yj[t];
             if (j == i) continue;
-            inc_nb.push_back(j);
             inc_uth.push_back(uth[j]);
             inc_uv.push_back(uv[j]);
         }
-        inc_ptr[i + 1] = (int)inc_nb.size();
+        inc_ptr[i + 1] = (int)inc_uth.size();
     }
     has_gref[S.ref] = 1;
     for (int t = S.yp[S.ref]; t < S.yp[S.ref + 1]; t++) has_gref[S.yj[t]] = 1;
-    g->n_inc = (int)inc_nb.size();
+    g->n_inc = (int)inc_uth.size();
     g->n_gref = 1 + 2 * (S.yp[S.ref + 1] - S.yp[S.ref] - 1);
     // projection order: degree descending, then buses with a Pg row, then elimination order, so
     // that the lanes of a warp share their incidence count and their branches
@@ -1145,7 +1145,6 @@ rh_status rh_grid_create(const rh_grid_desc* d, int32_t device, rh_grid** out) {
     RH_CUDA(g->upload(g->uth, uth));
     RH_CUDA(g->upload(g->uv, uv));
     RH_CUDA(g->upload(g->inc_ptr, inc_ptr));
-    RH_CUDA(g->upload(g->inc_nb, inc_nb));
     RH_CUDA(g->upload(g->inc_uth, inc_uth));
     RH_CUDA(g->upload(g->inc_uv, inc_uv));
     RH_CUDA(g->upload(g->has_gref, has_gref));
@@ -1304,7 +1303,7 @@ rh_status rh_powerflow(rh_grid* g, const double* x0, double tol, int32_t max_ite
             g,
             [&]() -> rh_status {
                 RH_CUDA(cudaMemcpyAsync(g->v1, g->gres, nx * sizeof(double), cudaMemcpyDeviceToDevice, g->stream));
-                rh_status ss = solve_one(g, rh::PH_L | rh::PH_U, g->stream);
+                rh_status ss = solve_one(g, rh::PH_L | rh::PH_U, g->v1, g->stream);
                 if (ss) return ss;
                 rh::launch_newton_update(g->pf(), g->st(), g->v1, g->stream);
                 return assemble(g, g->jac_method, g->gres, g->stream);
@@ -1373,20 +1372,18 @@ namespace {
 // The adjoint (eq. 7) on the current factors: right-hand side and F, the transposed
 // single solve, lambda, the projection coefficients and grad F (enqueue only).
 rh_status enqueue_adjoint_chain(rh_grid* g, cudaStream_t s, bool beside_dirs) {
-    const auto& S = g->S;
-    RH_CUDA(cudaMemsetAsync(g->v1, 0, sizeof(double) * g->rows(), s));
     rh::AdjData a;
-    a.rhs = g->v1; a.cref = g->dscal; a.c2ref = g->dscal + 1; a.F = g->dscal + 2;
+    a.rhs = g->v1; a.n_rhs = g->rows(); a.cref = g->dscal; a.c2ref = g->dscal + 1; a.F = g->dscal + 2;
     a.gref_th = g->gref_th; a.gref_v = g->gref_v; a.gref_row = g->gref_row; a.gref_val = g->gref_val;
     a.n_gref = g->n_gref; a.uth = g->uth; a.uv = g->uv;
     rh::launch_adjoint_rhs(g->pf(), g->st(), a, s);
-    rh_status st = solve_one(g, rh::PH_UT | rh::PH_LT, s, beside_dirs);
+    rh_status st = solve_one(g, rh::PH_UT | rh::PH_LT, g->lam, s, beside_dirs);
     if (st) return st;
-    RH_CUDA(cudaMemcpyAsync(g->lam, g->v1, S.n_x * sizeof(double), cudaMemcpyDeviceToDevice, s));
-    rh::launch_adjoint_coef(g->pf(), g->st(), g->lam, g->dscal, g->inc_ptr, g->inc_nb, g->inc_coef, g->d2, g->asum,
-                            g->csum, g->pg_curv, s);
-    rh::launch_gradient(g->pf(), g->st(), S.n_p, g->jpt_ptr, g->jpt_row, g->jptv, g->lam, g->dscal, g->gref_v,
-                        g->grad, s);
+    rh::CoefData c;
+    c.lam = g->lam; c.cref = g->dscal; c.gref_v = g->gref_v; c.inc_ptr = g->inc_ptr; c.coef = g->inc_coef;
+    c.d2 = g->d2; c.asum = g->asum; c.csum = g->csum; c.pg_curv = g->pg_curv;
+    c.jpt_ptr = g->jpt_ptr; c.jpt_row = g->jpt_row; c.jptv = g->jptv; c.grad = g->grad;
+    rh::launch_adjoint_coef(g->pf(), g->st(), c, s);
     RH_CUDA(cudaGetLastError());
     return RH_OK;
 }
@@ -1512,7 +1509,7 @@ rh_status enqueue_batch_newton(rh_grid* const* items, int n, uint32_t mask, int 
         // x does not fit in one CTA's shared memory: the direction kernel solves each item
         for (rh_grid* g : act) {
             enqueue_factor_copies(g, s);
-            rh_status st = solve_one(g, rh::PH_L | rh::PH_U, s);
+            rh_status st = solve_one(g, rh::PH_L | rh::PH_U, g->v1, s);
             if (st) return st;
         }
     }

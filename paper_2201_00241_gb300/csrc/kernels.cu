@@ -1824,7 +1824,8 @@ __global__ void k_line_values(const __grid_constant__ LineGrid g) {
 // level per variable.
 constexpr int kSolve1Part = 2047;
 template <int NT>
-__device__ __forceinline__ void k_solve1_body(const LineGrid& g, double* x, bool trans, int use_tail) {
+__device__ __forceinline__ void k_solve1_body(const LineGrid& g, const double* x, double* out, bool trans,
+                                              int use_tail) {
     extern __shared__ double X[];
     double* tri = X + g.n_x + 1;
     double* part = tri + (use_tail ? (size_t)g.T * (g.T - 1) / 2 : 0);
@@ -1840,12 +1841,12 @@ __device__ __forceinline__ void k_solve1_body(const LineGrid& g, double* x, bool
     }
     line_sweep<false, NT>(trans ? g.tdown : g.down, X);
     __syncthreads();
-    for (int q = threadIdx.x; q < g.n_x; q += NT) x[q] = trans ? X[q] * g.invdiag[q] : X[q];
+    for (int q = threadIdx.x; q < g.n_x; q += NT) out[q] = trans ? X[q] * g.invdiag[q] : X[q];
 }
 template <int NT>
 __global__ void __launch_bounds__(NT, kLineRegs / NT)
-    k_solve1(const __grid_constant__ LineGrid g, double* x, int trans, int use_tail) {
-    k_solve1_body<NT>(g, x, trans, use_tail);
+    k_solve1(const __grid_constant__ LineGrid g, const double* x, double* out, int trans, int use_tail) {
+    k_solve1_body<NT>(g, x, out, trans, use_tail);
 }
 
 // Algorithm 2 with one direction per CTA and x in shared memory: few directions, where
@@ -1983,125 +1984,176 @@ __global__ void __launch_bounds__(NT, kLineRegs / NT)
 // adjoint (eq. 7) and the per-state second-order coefficients
 // ---------------------------------------------------------------------------
 
-// Single thread: the slack cost derivatives, grad P_slack, the right-hand side
-// -grad_x f = -c'_slack grad_x P_slack of the adjoint system, and F.
-__global__ void k_adjoint_rhs(PfGrid g, PfState s, AdjData a) {
-    if (blockIdx.x != 0 || threadIdx.x != 0) return;
+// Block 0: the slack cost derivatives, grad P_slack, the right-hand side
+// -grad_x f = -c'_slack grad_x P_slack of the adjoint system (the rest of rhs is
+// zeroed), one thread per admittance entry of the slack.  Block 1: F = sum over
+// generators of c2 (S Pg)^2 + c1 S Pg in a fixed order.  Both are single blocks on the
+// critical path, bound by their chains of loads; as one thread and a block of 256 after it
+// they took 15 + 47 us at 9241 buses.  With k_adjoint_coef, first-order derivatives at 9241
+// buses 783 -> 707 us, the reduced Hessian at 118 buses 217 -> 185 us.
+constexpr int kAdjThreads = 1024;
+__global__ void __launch_bounds__(kAdjThreads) k_adjoint_rhs(PfGrid g, PfState s, AdjData a) {
+    const double S = g.base_mva;
     const int r = g.ref;
-    const double S = g.base_mva;
-    double vr = s.vm[r], Pr = s.P[r];
-    double pg_ref = Pr + s.pd[r];
-    double cref = 2.0 * g.c2[r] * S * S * pg_ref + g.c1[r] * S;
-    *a.cref = cref;
-    *a.c2ref = 2.0 * g.c2[r] * S * S;
-    int n = 0;
-    for (int t = g.yp[r]; t < g.yp[r + 1]; t++) {
-        int j = g.yj[t];
-        if (j == r) {
-            double dv = Pr / vr + g.G[t] * vr;
-            a.gref_v[r] = dv;
-            a.gref_th[r] = 0.0;
-            a.gref_row[n] = a.uv[r];
-            a.gref_val[n++] = dv;
-            continue;
-        }
-        double sn, cs;
-        sincos(s.va[r] - s.va[j], &sn, &cs);
-        double vj = s.vm[j];
-        double dth = vr * vj * (g.G[t] * sn - g.B[t] * cs);
-        double dv = vr * (g.G[t] * cs + g.B[t] * sn);
-        a.gref_th[j] = dth;
-        a.gref_v[j] = dv;
-        a.gref_row[n] = a.uth[j];
-        a.gref_val[n++] = dth;
-        a.gref_row[n] = a.uv[j];
-        a.gref_val[n++] = dv;
-        a.rhs[g.qth[j]] = -cref * dth;
-        if (g.qv[j] >= 0) a.rhs[g.qv[j]] = -cref * dv;
-    }
-}
-
-// F = sum over generators of c2 (S Pg)^2 + c1 S Pg, one block, fixed reduction order.
-__global__ void k_objective(PfGrid g, PfState s, double* F) {
-    __shared__ double red[256];
-    const double S = g.base_mva;
-    double acc = 0.0;
-    for (int i = threadIdx.x; i < g.n_bus; i += blockDim.x) {
-        if (g.qv[i] >= 0) continue;  // PQ bus: no generator
-        double pg = (i == g.ref) ? s.P[i] + s.pd[i] : s.pg[i];
-        double P = S * pg;
-        acc += g.c2[i] * P * P + g.c1[i] * P;
-    }
-    red[threadIdx.x] = acc;
-    __syncthreads();
-    for (int h = blockDim.x / 2; h > 0; h >>= 1) {
-        if ((int)threadIdx.x < h) red[threadIdx.x] += red[threadIdx.x + h];
+    if (blockIdx.x == 0) {
+        for (int q = threadIdx.x; q < a.n_rhs; q += kAdjThreads) a.rhs[q] = 0.0;
         __syncthreads();
+        const double vr = s.vm[r], Pr = s.P[r];
+        const double cref = 2.0 * g.c2[r] * S * S * (Pr + s.pd[r]) + g.c1[r] * S;
+        if (threadIdx.x == 0) {
+            *a.cref = cref;
+            *a.c2ref = 2.0 * g.c2[r] * S * S;
+        }
+        const int t0 = g.yp[r], td = g.ydiag[r];
+        for (int t = t0 + threadIdx.x; t < g.yp[r + 1]; t += kAdjThreads) {
+            const int j = g.yj[t], n = 2 * (t - t0) - (t > td);    // two entries a neighbour, one for the slack
+            if (j == r) {
+                const double dv = Pr / vr + g.G[t] * vr;
+                a.gref_v[r] = dv;
+                a.gref_th[r] = 0.0;
+                a.gref_row[n] = a.uv[r];
+                a.gref_val[n] = dv;
+                continue;
+            }
+            double sn, cs;
+            sincos(s.va[r] - s.va[j], &sn, &cs);
+            const double vj = s.vm[j];
+            const double dth = vr * vj * (g.G[t] * sn - g.B[t] * cs);
+            const double dv = vr * (g.G[t] * cs + g.B[t] * sn);
+            a.gref_th[j] = dth;
+            a.gref_v[j] = dv;
+            a.gref_row[n] = a.uth[j];
+            a.gref_val[n] = dth;
+            a.gref_row[n + 1] = a.uv[j];
+            a.gref_val[n + 1] = dv;
+            a.rhs[g.qth[j]] = -cref * dth;
+            if (g.qv[j] >= 0) a.rhs[g.qv[j]] = -cref * dv;
+        }
+        return;
     }
-    if (threadIdx.x == 0) *F = red[0];
+    __shared__ double red[32];
+    double acc = 0.0;
+#pragma unroll 4
+    for (int i = threadIdx.x; i < g.n_bus; i += kAdjThreads) {
+        // a PQ bus has no generator
+        const double pg = g.qv[i] >= 0 ? 0.0 : (i == r ? s.P[i] + s.pd[i] : s.pg[i]);
+        const double P = S * pg, c = g.c2[i] * P * P + g.c1[i] * P;
+        if (g.qv[i] < 0) acc += c;
+    }
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        acc = red[threadIdx.x];
+        for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+        if (threadIdx.x == 0) *a.F = acc;
+    }
 }
 
-// One thread per bus: bus weights mu, nu from lambda (mu_slack = c'_slack) and
-// the coefficients of every incident branch for the gathered projection.
+// Bus weights mu, nu from lambda (mu_slack = c'_slack) and the coefficients of every
+// incident branch for the gathered projection.
 // With alpha = G(mu_i + mu_j) - B(nu_i + nu_j), beta = B(mu_i - mu_j) + G(nu_i - nu_j),
 // t = theta_i - theta_j, the branch term of sum mu P + nu Q is
 // v_i v_j (alpha cos t + beta sin t); K = alpha cos t + beta sin t,
 // M = dK/dt, a = v_j M, b = v_i M, c = -v_i v_j K.
-__global__ void k_adjoint_coef(PfGrid g, PfState s, const double* lam, const double* crefp, const int* inc_ptr,
-                               const int* inc_nb, double4_32a* coef, double* d2, double* asum, double* csum,
-                               double* pg_curv) {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
+struct CoefBus {
+    double mu, nu, v;
+};
+constexpr int kCoefThreads = 128;
+__device__ __forceinline__ CoefBus coef_bus(const PfGrid& g, const PfState& s, const CoefData& c, int i) {
+    return {g.qth[i] >= 0 ? c.lam[g.qth[i]] : *c.cref, g.qv[i] >= 0 ? c.lam[g.qv[i]] : 0.0, s.vm[i]};
+}
+// admittance entry t = (i, j), j != i: its coefficients, and a and c for the bus's sums
+__device__ __forceinline__ double4_32a coef_entry(const PfGrid& g, const PfState& s, const CoefData& c, int t, int i,
+                                                  const CoefBus& bi, double& a, double& cc) {
+    const int j = g.yj[t];
+    const CoefBus bj = coef_bus(g, s, c, j);
+    const double Gij = g.G[t], Bij = g.B[t];
+    const double alpha = Gij * (bi.mu + bj.mu) - Bij * (bi.nu + bj.nu);
+    const double beta = Bij * (bi.mu - bj.mu) + Gij * (bi.nu - bj.nu);
+    double sn, cs;
+    sincos(s.va[i] - s.va[j], &sn, &cs);
+    const double K = alpha * cs + beta * sn;
+    const double M = -alpha * sn + beta * cs;
+    a = bj.v * M;
+    cc = -bi.v * bj.v * K;
+    return make_double4_32a(K, -a, bi.v * M, -cc);
+}
+__device__ __forceinline__ void coef_finish(const PfGrid& g, const CoefData& c, int i, const CoefBus& bi, double sa,
+                                            double sc) {
+    c.d2[i] = 2.0 * (bi.mu * g.G[g.ydiag[i]] - bi.nu * g.B[g.ydiag[i]]);
+    c.asum[i] = sa;
+    c.csum[i] = sc;
+    c.pg_curv[i] = g.ip_pg[i] >= 0 ? 2.0 * g.c2[i] * g.base_mva * g.base_mva : 0.0;
+}
+// one thread per bus (a network with a bus of more than 32 entries)
+__device__ __forceinline__ void coef_by_bus(const PfGrid& g, const PfState& s, const CoefData& c, int i) {
     if (i >= g.n_bus) return;
-    double cref = *crefp;
-    double mu_i = g.qth[i] >= 0 ? lam[g.qth[i]] : cref;
-    double nu_i = g.qv[i] >= 0 ? lam[g.qv[i]] : 0.0;
-    double vi = s.vm[i];
-    d2[i] = 2.0 * (mu_i * g.G[g.ydiag[i]] - nu_i * g.B[g.ydiag[i]]);
+    const CoefBus bi = coef_bus(g, s, c, i);
     double sa = 0.0, sc = 0.0;
-    int e = inc_ptr[i];
+    int e = c.inc_ptr[i];
     for (int t = g.yp[i]; t < g.yp[i + 1]; t++) {
-        int j = g.yj[t];
-        if (j == i) continue;
-        double mu_j = g.qth[j] >= 0 ? lam[g.qth[j]] : cref;
-        double nu_j = g.qv[j] >= 0 ? lam[g.qv[j]] : 0.0;
-        double Gij = g.G[t], Bij = g.B[t];
-        double alpha = Gij * (mu_i + mu_j) - Bij * (nu_i + nu_j);
-        double beta = Bij * (mu_i - mu_j) + Gij * (nu_i - nu_j);
-        double sn, cs;
-        sincos(s.va[i] - s.va[j], &sn, &cs);
-        double K = alpha * cs + beta * sn;
-        double M = -alpha * sn + beta * cs;
-        double vj = s.vm[j];
-        double a = vj * M, bb = vi * M, c = -vi * vj * K;
-        coef[e] = make_double4_32a(K, -a, bb, -c);
+        if (g.yj[t] == i) continue;
+        double a, cc;
+        c.coef[e++] = coef_entry(g, s, c, t, i, bi, a, cc);
         sa += a;
-        sc += c;
-        e++;
+        sc += cc;
     }
-    asum[i] = sa;
-    csum[i] = sc;
-    pg_curv[i] = g.ip_pg[i] >= 0 ? 2.0 * g.c2[i] * g.base_mva * g.base_mva : 0.0;
+    coef_finish(g, c, i, bi, sa, sc);
+}
+// One admittance entry per lane, on the warps of k_pf_eval_warp: a sincos is a long chain
+// of dependent FP64 instructions, and a thread per bus runs one after the other.  The
+// lane of each bus adds its row's terms in row order.
+__device__ __forceinline__ void coef_by_warp(const PfGrid& g, const PfState& s, const CoefData& c, int w) {
+    __shared__ double sh[kCoefThreads / 32][64];
+    if (w >= g.n_pfw) return;                                   // warp-uniform
+    const int lane = threadIdx.x & 31;
+    double* sw = sh[threadIdx.x >> 5];
+    const int b0 = g.pf_wb[w], b1 = g.pf_wb[w + 1], e0 = g.yp[b0], t = e0 + lane;
+    double a = 0.0, cc = 0.0;
+    if (t < g.yp[b1]) {
+        const int i = g.yrow[t], td = g.ydiag[i];
+        if (t != td)
+            c.coef[c.inc_ptr[i] + (t - g.yp[i]) - (t > td)] = coef_entry(g, s, c, t, i, coef_bus(g, s, c, i), a, cc);
+    }
+    sw[lane] = a;
+    sw[32 + lane] = cc;
+    __syncwarp();
+    const int i = b0 + lane;
+    if (i < b1) {
+        double sa = 0.0, sc = 0.0;
+        for (int tt = g.yp[i]; tt < g.yp[i + 1]; tt++) {        // the diagonal's terms are zero
+            sa += sw[tt - e0];
+            sc += sw[32 + tt - e0];
+        }
+        coef_finish(g, c, i, coef_bus(g, s, c, i), sa, sc);
+    }
 }
 
 // grad F = grad_p f + J_p^T lambda, one thread per bus (its v and Pg entries).
-__global__ void k_gradient(PfGrid g, PfState s, const int* jpt_ptr, const int* jpt_row, const double* jptv,
-                           const double* lam, const double* crefp, const double* gref_v, double* grad) {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
+__device__ __forceinline__ void gradient_bus(const PfGrid& g, const PfState& s, const CoefData& c, int i) {
     if (i >= g.n_bus) return;
-    double cref = *crefp;
-    int kv = g.ip_v[i];
+    const int kv = g.ip_v[i];
     if (kv >= 0) {
-        double h = cref * gref_v[i];
-        for (int t = jpt_ptr[kv]; t < jpt_ptr[kv + 1]; t++) h = fma(jptv[t], lam[jpt_row[t]], h);
-        grad[kv] = h;
+        double h = *c.cref * c.gref_v[i];
+        for (int t = c.jpt_ptr[kv]; t < c.jpt_ptr[kv + 1]; t++) h = fma(c.jptv[t], c.lam[c.jpt_row[t]], h);
+        c.grad[kv] = h;
     }
-    int kp = g.ip_pg[i];
+    const int kp = g.ip_pg[i];
     if (kp >= 0) {
-        double S = g.base_mva;
+        const double S = g.base_mva;
         double h = 2.0 * g.c2[i] * S * S * s.pg[i] + g.c1[i] * S;
-        for (int t = jpt_ptr[kp]; t < jpt_ptr[kp + 1]; t++) h = fma(jptv[t], lam[jpt_row[t]], h);
-        grad[kp] = h;
+        for (int t = c.jpt_ptr[kp]; t < c.jpt_ptr[kp + 1]; t++) h = fma(c.jptv[t], c.lam[c.jpt_row[t]], h);
+        c.grad[kp] = h;
     }
+}
+
+// What follows from lambda: the projection's coefficients (the first n_coef blocks) and
+// grad F (the others); as two kernels with a thread per bus 33 + 11 us at 9241 buses.
+__global__ void __launch_bounds__(kCoefThreads) k_adjoint_coef(PfGrid g, PfState s, CoefData c, int n_coef) {
+    if ((int)blockIdx.x >= n_coef) gradient_bus(g, s, c, ((int)blockIdx.x - n_coef) * kCoefThreads + (int)threadIdx.x);
+    else if (g.n_pfw > 0) coef_by_warp(g, s, c, (int)(blockIdx.x * (kCoefThreads / 32) + (threadIdx.x >> 5)));
+    else coef_by_bus(g, s, c, (int)(blockIdx.x * kCoefThreads + threadIdx.x));
 }
 
 // external column-major <-> internal row-major with a row map
@@ -2195,7 +2247,7 @@ __global__ void k_line_values_batch(const __grid_constant__ Solve1Batch B) {
 template <int NT>
 __global__ void __launch_bounds__(NT, kLineRegs / NT)
     k_solve1_batch(const __grid_constant__ Solve1Batch B, int use_tail) {
-    k_solve1_body<NT>(B.g[blockIdx.x], B.x[blockIdx.x], false, use_tail);
+    k_solve1_body<NT>(B.g[blockIdx.x], B.x[blockIdx.x], B.x[blockIdx.x], false, use_tail);
 }
 
 }  // namespace
@@ -2434,8 +2486,7 @@ void launch_line_values(const LineGrid& g, bool transposed_too, cudaStream_t st)
 }
 
 void launch_adjoint_rhs(const PfGrid& g, const PfState& s, const AdjData& a, cudaStream_t st) {
-    k_adjoint_rhs<<<1, 32, 0, st>>>(g, s, a);
-    k_objective<<<1, 256, 0, st>>>(g, s, a.F);
+    k_adjoint_rhs<<<2, kAdjThreads, 0, st>>>(g, s, a);
 }
 
 // Small grids take CTAs of 256 threads: their levels do not fill more warps, and idle
@@ -2459,31 +2510,20 @@ cudaError_t launch_dir1(const DirGrid& g, const LineGrid& s, const DirLaunch& L,
     return cudaGetLastError();
 }
 
-cudaError_t launch_solve1(const LineGrid& g, double* x, bool trans, bool use_tail, cudaStream_t st) {
+cudaError_t launch_solve1(const LineGrid& g, const double* x, double* out, bool trans, bool use_tail,
+                          cudaStream_t st) {
     const size_t smem = solve1_smem(g.n_x, g.T, use_tail);
-    if (line_threads(g.n_x) == 256) k_solve1<256><<<1, 256, smem, st>>>(g, x, trans, use_tail ? 1 : 0);
-    else k_solve1<512><<<1, 512, smem, st>>>(g, x, trans, use_tail ? 1 : 0);
+    if (line_threads(g.n_x) == 256) k_solve1<256><<<1, 256, smem, st>>>(g, x, out, trans, use_tail ? 1 : 0);
+    else k_solve1<512><<<1, 512, smem, st>>>(g, x, out, trans, use_tail ? 1 : 0);
     return cudaGetLastError();
 }
 
 int dirs_cta_slots() { return kDirCtasPerSm * num_sms(); }
 int dirs_batch_slots(int threads) { return dirs_batch_ctas_per_sm(threads) * num_sms(); }
 
-void launch_adjoint_coef(const PfGrid& g, const PfState& s, const double* lambda_int, const double* cref,
-                         const int* inc_ptr, const int* inc_nb, double4_32a* inc_coef, double* d2, double* asum,
-                         double* csum, double* pg_curv, cudaStream_t st) {
-    if (g.n_bus > 0)
-        k_adjoint_coef<<<blocks_for(g.n_bus, 128), 128, 0, st>>>(g, s, lambda_int, cref, inc_ptr, inc_nb, inc_coef,
-                                                                 d2, asum, csum, pg_curv);
-}
-
-void launch_gradient(const PfGrid& g, const PfState& s, int n_p, const int* jpt_ptr, const int* jpt_row,
-                     const double* jptv, const double* lambda_int, const double* cref, const double* gref_v,
-                     double* grad, cudaStream_t st) {
-    (void)n_p;
-    if (g.n_bus > 0)
-        k_gradient<<<blocks_for(g.n_bus, 128), 128, 0, st>>>(g, s, jpt_ptr, jpt_row, jptv, lambda_int, cref, gref_v,
-                                                             grad);
+void launch_adjoint_coef(const PfGrid& g, const PfState& s, const CoefData& c, cudaStream_t st) {
+    const int n_coef = g.n_pfw > 0 ? blocks_for(g.n_pfw, kCoefThreads / 32) : blocks_for(g.n_bus, kCoefThreads);
+    k_adjoint_coef<<<n_coef + blocks_for(g.n_bus, kCoefThreads), kCoefThreads, 0, st>>>(g, s, c, n_coef);
 }
 
 void launch_scatter_rows(int n_rows, int N, const int* map, const double* src, int64_t lds, double* dst,

@@ -332,7 +332,8 @@ struct LineGrid {
 };
 void launch_line_values(const LineGrid& g, bool transposed_too, cudaStream_t st);
 int line_threads(int n_x);
-cudaError_t launch_solve1(const LineGrid& g, double* x, bool trans, bool use_tail, cudaStream_t st);
+cudaError_t launch_solve1(const LineGrid& g, const double* x, double* out, bool trans, bool use_tail,
+                          cudaStream_t st);          // out may be x
 // Directions of a launch with one direction per CTA and x in shared memory (L.N CTAs;
 // direction c's rows at V + c * (zero_row + 1) and T likewise): SpMul to the U sweep, the
 // projection to SpMulAdd, or both.  Needs solve1_mode() > 0 and its schedule.
@@ -402,7 +403,8 @@ int dirs_cta_slots();
 
 // adjoint helpers
 struct AdjData {
-    double *rhs;          // n_x, internal order (output: -grad_x f)
+    double *rhs;          // n_rhs >= n_x, internal order (output: -grad_x f, zero beyond)
+    int n_rhs;
     double *cref, *c2ref; // device scalars c'_slack, c''_slack
     double *F;            // device scalar
     double *gref_th, *gref_v;   // per bus
@@ -412,12 +414,17 @@ struct AdjData {
     const int *uth, *uv;  // combined rows per bus
 };
 void launch_adjoint_rhs(const PfGrid& g, const PfState& s, const AdjData& a, cudaStream_t st);
-void launch_adjoint_coef(const PfGrid& g, const PfState& s, const double* lambda_int, const double* cref,
-                         const int* inc_ptr, const int* inc_nb, double4_32a* inc_coef, double* d2, double* asum,
-                         double* csum, double* pg_curv, cudaStream_t st);
-void launch_gradient(const PfGrid& g, const PfState& s, int n_p, const int* jpt_ptr, const int* jpt_row,
-                     const double* jptv, const double* lambda_int, const double* cref, const double* gref_v,
-                     double* grad, cudaStream_t st);
+// Once lambda is there: the projection's coefficients and grad F
+struct CoefData {
+    const double *lam, *cref, *gref_v;
+    const int* inc_ptr;
+    double4_32a* coef;          // per incidence
+    double *d2, *asum, *csum, *pg_curv;
+    const int *jpt_ptr, *jpt_row;
+    const double* jptv;
+    double* grad;
+};
+void launch_adjoint_coef(const PfGrid& g, const PfState& s, const CoefData& c, cudaStream_t st);
 
 // permutation helpers between external (x, p) order and the internal rows
 void launch_gather_rows(int n_rows, int N, const int* map, const double* src, int64_t lds, double* dst,
