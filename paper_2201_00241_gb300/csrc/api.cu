@@ -269,6 +269,7 @@ struct rh_grid {
         g.n_pe = (int64_t)S.rf_pe_bus.size(); g.pe_bus = rf_pe_bus; g.pe_pos = reinterpret_cast<const int4*>(rf_pe_pos);
         g.A = A; g.invdiag = invdiag; g.jmax = umax + 1; g.err = err;
         g.tailD = tailD; g.tail_pos = tail_pos;
+        g.triLd = triLd; g.triUd = triUd; g.triUtd = triUtd; g.triLtd = triLtd;
         return g;
     }
     int rows() const { return S.n_x + S.n_p + 1; }

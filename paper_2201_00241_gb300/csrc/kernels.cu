@@ -418,8 +418,7 @@ __global__ void __launch_bounds__(128) k_jac_ad(PfGrid g, PfState s, const int* 
 // for every later variable j of the bus's pattern (a PV bus has theta only), with
 // 1/u_tt, l_vt, 1/u_vv, u_tv from the bus's pivot job.  Thread x < n_piv does bus
 // x's block, the others one entry j each (positions a_tj, a_vj, a_jt, a_jv).
-__device__ __forceinline__ void k_rf_pivot_body(const RfGrid& g) {
-    const int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+__device__ __forceinline__ void k_rf_pivot_body(const RfGrid& g, int64_t x) {
     const int64_t e = x - g.n_piv;
     int k = 0, qt = 0, dt = 0, n_rows = 0;
     int4 p = make_int4(-1, -1, -1, -1);             // a_tj, a_vj, a_jt, a_jv
@@ -462,7 +461,7 @@ __device__ __forceinline__ void k_rf_pivot_body(const RfGrid& g) {
     }
 }
 __global__ void k_rf_pivot(RfGrid g) {
-    k_rf_pivot_body(g);
+    k_rf_pivot_body(g, (int64_t)blockIdx.x * blockDim.x + threadIdx.x);
 }
 
 // Pivot quantities of a bus from its block [a_tt a_tv; a_vt a_vv]: 1/u_tt,
@@ -638,6 +637,21 @@ __global__ void k_rf_update(RfGrid g, int64_t t0, int64_t nt, int j0, int njob) 
 // 1 / u_cc = s_c / a_cc, with one division per column for 1 / a_cc.
 constexpr int kTailTB = 16;
 
+// Entry (i, j) of the dense tail's triangles of the unit-diagonal factors L'', U' and of
+// their transposes, from a_ij, a_ji, the smaller index's diagonal and both inverse diagonals.
+__device__ __forceinline__ void tail_tri(double* triLd, double* triUd, double* triUtd, double* triLtd, int T, int i,
+                                         int j, double aij, double aji, double amin, double ii, double ij) {
+    if (i > j) {
+        const int o = j * (T - 1) - j * (j - 1) / 2 + (i - j - 1);
+        triLd[o] = aij * amin * ii;                   // L''_ij
+        triUtd[o] = aji * ij;                         // (U'^T)_ij = U'_ji
+    } else if (i < j) {
+        const int o = j * (j - 1) / 2 + i;
+        triUd[o] = aij * ii;                          // U'_ij
+        triLtd[o] = aji * amin * ij;                  // (L''^T)_ij = L''_ji
+    }
+}
+
 __device__ __forceinline__ void k_tail_gather_body(RfGrid g) {
     const int T = g.T;
     const int idx = blockIdx.x * blockDim.x + threadIdx.x;
@@ -662,10 +676,12 @@ __device__ __forceinline__ void tail_shell_entry(int p, int& r, int& c) {
     c = o == 0 ? m : (o <= q ? m + o : m);
 }
 
-// Eliminates the tile in Dk (unit-padded beyond kb) without divisions:
-// afterwards Dk[r][c] = s_{min(r,c)} a_rc (a the ordinary elimination's values
-// when the entry is final), S[c] = s_c and Rd[c] = 1 / Dk[c][c].
-__device__ __forceinline__ void tail_factor(double (*Dk)[kTailTB + 1], int kb, double* S, double* Rd) {
+// Eliminates the tile at D (leading dimension ld, unit-padded beyond kb) without
+// divisions: afterwards D[r][c] = s_{min(r,c)} a_rc (a the ordinary elimination's values
+// when the entry is final), S[c] = s_c and Rd[c] = 1 / D[c][c].  Run by the CTA's first
+// 256 threads, which meet at named barrier 1.
+__device__ __forceinline__ void tail_sync() { asm volatile("bar.sync 1, 256;" ::: "memory"); }
+__device__ __forceinline__ void tail_factor(double* D, int ld, int kb, double* S, double* Rd) {
     constexpr int TB = kTailTB;
     const int t = threadIdx.x;
     int er = 0, ec = 0;
@@ -673,28 +689,28 @@ __device__ __forceinline__ void tail_factor(double (*Dk)[kTailTB + 1], int kb, d
     double s = 1.0;
     for (int j = 0; j < kb - 1; j++) {
         const int na = (TB - 1 - j) * (TB - 1 - j);
-        const double d = Dk[j][j];
+        const double d = D[j * ld + j];
         const int sh = pivot_shift(d);
         if (t < na) {
-            const double prod = Dk[er][j] * Dk[j][ec];
-            Dk[er][ec] = scale_pow2(fma(d, Dk[er][ec], -prod), sh);
+            const double prod = D[er * ld + j] * D[j * ld + ec];
+            D[er * ld + ec] = scale_pow2(fma(d, D[er * ld + ec], -prod), sh);
         }
-        if (t == (int)blockDim.x - 1) {
+        if (t == 255) {
             s *= scale_pow2(d, sh);
             S[j + 1] = s;
         }
-        __syncthreads();
+        tail_sync();
     }
     if (t < TB) {
         if (t < kb) {
             if (t == 0) S[0] = 1.0;
-            Rd[t] = 1.0 / Dk[t][t];
+            Rd[t] = 1.0 / D[t * ld + t];
         } else {
             S[t] = 0.0;
             Rd[t] = 0.0;
         }
     }
-    __syncthreads();
+    tail_sync();
 }
 
 // Loads a TB x TB tile of the row-major T x T scratch at (i0, j0), rb x cb live.
@@ -762,7 +778,7 @@ __device__ __forceinline__ void k_tail_step_body(RfGrid g, int k) {
                 acc = ltile ? fma(Xk[r][q], Uk[q][cc], acc) : fma(Lk[r][q], Xk[q][cc], acc);
             X[r][cc] -= acc;
         }
-        tail_factor(Dk, kb, S, Rd);   // begins by reading only Dk; its barriers cover X
+        tail_factor(&Dk[0][0], TB + 1, kb, S, Rd);   // begins by reading only Dk; its barriers cover X
         // multipliers in place: u_jc / u_jj = Dk[j][c] Rd[j] above the diagonal,
         // l_rj = Dk[r][j] Rd[j] below it
         {
@@ -806,7 +822,7 @@ __device__ __forceinline__ void k_tail_step_body(RfGrid g, int k) {
         // U (r <= c: Dk / s_r) and L (r > c: Dk / Dk[c][c])
         const int kb = min(TB, T - k0);
         tail_diag_tile(g, k0, kb, k >= 1 ? k0 - TB : -1, Dk, Lk, Uk);
-        tail_factor(Dk, kb, S, Rd);
+        tail_factor(&Dk[0][0], TB + 1, kb, S, Rd);
         const int r = t / TB, cl = t % TB;
         if (t < TB) Xk[0][t] = t < kb ? 1.0 / S[t] : 0.0;
         __syncthreads();
@@ -853,6 +869,100 @@ __global__ void k_tail_scatter(RfGrid g) {
     pdl_wait();
     k_tail_scatter_body(g);
 }
+
+// The whole dense tail of T <= kTailOne in one CTA, beside the pivot steps (which touch no
+// entry of it): LU in shared memory over the same tiles, then the factor, its inverse
+// diagonal and the sweeps' triangles.  Such a tail has 2-4 tiles: launched tile by tile it is
+// mostly launches, loads and one diagonal tile factored in every CTA, where one SM needs
+// few FP64 cycles for all of it (T^3 / 3 multiply-adds at 2 a cycle).  A refactorisation's
+// launches after the last level, 5 + ceil(T / 16) of them and k_build_tail, are one: the
+// reduced Hessian at 118 buses (T = 16) 185 -> 175 us, eight re-solves at 1354 buses (T = 48)
+// 1124 -> 1092 us.  T = 80 would need 95 k cycles of the SM's FP64 pipes (T = 48: 38 k), more
+// than the launches it saves.
+constexpr int kTailThreads = 512;
+struct TailOne {
+    double M[kTailOne][kTailOne + 1];
+    double Mk[kTailTB][kTailTB + 1];   // multipliers of the current diagonal tile
+    double S[kTailTB], Rd[kTailTB], inv[kTailOne];
+};
+__device__ __forceinline__ void tail_one(const RfGrid& g, TailOne& s) {
+    constexpr int TB = kTailTB, LD = kTailOne + 1, Q = kTailOne * kTailOne / kTailThreads;
+    const int T = g.T, nt = (T + TB - 1) / TB, Tp = nt * TB, t = threadIdx.x;
+    int pos[Q];
+#pragma unroll
+    for (int q = 0; q < Q; q++) {
+        const int e = t + q * kTailThreads, i = e / Tp, j = e - i * Tp;
+        pos[q] = e < Tp * Tp && i < T && j < T ? g.tail_pos[i * T + j] : -1;
+        if (pos[q] >= 0 && !inb(pos[q], g.nnz)) pos[q] = -1;
+    }
+    pdl_wait();
+    pdl_trigger();
+#pragma unroll
+    for (int q = 0; q < Q; q++) {
+        const int e = t + q * kTailThreads, i = e / Tp, j = e - i * Tp;
+        if (e < Tp * Tp) s.M[i][j] = pos[q] >= 0 ? g.A[pos[q]] : (i == j && i >= T ? 1.0 : 0.0);
+    }
+    __syncthreads();
+    for (int k0 = 0; k0 < Tp; k0 += TB) {
+        const int kb = min(TB, T - k0), R = Tp - k0 - TB;
+        if (t < 256) {
+            tail_factor(&s.M[k0][k0], LD, kb, s.S, s.Rd);
+            // l_rc = D[r][c] / D[c][c] (the multiplier too), u_rc = D[r][c] / s_r with u_rc / u_rr the multiplier
+            const int r = t / TB, c = t % TB;
+            const double v = s.M[k0 + r][k0 + c], m = v * s.Rd[min(r, c)];
+            if (r != c) s.Mk[r][c] = m;
+            s.M[k0 + r][k0 + c] = r > c ? m : (r < kb ? v * (1.0 / s.S[r]) : v);
+        }
+        __syncthreads();
+        // panels, TB lanes to a row below (X U_kk = A_ik) or a column to the right (L_kk Y = A_kj)
+        for (int h = t / TB; h < 2 * R; h += kTailThreads / TB) {
+            const bool low = h < R;                       // the same for the warp
+            const int o = k0 + TB + (low ? h : h - R), l = t % TB;
+            double* at = low ? &s.M[o][k0 + l] : &s.M[k0 + l][o];
+            double x = *at;
+#pragma unroll
+            for (int j = 0; j < TB - 1; j++) {
+                const double xj = __shfl_sync(0xffffffffu, x, j, TB);
+                if (l > j) x = fma(-xj, low ? s.Mk[j][l] : s.Mk[l][j], x);
+            }
+            *at = low ? x * (s.S[l] * s.Rd[l]) : x;
+        }
+        __syncthreads();
+        for (int e = t; e < R * R; e += kTailThreads) {
+            const int i = k0 + TB + e / R, j = k0 + TB + e % R;
+            double acc = 0.0;
+#pragma unroll
+            for (int q = 0; q < TB; q++) acc = fma(s.M[i][k0 + q], s.M[k0 + q][j], acc);
+            s.M[i][j] -= acc;
+        }
+        __syncthreads();
+    }
+    if (t < T) {
+        const double v = s.M[t][t], tau = 1e-14 * __longlong_as_double((long long)*g.jmax), r = 1.0 / v;
+        s.inv[t] = r;
+        g.invdiag[g.t0 + t] = r;
+        if (!(fabs(v) > tau)) atomicOr(g.err, 1);
+    }
+#pragma unroll
+    for (int q = 0; q < Q; q++) {
+        const int e = t + q * kTailThreads, i = e / Tp, j = e - i * Tp;
+        if (e >= Tp * Tp || i >= T || j >= T) continue;
+        if (pos[q] >= 0) g.A[pos[q]] = s.M[i][j];
+        else s.M[i][j] = 0.0;                             // structurally zero
+    }
+    __syncthreads();
+    for (int e = t; e < T * T; e += kTailThreads) {
+        const int i = e / T, j = e - i * T;
+        tail_tri(g.triLd, g.triUd, g.triUtd, g.triLtd, T, i, j, s.M[i][j], s.M[j][i], s.M[i > j ? j : i][i > j ? j : i],
+                 s.inv[i], s.inv[j]);
+    }
+}
+__device__ __forceinline__ void rf_finish_body(const RfGrid& g) {
+    __shared__ TailOne tail;
+    if (blockIdx.x == 0) tail_one(g, tail);
+    else k_rf_pivot_body(g, (int64_t)(blockIdx.x - 1) * kTailThreads + threadIdx.x);
+}
+__global__ void __launch_bounds__(kTailThreads) k_rf_finish(RfGrid g) { rf_finish_body(g); }
 
 // Transposed copies of the factor values and of J_p, and the unit-diagonal
 // factors of the direction kernel.  With D = diag(U), J_x = L U = D L'' U' where
@@ -906,17 +1016,8 @@ __global__ void k_build_tail(int T, int t0, const int* __restrict__ pos, const d
     int i = idx / T, j = idx - i * T;
     if (i == j) return;
     int pij = pos[idx], pji = pos[j * T + i];
-    double aij = pij >= 0 ? A[pij] : 0.0, aji = pji >= 0 ? A[pji] : 0.0;
-    const double ii = invdiag[t0 + i], ij = invdiag[t0 + j];
-    if (i > j) {
-        int o = j * (T - 1) - j * (j - 1) / 2 + (i - j - 1);
-        triLd[o] = aij * A[pos[j * T + j]] * ii;    // L''_ij
-        triUtd[o] = aji * ij;                       // (U'^T)_ij = U'_ji
-    } else {
-        int o = j * (j - 1) / 2 + i;
-        triUd[o] = aij * ii;                        // U'_ij
-        triLtd[o] = aji * A[pos[i * T + i]] * ij;   // (L''^T)_ij = L''_ji
-    }
+    tail_tri(triLd, triUd, triUtd, triLtd, T, i, j, pij >= 0 ? A[pij] : 0.0, pji >= 0 ? A[pji] : 0.0,
+             A[pos[i > j ? j * T + j : i * T + i]], invdiag[t0 + i], invdiag[t0 + j]);
 }
 
 // ---------------------------------------------------------------------------
@@ -2212,8 +2313,9 @@ __global__ void k_rf_leaf_piv_batch(RfBatch B, int njob) {
     k_rf_leaf_piv_body(B.g[blockIdx.y], njob);
 }
 __global__ void k_rf_pivot_batch(RfBatch B) {
-    k_rf_pivot_body(B.g[blockIdx.y]);
+    k_rf_pivot_body(B.g[blockIdx.y], (int64_t)blockIdx.x * blockDim.x + threadIdx.x);
 }
+__global__ void __launch_bounds__(kTailThreads) k_rf_finish_batch(RfBatch B) { rf_finish_body(B.g[blockIdx.y]); }
 __global__ void k_tail_gather_batch(RfBatch B) {
     k_tail_gather_body(B.g[blockIdx.y]);
 }
@@ -2339,6 +2441,11 @@ cudaError_t launch_refactor(const RfGrid& g, const int* lev_ptr_host, const int6
         const int64_t t0 = tgt_lev_ptr_host[lev], nt = tgt_lev_ptr_host[lev + 1] - t0;
         const int j0 = piv_lev_ptr_host[lev], njob = piv_lev_ptr_host[lev + 1] - j0;
         if (nt > 0) chk(launch_pdl(pdl, k_rf_update, dim3(blocks_for(nt, 256)), dim3(256), 0, st, g, t0, nt, j0, njob));
+    }
+    if (tail_in_one(g.T)) {
+        chk(launch_pdl(pdl, k_rf_finish, dim3(1 + blocks_for((int64_t)g.n_piv + g.n_pe, kTailThreads)),
+                       dim3(kTailThreads), 0, st, g));
+        return e != cudaSuccess ? e : cudaGetLastError();
     }
     if (g.n_piv + g.n_pe > 0)
         chk(launch_pdl(pdl, k_rf_pivot, dim3(blocks_for((int64_t)g.n_piv + g.n_pe, 256)), dim3(256), 0, st, g));
@@ -2475,7 +2582,7 @@ void launch_scale_rows(int n, int N, const double* s, double* x, int64_t ld, cud
 
 void launch_build_tail(int T, int t0, const int* pos, const double* A, const double* invdiag, double* triLd,
                        double* triUd, double* triUtd, double* triLtd, cudaStream_t st) {
-    if (T > 1)
+    if (T > 1 && !tail_in_one(T))
         k_build_tail<<<blocks_for((int64_t)T * T, 256), 256, 0, st>>>(T, t0, pos, A, invdiag, triLd, triUd, triUtd,
                                                                       triLtd);
 }
@@ -2571,6 +2678,11 @@ cudaError_t launch_refactor_batch(const RfBatch& B, const int* lev_ptr_host, con
                            njob));
     }
     const int64_t np = (int64_t)B.g[0].n_piv + B.g[0].n_pe;
+    if (tail_in_one(B.g[0].T)) {
+        chk(launch_pdl(pdl, k_rf_finish_batch, dim3((unsigned)(1 + blocks_for(np, kTailThreads)), n), dim3(kTailThreads),
+                       0, st, B));
+        return e != cudaSuccess ? e : cudaGetLastError();
+    }
     if (np > 0) chk(launch_pdl(pdl, k_rf_pivot_batch, dim3((unsigned)blocks_for(np, 256), n), dim3(256), 0, st, B));
     const int T = B.g[0].T;
     if (T > 0) {
@@ -2588,7 +2700,7 @@ cudaError_t launch_refactor_batch(const RfBatch& B, const int* lev_ptr_host, con
 }
 
 void launch_tail_tri_batch(const TriBatch& B, cudaStream_t st) {
-    if (B.n > 0 && B.T > 1)
+    if (B.n > 0 && B.T > 1 && !tail_in_one(B.T))
         k_tail_tri_batch<<<dim3((unsigned)blocks_for((int64_t)B.T * B.T, 256), (unsigned)B.n), 256, 0, st>>>(B);
 }
 

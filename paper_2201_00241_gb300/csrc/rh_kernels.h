@@ -267,9 +267,14 @@ struct RfGrid {
     const int *pe_bus;
     const int4 *pe_pos;
     double *A, *invdiag;
+    double *triLd, *triUd, *triUtd, *triLtd;   // the tail's triangles, written with it when tail_in_one(T)
     const unsigned long long *jmax;
     int *err;
 };
+// Whether launch_refactor factors the dense tail in one CTA and writes its triangles too
+// (launch_build_tail and launch_tail_tri_batch then do nothing).
+constexpr int kTailOne = 64;
+inline bool tail_in_one(int T) { return T > 0 && T <= kTailOne; }
 // L2 prefetch of up to 8 read-only device arrays (16-byte aligned; the bytes of
 // each are rounded down to a multiple of 16); `first` is filled by the launcher.
 struct PrefetchList {
