@@ -225,8 +225,9 @@ rh_status rh_hessvec(rh_grid *grid, const double *W, int64_t ldw, int32_t N,
  * requests on grids of different sizes, computed by ONE kernel launch on
  * `stream` (asynchronous).  Items are independent; item i gets
  * ceil(N_i / width) CTAs (width = target directions per CTA, the right-hand-
- * side interleave width; 0 spreads the items so that they end together).  Up to 32
- * items per launch; larger batches take several launches.
+ * side interleave width; 0 spreads the items so that they end together, which may
+ * put the items on the largest grids in a launch of their own beside the others').
+ * Up to 32 items per launch; larger batches take several launches.
  *   grid    adjoint-ready grid (rh_adjoint for its current state); all items
  *           must be on the same device
  *   W, HW   DEVICE pointers, n_p x N column-major (ldw, ldhw >= n_p of the grid)
@@ -263,6 +264,8 @@ rh_status rh_batch_hessvec(int32_t n_items, const rh_hv_item *items, int32_t wid
  *                items than threads / 2 splits each row's dot product over up
  *                to split_lanes adjacent lanes (a power of two, 1 = no split, at
  *                most 32); 0 takes 32.
+ * With all three 0 the items on the largest grids may run one direction per CTA
+ * (512 threads, an SM each) beside the others.
  * RH_EINVAL for any other value (checked before anything else, also when
  * n_items is 0).  Every configuration computes each item's HW up to rounding.
  * rh_batch_hessvec(n, items, width, stream) is this call with {width, 0, 0}.

@@ -4,8 +4,8 @@ N directions, section 5.3).
 A batched launch (rh_batch_hessvec_cfg) has four choices that trade against one
 another and depend on the grids and the batch:
 
-* width: directions per CTA (the right-hand-side interleave width; 0 spreads each
-  item over the CTA slots).  Narrow widths spread a batch over more SMs, wide ones
+* width: directions per CTA (the right-hand-side interleave width; 0 spreads the
+  items so that they end together).  Narrow widths spread a batch over more SMs, wide ones
   amortise each CTA's per-level barrier over more directions.
 * threads: the CTA shape, one of the compiled 128 x 6, 192 x 4, 256 x 3 and
   384 x 2 (threads x resident CTAs per SM).  Small CTAs give an SM more

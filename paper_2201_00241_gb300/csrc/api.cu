@@ -792,51 +792,108 @@ __global__ void k_rto_apply(int n_p, int n_bus, const int* info, const double* p
 
 int nblk(int n, int t) { return (n + t - 1) / t; }
 
-// CTAs of each item of a batched launch whose width is left to the library.  A CTA with D
-// directions of a grid takes about
-//   t(D) = kLevelUs x (levels of the four sweeps) + kFlopUs x (flops of a direction) x D,
-// with the SM's CTA slots occupied (fitted on GB300: the 9241-bus grid takes 2.0 ms at
-// D = 1 and 5.6 ms at D = 10, the 1354-bus grid 0.40 ms at D = 4).  The items run side by
-// side, so the launch ends with its slowest CTA: the least T is taken for which every
-// item, at the most directions per CTA that end by T, gets all its CTAs into the slots at
-// once.  One CTA a direction instead, whatever the batch, puts a batch of many
-// directions through the slots in several waves of the latency-bound sweeps: a round of
-// 15 requests (118 to 9241 buses, 1920 directions) took 5.6 ms, 8 x 64 directions on the
-// 1354-bus grid 0.92 ms.
-void spread_batch(const rh_hv_item* items, int n, int slots, int* G) {
-    constexpr double kLevelUs = 4.5, kFlopUs = 0.27e-3;
+// CTAs of each item of a batched launch whose width is left to the library.  A CTA of the
+// batched direction kernel with D directions of a grid takes about
+//   t(D) = kLevelUs x (levels of the four sweeps) + (kRowUs + kFlopUs x D) x (flops of a direction),
+// with the SM's CTA slots occupied: a level's chain, the rows' loads, which the directions
+// share, and their arithmetic (fitted on GB300, D = 1 / 2 / 3: 2196 / 2526 / 3013 us on the
+// 9241-bus grid, 744 / 795 / 1001 on 2869 buses, 360 / 401 / 476 on 1354 buses, 119 / 122 /
+// 130 on 118 buses).  The items run side by side, so the launch ends with its slowest CTA:
+// the least T is taken for which every item, at the most directions per CTA that end by T,
+// gets all its CTAs into the slots at once.  One CTA a direction instead, whatever the
+// batch, puts a batch of many directions through the slots in several waves of the
+// latency-bound sweeps: a round of 15 requests (118 to 9241 buses, 1912 directions) took
+// 5.6 ms, 8 x 64 directions on the 1354-bus grid 0.92 ms.
+//
+// The items on the largest grids may run one direction per CTA with x in shared memory
+// instead (k_dir1_batch, an SM each, t(1) x kAlone), the others filling the SMs it leaves
+// and, once its last CTA has started, those that are done.  Their few directions are the
+// longest chains of a mixed batch: next to CTAs of many directions, which keep an SM's FP64
+// pipes busy, they end it.  Of the sets "the items on grids of at least n rows" the one with
+// the least predicted time is taken: the round of 15 requests takes 3.2 ms with none, 1.9
+// ms with the 9241-bus grid (184 directions), 2.3 with 2869 buses and more, 2.2 with 1354
+// buses and more; 8 x 64 directions on the 1354-bus grid take 488 us with none, 509 with all.
+struct BatchPlan {
+    int G[rh::kMaxBatch];                // CTAs (0: no directions, or one per CTA in k_dir1_batch)
+    bool alone[rh::kMaxBatch];
+};
+void plan_batch(const rh_hv_item* items, int n, int threads, bool may_alone, BatchPlan& P) {
+    constexpr double kLevelUs = 1.1, kRowUs = 0.78e-3, kFlopUs = 0.3e-3, kAlone = 0.36;
+    const int slots = rh::dirs_batch_slots(threads), per_sm = rh::dirs_batch_ctas_per_sm(threads), n_sm = slots / per_sm;
     std::vector<double> a(n), b(n);
     std::vector<int> cap(n);
-    double lo = 0.0, hi = 0.0;
     for (int k = 0; k < n; k++) {
         const auto& S = items[k].grid->S;
         const int T = S.n_x - S.t0;
         const double flops = 4.0 * (double)S.jp_col.size() + 4.0 * (S.nnz_l + S.nnz_u - S.n_x) +
                              8.0 * (double)S.yj.size();
-        a[k] = kLevelUs * (2.0 * S.n_flev + 2.0 * S.n_blev);
+        a[k] = kLevelUs * (2.0 * S.n_flev + 2.0 * S.n_blev) + kRowUs * flops;
         b[k] = kFlopUs * flops;
         // at most 256 directions, and the dense tail's rows in shared memory
         cap[k] = T > 1 ? std::max(1, rh::dirs_tail_cap() / T) : 256;
         cap[k] = std::min(std::min(cap[k], 256), std::max(1, items[k].N));
-        lo = std::max(lo, items[k].N > 0 ? a[k] + b[k] : 0.0);
-        hi = std::max(hi, a[k] + b[k] * cap[k]);
     }
-    auto ctas = [&](double t) {
-        int64_t sum = 0;
+    // the items outside `alone`: their time on `room` slots (0: none), and G
+    auto spread = [&](const bool* alone, int room, int* G) {
+        double lo = 0.0, hi = 0.0;
         for (int k = 0; k < n; k++) {
-            const int D = std::max(1, (int)std::min((double)cap[k], std::floor((t - a[k]) / b[k])));
-            // the fewest CTAs with at most D directions
-            G[k] = items[k].N > 0 ? (items[k].N + D - 1) / D : 0;
-            sum += G[k];
+            G[k] = 0;
+            if (alone[k] || items[k].N == 0) continue;
+            lo = std::max(lo, a[k] + b[k]);
+            hi = std::max(hi, a[k] + b[k] * cap[k]);
         }
-        return sum;
+        auto ctas = [&](double t) {
+            int64_t sum = 0;
+            for (int k = 0; k < n; k++) {
+                if (alone[k] || items[k].N == 0) continue;
+                const int D = std::max(1, (int)std::min((double)cap[k], std::floor((t - a[k]) / b[k])));
+                G[k] = (items[k].N + D - 1) / D;         // the fewest CTAs with at most D directions
+                sum += G[k];
+            }
+            return sum;
+        };
+        if (ctas(lo) <= room) return lo;
+        for (int it = 0; it < 40; it++) {
+            const double mid = 0.5 * (lo + hi);
+            (ctas(mid) <= room ? hi : lo) = mid;
+        }
+        // more CTAs than slots even at the caps: further waves
+        const int64_t all = ctas(hi);
+        return hi * (double)((all + room - 1) / room);
     };
-    if (ctas(lo) <= slots) return;
-    for (int it = 0; it < 40; it++) {
-        const double mid = 0.5 * (lo + hi);
-        (ctas(mid) <= slots ? hi : lo) = mid;
+    std::fill(P.alone, P.alone + n, false);
+    double best = spread(P.alone, slots, P.G);
+    if (!may_alone) return;
+    std::vector<int> order;
+    for (int k = 0; k < n; k++)
+        if (items[k].N > 0) order.push_back(k);
+    std::stable_sort(order.begin(), order.end(), [&](int p, int q) { return items[p].grid->S.n_x > items[q].grid->S.n_x; });
+    BatchPlan Q = P;
+    double sm_us = 0.0, longest = 0.0, shortest = 0.0;
+    int64_t dirs = 0;
+    for (size_t i = 0; i < order.size(); i++) {
+        const int k = order[i];
+        const auto& S = items[k].grid->S;
+        if (items[k].grid->n_line < 0 || rh::line_threads(S.n_x) != 512) break;
+        Q.alone[k] = true;
+        shortest = kAlone * (a[k] + b[k]);
+        longest = std::max(longest, shortest);
+        sm_us += shortest * items[k].N;
+        dirs += items[k].N;
+        if (i + 1 < order.size() && items[order[i + 1]].grid->S.n_x == S.n_x) continue;
+        // SMs that the last wave leaves, and when it starts
+        const int last = (int)((dirs - 1) % n_sm) + 1;
+        const double wave = sm_us / (double)dirs, start = wave * (double)((dirs - 1) / n_sm);
+        const bool rest = i + 1 < order.size();
+        const int room = per_sm * (n_sm - last);
+        double t = std::max(start + wave, longest);
+        if (rest) t = room > 0 ? std::max(t, start + spread(Q.alone, room, Q.G)) : t + spread(Q.alone, slots, Q.G);
+        if (t < best) {
+            best = t;
+            P = Q;
+        }
+        std::fill(Q.G, Q.G + n, 0);
     }
-    ctas(hi);
 }
 
 }  // namespace
@@ -1898,17 +1955,29 @@ rh_status rh_batch_hessvec_cfg(int32_t n_items, const rh_hv_item* items, const r
     std::unique_ptr<rh::DirBatch> B(new rh::DirBatch());
     for (int first = 0; first < n_items; first += rh::kMaxBatch) {
         int n = std::min(rh::kMaxBatch, n_items - first);
-        int spread[rh::kMaxBatch];
-        if (width == 0) spread_batch(items + first, n, rh::dirs_batch_slots(threads), spread);
+        BatchPlan P;
+        std::fill(P.alone, P.alone + n, false);
+        if (width == 0) plan_batch(items + first, n, threads, !cfg->threads && !cfg->split_lanes, P);
+        const bool alone = std::find(P.alone, P.alone + n, true) != P.alone + n;
         B->n_items = 0;
         B->cta_ptr[0] = 0;
-        for (int k = 0; k < n; k++) {
+        std::unique_ptr<rh::Dir1Batch> B1(alone ? new rh::Dir1Batch() : nullptr);
+        if (alone) {
+            B1->n_items = 0;
+            B1->cta_ptr[0] = 0;
+        }
+        // the longest chains first
+        std::vector<int> order(n);
+        for (int k = 0; k < n; k++) order[k] = k;
+        std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return items[first + a].grid->S.n_x > items[first + b].grid->S.n_x; });
+        for (int k : order) {
             const rh_hv_item& it = items[first + k];
             if (it.N == 0) continue;
             rh_grid* g = it.grid;
-            int G = width > 0 ? (it.N + width - 1) / width : spread[k];
+            const bool one = P.alone[k];
+            int G = one ? it.N : width > 0 ? (it.N + width - 1) / width : P.G[k];
             G = std::max(G, (it.N + 255) / 256);
-            rh::DirLaunch& L = B->l[B->n_items];
+            rh::DirLaunch& L = one ? B1->l[B1->n_items] : B->l[B->n_items];
             L.N = it.N;
             L.n_cta = G;
             L.ld = it.N;
@@ -1927,13 +1996,21 @@ rh_status rh_batch_hessvec_cfg(int32_t n_items, const rh_hv_item* items, const r
             int Tt = g->S.n_x - g->S.t0;
             L.use_tail = rh::dirs_tail_fits(Tt, it.N, G) ? 1 : 0;
             L.use_reach = 0;
+            if (one) {
+                L.use_tail = rh::solve1_mode(g->S.n_x, Tt) == 2 ? 1 : 0;
+                B1->g[B1->n_items] = g->dir();
+                B1->s[B1->n_items] = g->s1();
+                B1->cta_ptr[B1->n_items + 1] = B1->cta_ptr[B1->n_items] + G;
+                B1->n_items++;
+                continue;
+            }
             B->g[B->n_items] = g->dir();
             B->g[B->n_items].ks_cap = ks_cap;
             B->cta_ptr[B->n_items + 1] = B->cta_ptr[B->n_items] + G;
             B->n_items++;
         }
-        rh::launch_dirs_batch(*B, threads, (cudaStream_t)stream);
-        RH_CUDA(cudaGetLastError());
+        if (alone) RH_CUDA(rh::launch_dir1_batch(*B1, (cudaStream_t)stream));
+        RH_CUDA(rh::launch_dirs_batch(*B, threads, alone, (cudaStream_t)stream));
     }
     return RH_OK;
 }

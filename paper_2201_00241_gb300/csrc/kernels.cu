@@ -1763,6 +1763,7 @@ __global__ void __launch_bounds__(NT, MINB) k_dirs_batch(DirBatch B) {
     }
     __syncthreads();
     dirs_body(sg, sl, (int)blockIdx.x - B.cta_ptr[item], part, sref, nullptr);
+    pdl_wait();      // beside k_dir1_batch: what follows this launch follows both
 }
 
 // Sweeps of a right-hand side held in shared memory.  There is nothing to coalesce, so
@@ -1959,13 +1960,12 @@ __global__ void __launch_bounds__(NT, kLineRegs / NT)
 // 118 buses 108 -> 63 us, 45 at 2869 buses 513 -> 233, 256 at 9241 buses 2046 -> 1465.
 //   phases SPMUL L U (x is left in V), TPROJ UT LT MULADD (x from V), or all of them
 template <int NT>
-__global__ void __launch_bounds__(NT, kLineRegs / NT)
-    k_dir1(const __grid_constant__ DirGrid g, const __grid_constant__ LineGrid s, const __grid_constant__ DirLaunch L,
-           int use_tail) {
+__device__ __forceinline__ void dir1_body(const DirGrid& g, const LineGrid& s, const DirLaunch& L, const int c,
+                                          int use_tail) {
     extern __shared__ double X[];
     double* tri = X + g.n_x + 1;
     double* part = tri + (use_tail ? (size_t)s.T * (s.T - 1) / 2 : 0);
-    const int c = blockIdx.x, rows = g.zero_row + 1;
+    const int rows = g.zero_row + 1;
     if (L.ws_elems > 0 && !inb((int64_t)(c + 1) * rows - 1, L.ws_elems)) return;
     double* V = L.V + (int64_t)c * rows;
     double* Y = L.T + (int64_t)c * rows;
@@ -2079,6 +2079,22 @@ __global__ void __launch_bounds__(NT, kLineRegs / NT)
             if (inb(g.jpt_row[t], g.n_x)) h = fma(g.jptvd[t], X[g.jpt_row[t]], h);
         HW[k] = h;
     }
+}
+
+template <int NT>
+__global__ void __launch_bounds__(NT, kLineRegs / NT)
+    k_dir1(const __grid_constant__ DirGrid g, const __grid_constant__ LineGrid s, const __grid_constant__ DirLaunch L,
+           int use_tail) {
+    dir1_body<NT>(g, s, L, blockIdx.x, use_tail);
+}
+
+// Items of a batched launch, the directions of item i in CTAs [cta_ptr[i], cta_ptr[i + 1]).
+// The launch of the batch's other items may start beside this one.
+__global__ void __launch_bounds__(512, kLineRegs / 512) k_dir1_batch(const __grid_constant__ Dir1Batch B) {
+    pdl_trigger();
+    int i = 0;
+    while (i + 1 < B.n_items && (int)blockIdx.x >= B.cta_ptr[i + 1]) i++;
+    dir1_body<512>(B.g[i], B.s[i], B.l[i], (int)blockIdx.x - B.cta_ptr[i], B.l[i].use_tail);
 }
 
 // ---------------------------------------------------------------------------
@@ -2480,9 +2496,9 @@ cudaError_t prepare_kernels() {
     if (g_prepared[dev]) return cudaSuccess;
     e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
     if (e != cudaSuccess) return e;
-    const void* fns[7] = {(const void*)k_dirs, (const void*)k_solve1<256>, (const void*)k_solve1<512>,
+    const void* fns[8] = {(const void*)k_dirs, (const void*)k_solve1<256>, (const void*)k_solve1<512>,
                           (const void*)k_solve1_batch<256>, (const void*)k_solve1_batch<512>,
-                          (const void*)k_dir1<256>, (const void*)k_dir1<512>};
+                          (const void*)k_dir1<256>, (const void*)k_dir1<512>, (const void*)k_dir1_batch};
     for (const void* f : fns) {
         cudaFuncAttributes fa;
         e = cudaFuncGetAttributes(&fa, f);
@@ -2565,14 +2581,15 @@ int dirs_batch_ctas_per_sm(int threads) {
 }
 bool dirs_batch_shape_ok(int threads) { return dirs_batch_ctas_per_sm(threads) > 0; }
 
-void launch_dirs_batch(const DirBatch& B, int threads, cudaStream_t st) {
+cudaError_t launch_dirs_batch(const DirBatch& B, int threads, bool beside, cudaStream_t st) {
     const int n = B.n_items > 0 ? B.cta_ptr[B.n_items] : 0;
-    if (n <= 0) return;
+    if (n <= 0) return cudaSuccess;
+    const dim3 grid((unsigned)n), block((unsigned)threads);
     switch (threads) {
-        case 128: k_dirs_batch<128, 6><<<n, 128, 0, st>>>(B); break;
-        case 192: k_dirs_batch<192, 4><<<n, 192, 0, st>>>(B); break;
-        case 256: k_dirs_batch<256, 3><<<n, 256, 0, st>>>(B); break;
-        default: k_dirs_batch<kDirThreads, kDirCtasPerSm><<<n, kDirThreads, 0, st>>>(B); break;
+        case 128: return launch_pdl(beside, k_dirs_batch<128, 6>, grid, block, 0, st, B);
+        case 192: return launch_pdl(beside, k_dirs_batch<192, 4>, grid, block, 0, st, B);
+        case 256: return launch_pdl(beside, k_dirs_batch<256, 3>, grid, block, 0, st, B);
+        default: return launch_pdl(beside, k_dirs_batch<kDirThreads, kDirCtasPerSm>, grid, dim3(kDirThreads), 0, st, B);
     }
 }
 
@@ -2608,6 +2625,14 @@ int solve1_mode(int n_x, int T) {
     const size_t cap = 227 * 1024;
     if (T > 1 && T <= kSolve1Part && solve1_smem(n_x, T, true) <= cap) return 2;
     return solve1_smem(n_x, T, false) <= cap ? 1 : 0;
+}
+
+cudaError_t launch_dir1_batch(const Dir1Batch& B, cudaStream_t st) {
+    if (B.n_items <= 0) return cudaSuccess;
+    size_t smem = 0;
+    for (int i = 0; i < B.n_items; i++) smem = std::max(smem, solve1_smem(B.s[i].n_x, B.s[i].T, B.l[i].use_tail != 0));
+    k_dir1_batch<<<B.cta_ptr[B.n_items], 512, smem, st>>>(B);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_dir1(const DirGrid& g, const LineGrid& s, const DirLaunch& L, bool use_tail, cudaStream_t st) {

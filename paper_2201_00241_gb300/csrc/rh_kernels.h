@@ -132,7 +132,8 @@ struct DirBatch {
     DirLaunch l[kMaxBatch];
 };
 // threads: one of the compiled CTA shapes (dirs_batch_shape_ok)
-void launch_dirs_batch(const DirBatch& B, int threads, cudaStream_t st);
+// beside: started with the launch before it on `st` (launch_dir1_batch) instead of after it
+cudaError_t launch_dirs_batch(const DirBatch& B, int threads, bool beside, cudaStream_t st);
 bool dirs_batch_shape_ok(int threads);
 int dirs_batch_ctas_per_sm(int threads);   // resident CTAs per SM of a shape (0: not compiled)
 int dirs_batch_slots(int threads);         // resident CTAs of a shape on the current device
@@ -343,6 +344,17 @@ cudaError_t launch_solve1(const LineGrid& g, const double* x, double* out, bool 
 // direction c's rows at V + c * (zero_row + 1) and T likewise): SpMul to the U sweep, the
 // projection to SpMulAdd, or both.  Needs solve1_mode() > 0 and its schedule.
 cudaError_t launch_dir1(const DirGrid& g, const LineGrid& s, const DirLaunch& L, bool use_tail, cudaStream_t st);
+
+// Several items with one direction per CTA; all of line_threads(n_x) == 512.
+struct Dir1Batch {
+    int n_items;
+    int cta_ptr[kMaxBatch + 1];
+    DirGrid g[kMaxBatch];
+    LineGrid s[kMaxBatch];
+    DirLaunch l[kMaxBatch];
+};
+static_assert(sizeof(Dir1Batch) <= 32764, "kernel parameters");
+cudaError_t launch_dir1_batch(const Dir1Batch& B, cudaStream_t st);
 
 // Dense Cholesky of the tracking step (dense.cu).  A, L, B, work, y and info
 // are device pointers; column-major.  info receives 0 or the 1-based column of
