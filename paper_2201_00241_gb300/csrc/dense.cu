@@ -29,11 +29,11 @@
 //
 // The diagonal tile is eliminated without divisions: step j replaces every
 // trailing entry by 2^-e_j (d_j a_rc - a_rj a_cj), with d_j the current pivot and
-// 2^-e_j the power of two that brings it into [1, 2) (cross-multiplied
+// 2^-e_j a power of two, not 1 only where d_j is far from 1 (cross-multiplied
 // elimination, as in Bareiss's fraction-free Gaussian elimination, with an exact
 // power-of-two rescaling in place of Bareiss's exact division).  The trailing
 // block after step j is then s_{j+1} times the ordinary Schur complement, with
-// s_{j+1} = s_j 2^-e_j d_j in [s_j, 2 s_j): bounded by 2^TB inside a tile.  At the
+// s_{j+1} = s_j 2^-e_j d_j, within about 2^+-128 (see pivot_shift).  At the
 // end l_rc = a_rc / sqrt(s_c d_c) for r >= c (d_c = a_cc), one reciprocal
 // square root per column, and 1 / l_cc = s_c / sqrt(s_c d_c) and
 // 1 / d_c = s_c / (s_c d_c) follow by multiplications.  A step is one FMA and an
@@ -63,11 +63,11 @@ constexpr int kDenseThreads = 256;
 // while they fit in four warps.
 template <int TB>
 __device__ __forceinline__ void packed_entry(int p, int& r, int& c) {
-    const int e = TB * (TB + 1) / 2 - 1 - p;
-    int cc = 0;
-    while (cc + 1 < TB && (cc + 1) * TB - (cc + 1) * cc / 2 <= e) cc++;
-    c = cc;
-    r = cc + (e - (cc * TB - cc * (cc - 1) / 2));
+    int m = (int)((sqrtf(8.0f * (float)p + 1.0f) - 1.0f) * 0.5f);      // m (m + 1) / 2 <= p
+    m += (m + 1) * (m + 2) / 2 <= p;
+    m -= m * (m + 1) / 2 > p;
+    c = TB - 1 - m;
+    r = TB - 1 - (p - m * (m + 1) / 2);
 }
 
 // Loads the TB x TB tile of A at (i0, j0) with rb x cb live entries into T,
@@ -162,47 +162,61 @@ __device__ __forceinline__ void tile_sync() {
 // entries of the ordinary elimination (a_cc the pivot d_c), and
 //   W[c] = 1 / sqrt(s_c D[c][c]),  so l_rc = D[r][c] W[c] (the diagonal too),
 //   Inv[c] = s_c W[c] = 1 / l_cc,  Rd[c] = s_c W[c]^2 = 1 / D[c][c].
-// Run by the first NB threads of the CTA (and only by them); the last of them
-// keeps the running product s in S.  Column 0 is never updated, so the
-// TB (TB - 1) / 2 entries of the other columns are the ones that threads own.
+// Run by the first NB threads of the CTA (and only by them).  Column 0 is never updated, so
+// the TB (TB - 1) / 2 entries of the other columns are the ones that threads own, in a
+// register and, for the threads that need them as a pivot column, in D.
 template <int TB, int NB>
-__device__ __forceinline__ void chol_tile(double (*D)[TB + 1], int kb, double* S, double* W, double* Inv,
-                                          double* Rd) {
+__device__ __forceinline__ void chol_tile(double (*D)[TB + 1], int kb, double* W, double* Inv, double* Rd) {
     constexpr int NU = TB * (TB - 1) / 2;
     constexpr int QP = (NU + NB - 1) / NB;
     const int t = threadIdx.x;
     int er[QP], ec[QP];
+    double own[QP];
 #pragma unroll
-    for (int q = 0; q < QP; q++) packed_entry<TB>(min(t + q * NB, NU - 1), er[q], ec[q]);
-    double s = 1.0;
-    for (int j = 0; j < kb - 1; j++) {
+    for (int q = 0; q < QP; q++) {
+        packed_entry<TB>(min(t + q * NB, NU - 1), er[q], ec[q]);
+        own[q] = D[er[q]][ec[q]];
+    }
+#pragma unroll (TB <= 16 ? TB : 1)
+    for (int j = 0; j < TB - 1; j++) {
+        if (j >= kb - 1) break;
         const int na = (TB - 1 - j) * (TB - j) / 2;
         const double d = D[j][j];
         const int sh = pivot_shift(d);
 #pragma unroll
         for (int q = 0; q < QP; q++) {
-            if (t + q * NB < na) {
-                const int r = er[q], c = ec[q];
-                const double prod = D[r][j] * D[c][j];
-                D[r][c] = scale_pow2(fma(d, D[r][c], -prod), sh);
+            if ((t & ~31) + q * NB < na) {                   // the same for the warp
+                double v = fma(d, own[q], -(D[er[q]][j] * D[ec[q]][j]));
+                if (sh) v = scale_pow2(v, sh);
+                if (t + q * NB < na) {
+                    own[q] = v;
+                    D[er[q]][ec[q]] = v;
+                }
             }
-        }
-        if (t == NB - 1) {
-            s *= scale_pow2(d, sh);
-            S[j + 1] = s;
         }
         tile_sync<NB>();
     }
-    if (t < kb) {
-        const double st = t ? S[t] : 1.0;        // S[0] is never written (kb = 1 has no step)
-        const double w = rsqrt(st * D[t][t]);
-        W[t] = w;
-        Inv[t] = st * w;
-        Rd[t] = (st * w) * w;
-    } else if (t < TB) {
-        W[t] = 0.0;
-        Inv[t] = 0.0;
-        Rd[t] = 0.0;
+    if (t < 32) {
+        // s_t: the product of the scaled pivots before t
+        const double d = t < kb - 1 ? D[t][t] : 1.0;
+        double st = scale_pow2(d, pivot_shift(d));
+        st = __shfl_up_sync(0xffffffffu, st, 1);
+        if (t == 0) st = 1.0;
+#pragma unroll
+        for (int o = 1; o < TB; o <<= 1) {
+            const double u = __shfl_up_sync(0xffffffffu, st, o);
+            if (t >= o) st *= u;
+        }
+        if (t < kb) {
+            const double w = rsqrt(st * D[t][t]);
+            W[t] = w;
+            Inv[t] = st * w;
+            Rd[t] = (st * w) * w;
+        } else if (t < TB) {
+            W[t] = 0.0;
+            Inv[t] = 0.0;
+            Rd[t] = 0.0;
+        }
     }
     tile_sync<NB>();
 }
@@ -253,7 +267,7 @@ __global__ void __launch_bounds__(kDenseThreads)
     __shared__ double X[TB][TB + 1];
     __shared__ double Li[TB][TB + 1];
     __shared__ double Lc[TB][TB + 1];
-    __shared__ double S[TB], W[TB], Inv[TB], Rd[TB], Z[TB];
+    __shared__ double W[TB], Inv[TB], Rd[TB], Z[TB];
     __shared__ int Es[TB];
     const int t = threadIdx.x;
     const int nt = (n + TB - 1) / TB;
@@ -298,7 +312,7 @@ __global__ void __launch_bounds__(kDenseThreads)
             // the factorisation needs half the CTA: the other half updates X meanwhile
             constexpr int H = kDenseThreads / 2;
             if (t < H) {
-                chol_tile<TB, H>(D, kb, S, W, Inv, Rd);
+                chol_tile<TB, H>(D, kb, W, Inv, Rd);
             } else {
                 for (int e = t - H; e < TB * TB; e += H) update_x(e);
             }
@@ -307,7 +321,7 @@ __global__ void __launch_bounds__(kDenseThreads)
 #pragma unroll
             for (int q = 0; q < R; q++) update_x(t + q * kDenseThreads);
             __syncthreads();
-            chol_tile<TB, kDenseThreads>(D, kb, S, W, Inv, Rd);
+            chol_tile<TB, kDenseThreads>(D, kb, W, Inv, Rd);
         }
         diag_multipliers<TB>(D, Rd);
         // X L_cc^T = A_ic, unscaled (x_rj l_jj): the rows are independent, each
@@ -346,7 +360,7 @@ __global__ void __launch_bounds__(kDenseThreads)
         else
             equilibrate_diag<TB>(D, Es);
         __syncthreads();
-        chol_tile<TB, kDenseThreads>(D, kb, S, W, Inv, Rd);
+        chol_tile<TB, kDenseThreads>(D, kb, W, Inv, Rd);
         chol_store_tile<TB>(A, lda, k0, kb, D, W, Es, info);
         return;
     }
@@ -376,7 +390,7 @@ __global__ void __launch_bounds__(kDenseThreads)
             equilibrate_diag<TB>(D, Es);
         }
         __syncthreads();
-        chol_tile<TB, kDenseThreads>(D, kb, S, W, Inv, Rd);
+        chol_tile<TB, kDenseThreads>(D, kb, W, Inv, Rd);
         diag_multipliers<TB>(D, Rd);
         if (t < 32) {
             const int r = t % TB;

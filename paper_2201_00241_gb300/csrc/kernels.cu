@@ -669,8 +669,9 @@ __global__ void k_tail_gather(RfGrid g) {
 // last diagonal entry): the entries with r, c > j are exactly p < (TB-1-j)^2.
 __device__ __forceinline__ void tail_shell_entry(int p, int& r, int& c) {
     constexpr int TB = kTailTB;
-    int q = 0;
-    while ((q + 1) * (q + 1) <= p) q++;
+    int q = (int)sqrtf((float)p);
+    q += (q + 1) * (q + 1) <= p;
+    q -= q * q > p;
     const int m = TB - 1 - q, o = p - q * q;
     r = o <= q ? m : m + (o - q);
     c = o == 0 ? m : (o <= q ? m + o : m);
@@ -686,28 +687,37 @@ __device__ __forceinline__ void tail_factor(double* D, int ld, int kb, double* S
     const int t = threadIdx.x;
     int er = 0, ec = 0;
     tail_shell_entry(min(t, (TB - 1) * (TB - 1) - 1), er, ec);
-    double s = 1.0;
-    for (int j = 0; j < kb - 1; j++) {
+    double own = D[er * ld + ec];
+#pragma unroll
+    for (int j = 0; j < TB - 1; j++) {
+        if (j >= kb - 1) break;
         const int na = (TB - 1 - j) * (TB - 1 - j);
-        const double d = D[j * ld + j];
-        const int sh = pivot_shift(d);
-        if (t < na) {
-            const double prod = D[er * ld + j] * D[j * ld + ec];
-            D[er * ld + ec] = scale_pow2(fma(d, D[er * ld + ec], -prod), sh);
-        }
-        if (t == 255) {
-            s *= scale_pow2(d, sh);
-            S[j + 1] = s;
+        if ((t & ~31) < na) {                            // the same for the warp
+            const double d = D[j * ld + j];
+            const int sh = pivot_shift(d);
+            double v = fma(d, own, -(D[er * ld + j] * D[j * ld + ec]));
+            if (sh) v = scale_pow2(v, sh);
+            if (t < na) {
+                own = v;
+                D[er * ld + ec] = v;
+            }
         }
         tail_sync();
     }
-    if (t < TB) {
-        if (t < kb) {
-            if (t == 0) S[0] = 1.0;
-            Rd[t] = 1.0 / D[t * ld + t];
-        } else {
-            S[t] = 0.0;
-            Rd[t] = 0.0;
+    if (t < 32) {
+        // s_t: the product of the scaled pivots before t
+        const double d = t < kb - 1 ? D[t * ld + t] : 1.0;
+        double st = scale_pow2(d, pivot_shift(d));
+        st = __shfl_up_sync(0xffffffffu, st, 1);
+        if (t == 0) st = 1.0;
+#pragma unroll
+        for (int o = 1; o < TB; o <<= 1) {
+            const double u = __shfl_up_sync(0xffffffffu, st, o);
+            if (t >= o) st *= u;
+        }
+        if (t < TB) {
+            S[t] = t < kb ? st : 0.0;
+            Rd[t] = t < kb ? 1.0 / D[t * ld + t] : 0.0;
         }
     }
     tail_sync();

@@ -182,14 +182,17 @@ __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.lau
 // ---- division-free elimination of dense tiles -----------------------------------
 // The diagonal tiles of the dense factorisations (the refactorisation's dense
 // tail LU, the tracking step's Cholesky) are eliminated by cross-multiplied steps
-// a_rc <- 2^-e (d a_rc - a_rj a_jc), d the current pivot and 2^-e the power of two
-// that brings it into [1, 2), instead of a reciprocal of every pivot on the
-// critical path.
-// e with 2^-e d in [1, 2) for a positive normal pivot d (e <= 1022, so 2^-e is
-// normal too); 0 for any other value, where the factorisation has failed.
+// a_rc <- 2^-e (d a_rc - a_rj a_jc), d the current pivot, instead of a reciprocal of
+// every pivot on the critical path.  e is 0 while d lies within 2^+-64 and otherwise the
+// power of two that brings |d| into [1, 2): the values then stay within about 2^+-200 of
+// the tile's own, and most steps do not carry the exponent update (12 dependent integer
+// instructions) in their chain.  A 16 x 16 tile of the tail's LU: 8300 cycles with the
+// update, the own entry and its indexes in every step, 6000 without.
+// e for a pivot d: 0 also where d is zero, subnormal, infinite or NaN and the
+// factorisation has failed (|e| <= 1022, so 2^-e is normal).
 __device__ __forceinline__ int pivot_shift(double d) {
-    const int f = (int)((__double_as_longlong(d) >> 52) & 0x7ff);
-    return (d > 0.0 && f != 0 && f != 0x7ff) ? min(f - 1023, 1022) : 0;
+    const int f = (__double2hiint(d) >> 20) & 0x7ff, e = f - 1023;
+    return ((unsigned)(e + 64) > 128u && f != 0 && f != 0x7ff) ? min(e, 1022) : 0;
 }
 
 // v * 2^-sh for |sh| <= 1022 by an integer update of the exponent field, with
