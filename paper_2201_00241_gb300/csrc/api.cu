@@ -91,6 +91,7 @@ struct rh_grid {
     int *blev_ptr = nullptr, *blev_bus = nullptr, *blev_maxext = nullptr;
     int *rf_lev_bus = nullptr, *rf_tgt_pos = nullptr, *rf_grp = nullptr, *rf_xgrp = nullptr;
     int64_t* rf_xptr = nullptr;
+    int4* rf_lev = nullptr;                       // per level: first target, targets, first pivot job, jobs
     int *rf_piv_bus = nullptr, *rf_piv_pos = nullptr;
     double4_32a* rf_piv = nullptr;          // per sparse bus: 1/u_tt, l_vt, 1/u_vv, u_tv
     int *rf_pe_bus = nullptr, *rf_pe_pos = nullptr;
@@ -264,7 +265,7 @@ struct rh_grid {
         g.rf_lev_bus = rf_lev_bus; g.q0 = q0; g.nv = nv;
         g.rowptr = rowptr; g.col = col; g.diagpos = diagpos; g.tpos = tpos;
         g.tgt_pos = rf_tgt_pos; g.grp = reinterpret_cast<const int2*>(rf_grp);
-        g.xptr = rf_xptr; g.xgrp = reinterpret_cast<const int2*>(rf_xgrp);
+        g.lev = rf_lev; g.xptr = rf_xptr; g.xgrp = reinterpret_cast<const int2*>(rf_xgrp);
         g.piv = rf_piv; g.n_piv = S.tail_bus0; g.piv_bus = rf_piv_bus; g.piv_pos = rf_piv_pos;
         g.n_pe = (int64_t)S.rf_pe_bus.size(); g.pe_bus = rf_pe_bus; g.pe_pos = reinterpret_cast<const int4*>(rf_pe_pos);
         g.A = A; g.invdiag = invdiag; g.jmax = umax + 1; g.err = err;
@@ -1171,6 +1172,13 @@ rh_status rh_grid_create(const rh_grid_desc* d, int32_t device, rh_grid** out) {
     RH_CUDA(g->upload(g->rf_tgt_pos, S.rf_tgt_pos));
     RH_CUDA(g->upload(g->rf_grp, S.rf_grp));
     RH_CUDA(g->upload(g->rf_xptr, S.rf_xptr));
+    {
+        std::vector<int4> lev(S.rf_n_lev);
+        for (int l = 0; l < S.rf_n_lev; l++)
+            lev[l] = make_int4((int)S.rf_tgt_lev_ptr[l], (int)(S.rf_tgt_lev_ptr[l + 1] - S.rf_tgt_lev_ptr[l]),
+                               S.rf_piv_lev_ptr[l], S.rf_piv_lev_ptr[l + 1] - S.rf_piv_lev_ptr[l]);
+        RH_CUDA(g->upload(g->rf_lev, lev));
+    }
     RH_CUDA(g->upload(g->rf_xgrp, S.rf_xgrp));
     RH_CUDA(g->upload(g->rf_piv_bus, S.rf_piv_bus));
     RH_CUDA(g->upload(g->rf_piv_pos, S.rf_piv_pos));

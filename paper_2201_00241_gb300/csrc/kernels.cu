@@ -545,72 +545,106 @@ __device__ __forceinline__ double rf_group(const RfGrid& g, int2 d, int2 tu, int
 // as soon as this one's wait is over: between two levels only the values' loads, their
 // FMAs and the hand-over remain.  First-order derivatives at 9241 buses 894 -> 783 us (74
 // launches), eight Newton re-solves at 1354 buses 1203 -> 1124 us.
-__device__ __forceinline__ void k_rf_update_body(const RfGrid& g, int64_t t0, int64_t nt, int j0, int njob) {
-    const int64_t tl = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int64_t t = t0 + (tl < nt ? tl : 0);
-    const int64_t wbase = tl - (int64_t)(threadIdx.x & 31);
-    const bool job_warp = wbase < 4 * (int64_t)njob, mine = tl < 4 * (int64_t)njob;
-    const int e = (int)(tl & 3);
-    const int64_t q = tl >> 2;
-    int p = -1, pos3 = -1, pp = -1, bus = 0;
-    int2 d = make_int2(0, 0), tu = make_int2(-1, 0), vu = tu;
-    int2 x[2][3] = {{d, tu, vu}, {d, tu, vu}};
-    int64_t x0 = 0, x1 = 0;
+struct RfPre {
+    int p, pos3, pp, bus;
+    int2 d, tu, vu, x[2][3];
+    int64_t x0, x1;
+};
+__device__ __forceinline__ void rf_load(const RfGrid& g, int64_t t0, int64_t nt, int j0, int njob, int64_t tl,
+                                        RfPre& r) {
+    r.p = r.pos3 = r.pp = -1;
+    r.bus = 0;
+    r.d = make_int2(0, 0);
+    r.tu = r.vu = make_int2(-1, 0);
+    r.x0 = r.x1 = 0;
     if (tl < nt) {
-        p = g.tgt_pos[t];
-        d = g.grp[3 * t];
-        tu = g.grp[3 * t + 1];
-        vu = g.grp[3 * t + 2];
-        x0 = g.xptr[t];
-        x1 = g.xptr[t + 1];
+        const int64_t t = t0 + tl;
+        r.p = g.tgt_pos[t];
+        r.d = g.grp[3 * t];
+        r.tu = g.grp[3 * t + 1];
+        r.vu = g.grp[3 * t + 2];
+        r.x0 = g.xptr[t];
+        r.x1 = g.xptr[t + 1];
     }
-    if (mine) {
-        pos3 = g.piv_pos[4 * (j0 + q) + 3];
-        pp = g.piv_pos[4 * (j0 + q) + e];
-        bus = g.piv_bus[j0 + q];
+    if (tl < 4 * (int64_t)njob) {
+        const int64_t q = j0 + (tl >> 2);
+        r.pos3 = g.piv_pos[4 * q + 3];
+        r.pp = g.piv_pos[4 * q + (tl & 3)];
+        r.bus = g.piv_bus[q];
     }
 #pragma unroll
     for (int m = 0; m < 2; m++)
-        if (x0 + m < x1) {
-            x[m][0] = g.xgrp[3 * (x0 + m)];
-            x[m][1] = g.xgrp[3 * (x0 + m) + 1];
-            x[m][2] = g.xgrp[3 * (x0 + m) + 2];
-        }
-    pdl_wait();
-    pdl_trigger();
+#pragma unroll
+        for (int k = 0; k < 3; k++) r.x[m][k] = r.x0 + m < r.x1 ? g.xgrp[3 * (r.x0 + m) + k] : make_int2(-1, 0);
+}
+// All lanes of a warp call it with consecutive tl.
+__device__ __forceinline__ void rf_apply(const RfGrid& g, int njob, int64_t tl, const RfPre& r) {
     double nv = 0.0;
-    if (p >= 0 && inb(p, g.nnz)) {
-        double acc = rf_group(g, d, tu, vu, 0.0);
-        if (x0 < x1) acc = rf_group(g, x[0][0], x[0][1], x[0][2], acc);
-        if (x0 + 1 < x1) acc = rf_group(g, x[1][0], x[1][1], x[1][2], acc);
-        int64_t c = x0 + 2;
-        for (; c + 1 < x1; c += 2) {
+    if (r.p >= 0 && inb(r.p, g.nnz)) {
+        double acc = rf_group(g, r.d, r.tu, r.vu, 0.0);
+        if (r.x0 < r.x1) acc = rf_group(g, r.x[0][0], r.x[0][1], r.x[0][2], acc);
+        if (r.x0 + 1 < r.x1) acc = rf_group(g, r.x[1][0], r.x[1][1], r.x[1][2], acc);
+        int64_t c = r.x0 + 2;
+        for (; c + 1 < r.x1; c += 2) {
             const int2 da = g.xgrp[3 * c], tua = g.xgrp[3 * c + 1], vua = g.xgrp[3 * c + 2];
             const int2 db = g.xgrp[3 * c + 3], tub = g.xgrp[3 * c + 4], vub = g.xgrp[3 * c + 5];
             acc = rf_group(g, da, tua, vua, acc);
             acc = rf_group(g, db, tub, vub, acc);
         }
-        if (c < x1) acc = rf_group(g, g.xgrp[3 * c], g.xgrp[3 * c + 1], g.xgrp[3 * c + 2], acc);
-        nv = g.A[p] - acc;
-        g.A[p] = nv;
+        if (c < r.x1) acc = rf_group(g, g.xgrp[3 * c], g.xgrp[3 * c + 1], g.xgrp[3 * c + 2], acc);
+        nv = g.A[r.p] - acc;
+        g.A[r.p] = nv;
     }
     // pivot jobs: the quads are whole within a warp, and a warp that holds any of
     // them runs the shuffles with all its lanes
-    if (job_warp) {
+    if (tl - (int64_t)(threadIdx.x & 31) < 4 * (int64_t)njob) {
+        const int e = (int)(tl & 3);
+        const bool mine = tl < 4 * (int64_t)njob;
         double v = nv;
-        if (mine && p < 0) v = (pp >= 0 && inb(pp, g.nnz)) ? g.A[pp] : 0.0;
+        if (mine && r.p < 0) v = (r.pp >= 0 && inb(r.pp, g.nnz)) ? g.A[r.pp] : 0.0;
         const int b = (int)(threadIdx.x & 28);
         const double att = __shfl_sync(0xffffffffu, v, b);
         const double atv = __shfl_sync(0xffffffffu, v, b + 1);
         const double avt = __shfl_sync(0xffffffffu, v, b + 2);
         const double avv = __shfl_sync(0xffffffffu, v, b + 3);
         // the two reciprocals in one division: 1/a_tt on lane 0 of the quad, 1/det on lane 3
-        const double x = e == 0 ? att : (e == 3 && pos3 >= 0 ? rf_det(att, atv, avt, avv) : 1.0);
-        const double r = 1.0 / x;
-        const double idet = __shfl_sync(0xffffffffu, r, b + 3);
-        if (mine && e == 0) rf_piv_store(g, bus, att, atv, avt, r, idet, pos3 >= 0);
+        const double x = e == 0 ? att : (e == 3 && r.pos3 >= 0 ? rf_det(att, atv, avt, avv) : 1.0);
+        const double rx = 1.0 / x;
+        const double idet = __shfl_sync(0xffffffffu, rx, b + 3);
+        if (mine && e == 0) rf_piv_store(g, r.bus, att, atv, avt, rx, idet, r.pos3 >= 0);
     }
 }
+__device__ __forceinline__ void k_rf_update_body(const RfGrid& g, int64_t t0, int64_t nt, int j0, int njob) {
+    const int64_t tl = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    RfPre r;
+    rf_load(g, t0, nt, j0, njob, tl, r);
+    pdl_wait();
+    pdl_trigger();
+    rf_apply(g, njob, tl, r);
+}
+
+// Levels l0 .. l1 - 1, of at most kRfThreads targets each, in one CTA: a CTA barrier between
+// two of them takes less than a launch.  A thread reads its target's groups of the next
+// level before the barrier.  The reduced Hessian at 118 buses (13 levels) 176 -> 172 us.
+// (Wider levels on a cluster of 8 CTAs with a cluster barrier between them were slower
+// than their launches: eight re-solves at 1354 buses 1081 -> 1113 us.)
+constexpr int kRfThreads = 512;
+__device__ __forceinline__ void rf_levels_body(const RfGrid& g, int l0, int l1) {
+    int4 lv = g.lev[l0];                                    // first target, targets, first pivot job, jobs
+    RfPre r;
+    rf_load(g, lv.x, lv.y, lv.z, lv.w, threadIdx.x, r);
+    pdl_wait();
+    pdl_trigger();
+    for (int l = l0; l < l1; l++) {
+        rf_apply(g, lv.w, threadIdx.x, r);
+        if (l + 1 < l1) {
+            lv = g.lev[l + 1];
+            rf_load(g, lv.x, lv.y, lv.z, lv.w, threadIdx.x, r);
+            __syncthreads();
+        }
+    }
+}
+__global__ void __launch_bounds__(kRfThreads) k_rf_levels(RfGrid g, int l0, int l1) { rf_levels_body(g, l0, l1); }
 __global__ void k_rf_update(RfGrid g, int64_t t0, int64_t nt, int j0, int njob) {
     k_rf_update_body(g, t0, nt, j0, njob);
 }
@@ -2335,6 +2369,9 @@ __global__ void k_newton_update_batch(PfBatch B) {
 __global__ void k_rf_update_batch(RfBatch B, int64_t t0, int64_t nt, int j0, int njob) {
     k_rf_update_body(B.g[blockIdx.y], t0, nt, j0, njob);
 }
+__global__ void __launch_bounds__(kRfThreads) k_rf_levels_batch(RfBatch B, int l0, int l1) {
+    rf_levels_body(B.g[blockIdx.y], l0, l1);
+}
 __global__ void k_rf_leaf_piv_batch(RfBatch B, int njob) {
     k_rf_leaf_piv_body(B.g[blockIdx.y], njob);
 }
@@ -2451,6 +2488,14 @@ void launch_prefetch_l2(const PrefetchList& in, cudaStream_t st) {
     if (nc > 0) k_prefetch_l2<<<(unsigned)((nc + 31) / 32), 32, 0, st>>>(L);
 }
 
+// The first of the last levels that one CTA runs in one launch (n_lev: none; a single level
+// is no gain).
+static int rf_one_cta(const int64_t* tgt_lev_ptr_host, int n_lev) {
+    int l = n_lev;
+    while (l > 0 && tgt_lev_ptr_host[l] - tgt_lev_ptr_host[l - 1] <= kRfThreads) l--;
+    return n_lev - l > 1 ? l : n_lev;
+}
+
 cudaError_t launch_refactor(const RfGrid& g, const int* lev_ptr_host, const int64_t* tgt_lev_ptr_host,
                             const int* piv_lev_ptr_host, int n_lev, cudaStream_t st) {
     (void)lev_ptr_host;
@@ -2463,11 +2508,13 @@ cudaError_t launch_refactor(const RfGrid& g, const int* lev_ptr_host, const int6
     if (n_lev > 0 && piv_lev_ptr_host[0] > 0)
         chk(launch_pdl(pdl, k_rf_leaf_piv, dim3(blocks_for(piv_lev_ptr_host[0], 128)), dim3(128), 0, st, g,
                        piv_lev_ptr_host[0]));
-    for (int lev = 0; lev < n_lev; lev++) {
+    const int l0 = rf_one_cta(tgt_lev_ptr_host, n_lev);
+    for (int lev = 0; lev < l0; lev++) {
         const int64_t t0 = tgt_lev_ptr_host[lev], nt = tgt_lev_ptr_host[lev + 1] - t0;
         const int j0 = piv_lev_ptr_host[lev], njob = piv_lev_ptr_host[lev + 1] - j0;
         if (nt > 0) chk(launch_pdl(pdl, k_rf_update, dim3(blocks_for(nt, 256)), dim3(256), 0, st, g, t0, nt, j0, njob));
     }
+    if (l0 < n_lev) chk(launch_pdl(pdl, k_rf_levels, dim3(1), dim3(kRfThreads), 0, st, g, l0, n_lev));
     if (tail_in_one(g.T)) {
         chk(launch_pdl(pdl, k_rf_finish, dim3(1 + blocks_for((int64_t)g.n_piv + g.n_pe, kTailThreads)),
                        dim3(kTailThreads), 0, st, g));
@@ -2705,13 +2752,15 @@ cudaError_t launch_refactor_batch(const RfBatch& B, const int* lev_ptr_host, con
     if (n_lev > 0 && piv_lev_ptr_host[0] > 0)
         chk(launch_pdl(pdl, k_rf_leaf_piv_batch, dim3((unsigned)blocks_for(piv_lev_ptr_host[0], 128), n), dim3(128), 0, st,
                        B, piv_lev_ptr_host[0]));
-    for (int lev = 0; lev < n_lev; lev++) {
+    const int l0 = rf_one_cta(tgt_lev_ptr_host, n_lev);
+    for (int lev = 0; lev < l0; lev++) {
         const int64_t t0 = tgt_lev_ptr_host[lev], nt = tgt_lev_ptr_host[lev + 1] - t0;
         const int j0 = piv_lev_ptr_host[lev], njob = piv_lev_ptr_host[lev + 1] - j0;
         if (nt > 0)
             chk(launch_pdl(pdl, k_rf_update_batch, dim3((unsigned)blocks_for(nt, 256), n), dim3(256), 0, st, B, t0, nt, j0,
                            njob));
     }
+    if (l0 < n_lev) chk(launch_pdl(pdl, k_rf_levels_batch, dim3(1, n), dim3(kRfThreads), 0, st, B, l0, n_lev));
     const int64_t np = (int64_t)B.g[0].n_piv + B.g[0].n_pe;
     if (tail_in_one(B.g[0].T)) {
         chk(launch_pdl(pdl, k_rf_finish_batch, dim3((unsigned)(1 + blocks_for(np, kTailThreads)), n), dim3(kTailThreads),

@@ -261,6 +261,7 @@ struct RfGrid {
     // its further groups [xptr[t], xptr[t + 1])
     const int2 *grp, *xgrp;
     const int64_t *xptr;
+    const int4 *lev;                   // per level: first target, targets, first pivot job, pivot jobs
     // pivot quantities per sparse bus (1/u_tt, l_vt, 1/u_vv, u_tv), written by the
     // pivot jobs (bus piv_bus[q], block positions piv_pos[4 q ..]; see launch_refactor)
     double4_32a *piv;
