@@ -496,9 +496,9 @@ rh_status capture_graph(rh_grid* g, F&& enqueue, cudaGraphExec_t* exec, int* ker
 // Injections, residual (when gres is given) and the values of J_x (into the
 // slots of A, cleared first together with the maxima and the pivot flag) and J_p,
 // by the analytic formulas or by coloured forward-mode AD (enqueue only).
-rh_status assemble(rh_grid* g, int method, double* gres, cudaStream_t s) {
+rh_status assemble(rh_grid* g, int method, double* gres, cudaStream_t s, bool chained = false) {
     const bool ad = (method == RH_JAC_COLORED_AD);
-    rh::launch_pf_prep(g->pf(), g->st(), g->A, g->umax, g->err, true, s);
+    rh::launch_pf_prep(g->pf(), g->st(), g->A, g->umax, g->err, true, chained, s);
     rh::launch_pf_eval(g->pf(), g->st(), gres, g->A, g->jpv, g->umax, g->umax + 1, !ad, s);
     if (ad)
         RH_CUDA(rh::launch_jac_ad(g->pf(), g->st(), g->col_th, g->col_v, g->col_pg,
@@ -726,23 +726,28 @@ rh_status dirs(rh_grid* g, int N, int64_t ld, double* V, double* T, const double
     return RH_OK;
 }
 
-// single right-hand side in g->v1 (internal order), the solution in `out`.  beside_dirs: as
+// single right-hand side `in` (internal order), the solution in `out`.  beside_dirs: as
 // one CTA of the direction kernel, which fits in the slot a direction launch of
 // fewer CTAs than the device holds leaves free (k_solve1's shared-memory x
 // needs a shared-memory carveout that an SM running k_dirs does not have).
-rh_status solve_one(rh_grid* g, unsigned phases, double* out, cudaStream_t s, bool beside_dirs = false) {
+// *chained: whether the operation before is a kernel, and on return whether the last one is.
+rh_status solve_one(rh_grid* g, unsigned phases, const double* in, double* out, cudaStream_t s, bool* chained,
+                    bool beside_dirs = false) {
     const int mode = beside_dirs || g->n_line < 0 ? 0 : rh::solve1_mode(g->S.n_x, g->S.n_x - g->S.t0);
     if (mode > 0) {
-        RH_CUDA(rh::launch_solve1(g->s1(), g->v1, out, (phases & rh::PH_LT) != 0, mode == 2, s));
+        RH_CUDA(rh::launch_solve1(g->s1(), in, out, (phases & rh::PH_LT) != 0, mode == 2, *chained, s));
+        *chained = true;
         return RH_OK;
     }
     // through k_dirs, whose factors are unit-diagonal (J_x = D L'' U'): the right-hand
     // side of J_x z = b enters as D^-1 b, and J_x^T's solution D psi leaves as psi
+    if (in != g->v1) RH_CUDA(cudaMemcpyAsync(g->v1, in, g->S.n_x * sizeof(double), cudaMemcpyDeviceToDevice, s));
     if (phases & rh::PH_L) rh::launch_scale_rows(g->S.n_x, 1, g->invdiag, g->v1, 1, s);
     rh_status st = dirs(g, 1, 1, g->v1, g->v1, nullptr, 0, 0, nullptr, 0, phases, s);
     if (st) return st;
     if (phases & rh::PH_LT) rh::launch_scale_rows(g->S.n_x, 1, g->invdiag, g->v1, 1, s);
     if (out != g->v1) RH_CUDA(cudaMemcpyAsync(out, g->v1, g->S.n_x * sizeof(double), cudaMemcpyDeviceToDevice, s));
+    *chained = false;
     return RH_OK;
 }
 
@@ -1368,11 +1373,11 @@ rh_status rh_powerflow(rh_grid* g, const double* x0, double tol, int32_t max_ite
         st = capture_graph(
             g,
             [&]() -> rh_status {
-                RH_CUDA(cudaMemcpyAsync(g->v1, g->gres, nx * sizeof(double), cudaMemcpyDeviceToDevice, g->stream));
-                rh_status ss = solve_one(g, rh::PH_L | rh::PH_U, g->v1, g->stream);
+                bool chained = false;
+                rh_status ss = solve_one(g, rh::PH_L | rh::PH_U, g->gres, g->v1, g->stream, &chained);
                 if (ss) return ss;
-                rh::launch_newton_update(g->pf(), g->st(), g->v1, g->stream);
-                return assemble(g, g->jac_method, g->gres, g->stream);
+                rh::launch_newton_update(g->pf(), g->st(), g->v1, chained, g->stream);
+                return assemble(g, g->jac_method, g->gres, g->stream, true);
             },
             &g->nt_step_exec, &nk);
         if (st) return st;
@@ -1443,13 +1448,14 @@ rh_status enqueue_adjoint_chain(rh_grid* g, cudaStream_t s, bool beside_dirs) {
     a.gref_th = g->gref_th; a.gref_v = g->gref_v; a.gref_row = g->gref_row; a.gref_val = g->gref_val;
     a.n_gref = g->n_gref; a.uth = g->uth; a.uv = g->uv;
     rh::launch_adjoint_rhs(g->pf(), g->st(), a, s);
-    rh_status st = solve_one(g, rh::PH_UT | rh::PH_LT, g->lam, s, beside_dirs);
+    bool chained = true;
+    rh_status st = solve_one(g, rh::PH_UT | rh::PH_LT, g->v1, g->lam, s, &chained, beside_dirs);
     if (st) return st;
     rh::CoefData c;
     c.lam = g->lam; c.cref = g->dscal; c.gref_v = g->gref_v; c.inc_ptr = g->inc_ptr; c.coef = g->inc_coef;
     c.d2 = g->d2; c.asum = g->asum; c.csum = g->csum; c.pg_curv = g->pg_curv;
     c.jpt_ptr = g->jpt_ptr; c.jpt_row = g->jpt_row; c.jptv = g->jptv; c.grad = g->grad;
-    rh::launch_adjoint_coef(g->pf(), g->st(), c, s);
+    rh::launch_adjoint_coef(g->pf(), g->st(), c, chained, s);
     RH_CUDA(cudaGetLastError());
     return RH_OK;
 }
@@ -1575,11 +1581,12 @@ rh_status enqueue_batch_newton(rh_grid* const* items, int n, uint32_t mask, int 
         // x does not fit in one CTA's shared memory: the direction kernel solves each item
         for (rh_grid* g : act) {
             enqueue_factor_copies(g, s);
-            rh_status st = solve_one(g, rh::PH_L | rh::PH_U, g->v1, s);
+            bool chained = false;
+            rh_status st = solve_one(g, rh::PH_L | rh::PH_U, g->v1, g->v1, s, &chained);
             if (st) return st;
         }
     }
-    rh::launch_newton_update_batch(*B, s);
+    rh::launch_newton_update_batch(*B, mode > 0, s);
     RH_CUDA(cudaGetLastError());
     return RH_OK;
 }

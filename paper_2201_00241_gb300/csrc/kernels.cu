@@ -156,7 +156,11 @@ __device__ __forceinline__ void k_pf_eval_body(PfGrid g, PfState s, double* gres
     atomicMax(jmax, jm);
 }
 __global__ void k_pf_eval(PfGrid g, PfState s, double* gres, double* A, double* jpv,
-                          unsigned long long* gmax, unsigned long long* jmax, int want_jac) { k_pf_eval_body(g, s, gres, A, jpv, gmax, jmax, want_jac); }
+                          unsigned long long* gmax, unsigned long long* jmax, int want_jac) {
+    pdl_wait();
+    pdl_trigger();
+    k_pf_eval_body(g, s, gres, A, jpv, gmax, jmax, want_jac);
+}
 
 // Per-state preparation of the assembly: sin and cos of every bus angle (the
 // assembly then forms sin and cos of each angle difference with two products), and,
@@ -182,6 +186,7 @@ __device__ __forceinline__ void pf_prep_body(const PfGrid& g, const PfState& s, 
         }
 }
 __global__ void k_pf_prep(PfGrid g, PfState s, double* A, unsigned long long* umax, int* err, int zero) {
+    pdl_wait();
     pf_prep_body(g, s, A, umax, err, zero);
 }
 
@@ -295,6 +300,8 @@ __device__ __forceinline__ void pf_eval_warp_body(const PfGrid& g, const PfState
 __global__ void __launch_bounds__(32 * kPfWarps) k_pf_eval_warp(PfGrid g, PfState s, double* gres, double* A,
                                                                 double* jpv, unsigned long long* gmax,
                                                                 unsigned long long* jmax, int want_jac) {
+    pdl_wait();
+    pdl_trigger();
     pf_eval_warp_body(g, s, gres, A, jpv, gmax, jmax, want_jac);
 }
 
@@ -304,7 +311,11 @@ __device__ __forceinline__ void k_newton_update_body(PfGrid g, PfState s, const 
     if (g.qth[i] >= 0) s.va[i] -= dx[g.qth[i]];
     if (g.qv[i] >= 0) s.vm[i] -= dx[g.qv[i]];
 }
-__global__ void k_newton_update(PfGrid g, PfState s, const double* dx) { k_newton_update_body(g, s, dx); }
+__global__ void k_newton_update(PfGrid g, PfState s, const double* dx) {
+    pdl_wait();
+    pdl_trigger();
+    k_newton_update_body(g, s, dx);
+}
 
 // ---------------------------------------------------------------------------
 // coloured forward-mode Jacobian (section 4.2.2, Fig. 2)
@@ -1959,6 +1970,7 @@ __device__ __forceinline__ void line_values_body(const LineGrid& g, bool trans, 
 }
 // blockIdx.y 0: of the factors into `line`, 1: of their transpose into `tline`
 __global__ void k_line_values(const __grid_constant__ LineGrid g) {
+    pdl_wait();
     line_values_body(g, blockIdx.y != 0, blockIdx.y ? g.tline : g.line);
 }
 
@@ -1992,6 +2004,8 @@ __device__ __forceinline__ void k_solve1_body(const LineGrid& g, const double* x
 template <int NT>
 __global__ void __launch_bounds__(NT, kLineRegs / NT)
     k_solve1(const __grid_constant__ LineGrid g, const double* x, double* out, int trans, int use_tail) {
+    pdl_wait();
+    if (NT == 256) pdl_trigger();
     k_solve1_body<NT>(g, x, out, trans, use_tail);
 }
 
@@ -2312,6 +2326,8 @@ __device__ __forceinline__ void gradient_bus(const PfGrid& g, const PfState& s, 
 // What follows from lambda: the projection's coefficients (the first n_coef blocks) and
 // grad F (the others); as two kernels with a thread per bus 33 + 11 us at 9241 buses.
 __global__ void __launch_bounds__(kCoefThreads) k_adjoint_coef(PfGrid g, PfState s, CoefData c, int n_coef) {
+    pdl_wait();
+    pdl_trigger();
     if ((int)blockIdx.x >= n_coef) gradient_bus(g, s, c, ((int)blockIdx.x - n_coef) * kCoefThreads + (int)threadIdx.x);
     else if (g.n_pfw > 0) coef_by_warp(g, s, c, (int)(blockIdx.x * (kCoefThreads / 32) + (threadIdx.x >> 5)));
     else coef_by_bus(g, s, c, (int)(blockIdx.x * kCoefThreads + threadIdx.x));
@@ -2342,6 +2358,8 @@ int blocks_for(int64_t n, int t) { return (int)((n + t - 1) / t); }
 // Newton power flow over several grids of one topology: item blockIdx.y
 // ---------------------------------------------------------------------------
 __global__ void k_pf_eval_batch(PfBatch B) {
+    pdl_wait();
+    pdl_trigger();
     const PfBatchItem& it = B.it[blockIdx.y];
     k_pf_eval_body(it.g, it.s, it.x, it.A, it.jpv, it.umax, it.umax + 1, 1);
 }
@@ -2350,6 +2368,8 @@ __global__ void k_pf_prep_batch(PfBatch B) {
     pf_prep_body(it.g, it.s, it.A, it.umax, nullptr, 1);
 }
 __global__ void __launch_bounds__(32 * kPfWarps) k_pf_eval_warp_batch(PfBatch B) {
+    pdl_wait();
+    pdl_trigger();
     const PfBatchItem& it = B.it[blockIdx.y];
     pf_eval_warp_body(it.g, it.s, it.x, it.A, it.jpv, it.umax, it.umax + 1, 1);
 }
@@ -2362,6 +2382,8 @@ __global__ void k_batch_status(PfBatch B, double* out) {
 }
 
 __global__ void k_newton_update_batch(PfBatch B) {
+    pdl_wait();
+    pdl_trigger();
     const PfBatchItem& it = B.it[blockIdx.y];
     k_newton_update_body(it.g, it.s, it.x);
 }
@@ -2406,12 +2428,16 @@ __global__ void k_tail_tri_batch(TriBatch B) {
 }
 
 __global__ void k_line_values_batch(const __grid_constant__ Solve1Batch B) {
+    pdl_wait();
+    pdl_trigger();
     line_values_body(B.g[blockIdx.y], false, B.g[blockIdx.y].line);
 }
 
 template <int NT>
 __global__ void __launch_bounds__(NT, kLineRegs / NT)
     k_solve1_batch(const __grid_constant__ Solve1Batch B, int use_tail) {
+    pdl_wait();
+    pdl_trigger();
     k_solve1_body<NT>(B.g[blockIdx.x], B.x[blockIdx.x], B.x[blockIdx.x], false, use_tail);
 }
 
@@ -2431,8 +2457,8 @@ static unsigned prep_blocks(const PfGrid& g) {
     return (unsigned)(b < 1 ? 1 : (b > 1024 ? 1024 : b));
 }
 void launch_pf_prep(const PfGrid& g, const PfState& s, double* A, unsigned long long* umax, int* err, bool zero,
-                    cudaStream_t st) {
-    k_pf_prep<<<prep_blocks(g), 256, 0, st>>>(g, s, A, umax, err, zero ? 1 : 0);
+                    bool chained, cudaStream_t st) {
+    launch_pdl(chained, k_pf_prep, dim3(prep_blocks(g)), dim3(256), 0, st, g, s, A, umax, err, zero ? 1 : 0);
 }
 void launch_pf_prep_batch(const PfBatch& B, cudaStream_t st) {
     if (B.n > 0) k_pf_prep_batch<<<dim3(prep_blocks(B.it[0].g), (unsigned)B.n), 256, 0, st>>>(B);
@@ -2441,10 +2467,11 @@ void launch_pf_prep_batch(const PfBatch& B, cudaStream_t st) {
 void launch_pf_eval(const PfGrid& g, const PfState& s, double* gres, double* A, double* jpv,
                     unsigned long long* gmax, unsigned long long* jmax, bool want_jac, cudaStream_t st) {
     if (g.n_pfw > 0)
-        k_pf_eval_warp<<<(g.n_pfw + kPfWarps - 1) / kPfWarps, 32 * kPfWarps, 0, st>>>(g, s, gres, A, jpv, gmax, jmax,
-                                                                                   want_jac);
+        launch_pdl(true, k_pf_eval_warp, dim3((g.n_pfw + kPfWarps - 1) / kPfWarps), dim3(32 * kPfWarps), 0, st, g, s,
+                   gres, A, jpv, gmax, jmax, want_jac ? 1 : 0);
     else if (g.n_bus > 0)
-        k_pf_eval<<<blocks_for(g.n_bus, 64), 64, 0, st>>>(g, s, gres, A, jpv, gmax, jmax, want_jac);
+        launch_pdl(true, k_pf_eval, dim3(blocks_for(g.n_bus, 64)), dim3(64), 0, st, g, s, gres, A, jpv, gmax, jmax,
+                   want_jac ? 1 : 0);
 }
 
 cudaError_t launch_jac_ad(const PfGrid& g, const PfState& s, const int* col_th, const int* col_v, const int* col_pg,
@@ -2456,8 +2483,8 @@ cudaError_t launch_jac_ad(const PfGrid& g, const PfState& s, const int* col_th, 
     return cudaGetLastError();
 }
 
-void launch_newton_update(const PfGrid& g, const PfState& s, const double* dx, cudaStream_t st) {
-    if (g.n_bus > 0) k_newton_update<<<blocks_for(g.n_bus, 128), 128, 0, st>>>(g, s, dx);
+void launch_newton_update(const PfGrid& g, const PfState& s, const double* dx, bool chained, cudaStream_t st) {
+    if (g.n_bus > 0) launch_pdl(chained, k_newton_update, dim3(blocks_for(g.n_bus, 128)), dim3(128), 0, st, g, s, dx);
 }
 
 // L2 prefetch of read-only arrays: one bulk prefetch of up to kPrefetchChunk bytes
@@ -2663,7 +2690,8 @@ void launch_build_tail(int T, int t0, const int* pos, const double* A, const dou
 
 void launch_line_values(const LineGrid& g, bool transposed_too, cudaStream_t st) {
     if (g.n_line > 0)
-        k_line_values<<<dim3((unsigned)blocks_for(g.n_line, 256), transposed_too ? 2u : 1u), 256, 0, st>>>(g);
+        launch_pdl(true, k_line_values, dim3((unsigned)blocks_for(g.n_line, 256), transposed_too ? 2u : 1u), dim3(256), 0,
+                   st, g);
 }
 
 void launch_adjoint_rhs(const PfGrid& g, const PfState& s, const AdjData& a, cudaStream_t st) {
@@ -2699,20 +2727,21 @@ cudaError_t launch_dir1(const DirGrid& g, const LineGrid& s, const DirLaunch& L,
     return cudaGetLastError();
 }
 
-cudaError_t launch_solve1(const LineGrid& g, const double* x, double* out, bool trans, bool use_tail,
+cudaError_t launch_solve1(const LineGrid& g, const double* x, double* out, bool trans, bool use_tail, bool chained,
                           cudaStream_t st) {
     const size_t smem = solve1_smem(g.n_x, g.T, use_tail);
-    if (line_threads(g.n_x) == 256) k_solve1<256><<<1, 256, smem, st>>>(g, x, out, trans, use_tail ? 1 : 0);
-    else k_solve1<512><<<1, 512, smem, st>>>(g, x, out, trans, use_tail ? 1 : 0);
-    return cudaGetLastError();
+    const bool small = line_threads(g.n_x) == 256;
+    return launch_pdl(chained, small ? k_solve1<256> : k_solve1<512>, dim3(1), dim3(small ? 256 : 512), smem, st, g, x,
+                      out, trans ? 1 : 0, use_tail ? 1 : 0);
 }
 
 int dirs_cta_slots() { return kDirCtasPerSm * num_sms(); }
 int dirs_batch_slots(int threads) { return dirs_batch_ctas_per_sm(threads) * num_sms(); }
 
-void launch_adjoint_coef(const PfGrid& g, const PfState& s, const CoefData& c, cudaStream_t st) {
+void launch_adjoint_coef(const PfGrid& g, const PfState& s, const CoefData& c, bool chained, cudaStream_t st) {
     const int n_coef = g.n_pfw > 0 ? blocks_for(g.n_pfw, kCoefThreads / 32) : blocks_for(g.n_bus, kCoefThreads);
-    k_adjoint_coef<<<n_coef + blocks_for(g.n_bus, kCoefThreads), kCoefThreads, 0, st>>>(g, s, c, n_coef);
+    launch_pdl(chained, k_adjoint_coef, dim3(n_coef + blocks_for(g.n_bus, kCoefThreads)), dim3(kCoefThreads), 0, st, g, s, c,
+               n_coef);
 }
 
 void launch_scatter_rows(int n_rows, int N, const int* map, const double* src, int64_t lds, double* dst,
@@ -2723,19 +2752,20 @@ void launch_scatter_rows(int n_rows, int N, const int* map, const double* src, i
 
 void launch_pf_eval_batch(const PfBatch& B, cudaStream_t st) {
     if (B.n > 0 && B.it[0].g.n_pfw > 0)
-        k_pf_eval_warp_batch<<<dim3((unsigned)((B.it[0].g.n_pfw + kPfWarps - 1) / kPfWarps), (unsigned)B.n),
-                               32 * kPfWarps, 0, st>>>(B);
+        launch_pdl(true, k_pf_eval_warp_batch,
+                   dim3((unsigned)((B.it[0].g.n_pfw + kPfWarps - 1) / kPfWarps), (unsigned)B.n), dim3(32 * kPfWarps), 0, st, B);
     else if (B.n > 0 && B.max_bus > 0)
-        k_pf_eval_batch<<<dim3((unsigned)blocks_for(B.max_bus, 64), (unsigned)B.n), 64, 0, st>>>(B);
+        launch_pdl(true, k_pf_eval_batch, dim3((unsigned)blocks_for(B.max_bus, 64), (unsigned)B.n), dim3(64), 0, st, B);
 }
 
 void launch_batch_status(const PfBatch& B, double* out, cudaStream_t st) {
     if (B.n > 0) k_batch_status<<<1, 32, 0, st>>>(B, out);
 }
 
-void launch_newton_update_batch(const PfBatch& B, cudaStream_t st) {
+void launch_newton_update_batch(const PfBatch& B, bool chained, cudaStream_t st) {
     if (B.n > 0 && B.max_bus > 0)
-        k_newton_update_batch<<<dim3((unsigned)blocks_for(B.max_bus, 128), (unsigned)B.n), 128, 0, st>>>(B);
+        launch_pdl(chained, k_newton_update_batch, dim3((unsigned)blocks_for(B.max_bus, 128), (unsigned)B.n), dim3(128), 0,
+                   st, B);
 }
 
 cudaError_t launch_refactor_batch(const RfBatch& B, const int* lev_ptr_host, const int64_t* tgt_lev_ptr_host,
@@ -2791,11 +2821,14 @@ void launch_tail_tri_batch(const TriBatch& B, cudaStream_t st) {
 cudaError_t launch_solve1_batch(const Solve1Batch& B, bool use_tail, int n_x, int T, cudaStream_t st) {
     if (B.n <= 0) return cudaSuccess;
     const int nl = B.g[0].n_line;      // one topology: the same for every item
-    if (nl > 0) k_line_values_batch<<<dim3((unsigned)blocks_for(nl, 256), (unsigned)B.n), 256, 0, st>>>(B);
-    const size_t smem = solve1_smem(n_x, T, use_tail);
-    if (line_threads(n_x) == 256) k_solve1_batch<256><<<B.n, 256, smem, st>>>(B, use_tail ? 1 : 0);
-    else k_solve1_batch<512><<<B.n, 512, smem, st>>>(B, use_tail ? 1 : 0);
-    return cudaGetLastError();
+    if (nl > 0) {
+        const cudaError_t e = launch_pdl(true, k_line_values_batch, dim3((unsigned)blocks_for(nl, 256), (unsigned)B.n),
+                                         dim3(256), 0, st, B);
+        if (e != cudaSuccess) return e;
+    }
+    const bool small = line_threads(n_x) == 256;
+    return launch_pdl(nl > 0, small ? k_solve1_batch<256> : k_solve1_batch<512>, dim3((unsigned)B.n),
+                      dim3(small ? 256 : 512), solve1_smem(n_x, T, use_tail), st, B, use_tail ? 1 : 0);
 }
 
 void launch_gather_rows(int n_rows, int N, const int* map, const double* src, int64_t lds, double* dst,

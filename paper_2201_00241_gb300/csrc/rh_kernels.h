@@ -233,13 +233,15 @@ inline cudaError_t launch_pdl(bool pdl, void (*kern)(KArgs...), dim3 grid, dim3 
 void launch_injections(const PfGrid& g, const PfState& s, cudaStream_t st);
 // residual (internal order) and/or Jacobian values; gmax / jmax receive
 // max |g| and max |J_x| as ordered bit patterns (zeroed by the caller).
+// `chained`, here and below: the operation before it on `st` is a kernel, and the launch is
+// scheduled with it (see above); launch_pf_eval and launch_line_values always follow one.
 // Before launch_pf_eval: sin and cos of every bus angle into s.sc and, with zero,
 // A (nnz_a slots), the two maxima and *err (if given) cleared.
 void launch_pf_prep(const PfGrid& g, const PfState& s, double* A, unsigned long long* umax, int* err, bool zero,
-                    cudaStream_t st);
+                    bool chained, cudaStream_t st);
 void launch_pf_eval(const PfGrid& g, const PfState& s, double* gres, double* A, double* jpv,
                     unsigned long long* gmax, unsigned long long* jmax, bool want_jac, cudaStream_t st);
-void launch_newton_update(const PfGrid& g, const PfState& s, const double* dx, cudaStream_t st);
+void launch_newton_update(const PfGrid& g, const PfState& s, const double* dx, bool chained, cudaStream_t st);
 // Coloured forward-mode Jacobian (section 4.2.2): the injections evaluated on
 // dual numbers whose tangents are the seed colours (col_th, col_v, col_pg per
 // bus), in chunks of tangents; writes the J_x slots of A (and max |J_x| into
@@ -342,7 +344,7 @@ struct LineGrid {
 };
 void launch_line_values(const LineGrid& g, bool transposed_too, cudaStream_t st);
 int line_threads(int n_x);
-cudaError_t launch_solve1(const LineGrid& g, const double* x, double* out, bool trans, bool use_tail,
+cudaError_t launch_solve1(const LineGrid& g, const double* x, double* out, bool trans, bool use_tail, bool chained,
                           cudaStream_t st);          // out may be x
 // Directions of a launch with one direction per CTA and x in shared memory (L.N CTAs;
 // direction c's rows at V + c * (zero_row + 1) and T likewise): SpMul to the U sweep, the
@@ -408,7 +410,7 @@ cudaError_t launch_refactor_batch(const RfBatch& B, const int* lev_ptr_host, con
 // the dense tail's triangles of the single solves (L, and U with columns scaled by 1/u_jj)
 void launch_tail_tri_batch(const TriBatch& B, cudaStream_t st);
 cudaError_t launch_solve1_batch(const Solve1Batch& B, bool use_tail, int n_x, int T, cudaStream_t st);
-void launch_newton_update_batch(const PfBatch& B, cudaStream_t st);
+void launch_newton_update_batch(const PfBatch& B, bool chained, cudaStream_t st);
 
 int dense_tile(int n);
 cudaError_t launch_potrf(int n, double* A, int64_t lda, int* info, double* y, cudaStream_t s);
@@ -445,7 +447,7 @@ struct CoefData {
     const double* jptv;
     double* grad;
 };
-void launch_adjoint_coef(const PfGrid& g, const PfState& s, const CoefData& c, cudaStream_t st);
+void launch_adjoint_coef(const PfGrid& g, const PfState& s, const CoefData& c, bool chained, cudaStream_t st);
 
 // permutation helpers between external (x, p) order and the internal rows
 void launch_gather_rows(int n_rows, int N, const int* map, const double* src, int64_t lds, double* dst,
