@@ -478,7 +478,7 @@ def measure_per_block(lg, H, sptr, reps=5):
     blocks()
     t = _event_ms(blocks, reps)
     return {"hvp_per_s": lg.n_p / (t * 1e-3), "ms": t, "blocks": -(-lg.n_p // BLOCK_N),
-            "note": "HVP only (state resident): rh_hessian, one k_dirs launch per block of 256 columns"}
+            "note": "HVP only (state resident): rh_hessian, one direction launch per block of 256 columns"}
 
 
 def measure_plain_paths(lg, n_single=32, reps=3):

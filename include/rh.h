@@ -264,8 +264,9 @@ rh_status rh_batch_hessvec(int32_t n_items, const rh_hv_item *items, int32_t wid
  *                items than threads / 2 splits each row's dot product over up
  *                to split_lanes adjacent lanes (a power of two, 1 = no split, at
  *                most 32); 0 takes 32.
- * With all three 0 the items on the largest grids may run one direction per CTA
- * (512 threads, an SM each) beside the others.
+ * With width 0 and the defaults of the other two (0, or 384 and 32) the items on
+ * the largest grids may run one direction per CTA (512 threads, an SM each)
+ * beside the others.
  * RH_EINVAL for any other value (checked before anything else, also when
  * n_items is 0).  Every configuration computes each item's HW up to rounding.
  * rh_batch_hessvec(n, items, width, stream) is this call with {width, 0, 0}.

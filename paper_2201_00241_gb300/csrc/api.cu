@@ -1972,7 +1972,7 @@ rh_status rh_batch_hessvec_cfg(int32_t n_items, const rh_hv_item* items, const r
         int n = std::min(rh::kMaxBatch, n_items - first);
         BatchPlan P;
         std::fill(P.alone, P.alone + n, false);
-        if (width == 0) plan_batch(items + first, n, threads, !cfg->threads && !cfg->split_lanes, P);
+        if (width == 0) plan_batch(items + first, n, threads, threads == 384 && ks_cap == 32, P);
         const bool alone = std::find(P.alone, P.alone + n, true) != P.alone + n;
         B->n_items = 0;
         B->cta_ptr[0] = 0;
