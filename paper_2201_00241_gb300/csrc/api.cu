@@ -809,7 +809,10 @@ int nblk(int n, int t) { return (n + t - 1) / t; }
 // gets all its CTAs into the slots at once.  One CTA a direction instead, whatever the
 // batch, puts a batch of many directions through the slots in several waves of the
 // latency-bound sweeps: a round of 15 requests (118 to 9241 buses, 1912 directions) took
-// 5.6 ms, 8 x 64 directions on the 1354-bus grid 0.92 ms.
+// 5.6 ms, 8 x 64 directions on the 1354-bus grid 0.92 ms.  A CTA with an SM to itself takes
+// kSole x t(D) (one product an SM: 281 us for 360 at 1354 buses, 571 for 744 at 2869), so
+// fewer CTAs of more directions can end sooner: 8 x 64 directions at 1354 buses 488 us in 256
+// CTAs of 2, 479 in 128 of 4.
 //
 // The items on the largest grids may run one direction per CTA with x in shared memory
 // instead (k_dir1_batch, an SM each, t(1) x kAlone), the others filling the SMs it leaves
@@ -824,7 +827,7 @@ struct BatchPlan {
     bool alone[rh::kMaxBatch];
 };
 void plan_batch(const rh_hv_item* items, int n, int threads, bool may_alone, BatchPlan& P) {
-    constexpr double kLevelUs = 1.1, kRowUs = 0.78e-3, kFlopUs = 0.3e-3, kAlone = 0.36;
+    constexpr double kLevelUs = 1.1, kRowUs = 0.78e-3, kFlopUs = 0.3e-3, kAlone = 0.36, kSole = 0.77;
     const int slots = rh::dirs_batch_slots(threads), per_sm = rh::dirs_batch_ctas_per_sm(threads), n_sm = slots / per_sm;
     std::vector<double> a(n), b(n);
     std::vector<int> cap(n);
@@ -839,8 +842,8 @@ void plan_batch(const rh_hv_item* items, int n, int threads, bool may_alone, Bat
         cap[k] = T > 1 ? std::max(1, rh::dirs_tail_cap() / T) : 256;
         cap[k] = std::min(std::min(cap[k], 256), std::max(1, items[k].N));
     }
-    // the items outside `alone`: their time on `room` slots (0: none), and G
-    auto spread = [&](const bool* alone, int room, int* G) {
+    // the items outside `alone`: their time on `room` slots at the rates of full SMs, and G
+    auto fill = [&](const bool* alone, int room, int* G) {
         double lo = 0.0, hi = 0.0;
         for (int k = 0; k < n; k++) {
             G[k] = 0;
@@ -866,6 +869,13 @@ void plan_batch(const rh_hv_item* items, int n, int threads, bool may_alone, Bat
         // more CTAs than slots even at the caps: further waves
         const int64_t all = ctas(hi);
         return hi * (double)((all + room - 1) / room);
+    };
+    // the same, or one CTA an SM where that ends sooner
+    auto spread = [&](const bool* alone, int room, int* G) {
+        int H[rh::kMaxBatch];
+        const double two = fill(alone, room, G), one = room >= per_sm ? kSole * fill(alone, room / per_sm, H) : two;
+        if (one < two) std::copy(H, H + n, G);
+        return std::min(one, two);
     };
     std::fill(P.alone, P.alone + n, false);
     double best = spread(P.alone, slots, P.G);
