@@ -369,9 +369,10 @@ rh_status rh_fp64_fma_rate(int32_t device, int32_t ctas_per_sm, int32_t threads_
 
 /*
  * Solve J_x X = R (trans = 0) or J_x^T X = R (trans = 1) with the current
- * device factors (after rh_adjoint or rh_refactor), in place.  R is n_x x nrhs,
- * column-major, leading dimension ldr >= n_x, indexed like x.  These are the
- * batched sparse solves of Algorithm 2 on their own.
+ * device factors (after rh_adjoint or rh_refactor; after rh_powerflow or
+ * rh_batch_powerflow those of the grid's last Newton step), in place.  R is
+ * n_x x nrhs, column-major, leading dimension ldr >= n_x, indexed like x.  These
+ * are the batched sparse solves of Algorithm 2 on their own.
  */
 rh_status rh_solve(rh_grid *grid, double *R, int64_t ldr, int32_t nrhs, int32_t trans,
                    void *stream, uint32_t flags);

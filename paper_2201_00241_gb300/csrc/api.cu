@@ -132,6 +132,9 @@ struct rh_grid {
     size_t stage_n = 0;
 
     bool adjoint_ready = false;
+    // the last factors are a Newton step's: Ad, Atd and the tail's transposed triangles are
+    // behind them (rh_solve takes them from the line arrays)
+    bool copies_behind = false;
     // batched Newton (rh_batch_powerflow): the grid's identity and structure, the
     // captured per-iteration graphs of batches led by this grid, keyed by the items'
     // identities and the set of items still iterating, and a status buffer
@@ -509,7 +512,7 @@ rh_status assemble(rh_grid* g, int method, double* gres, cudaStream_t s, bool ch
 
 // From the current LU: the direction kernel's unit-diagonal factors and J_p, the dense
 // tail's triangles, and the single solves' line arrays (enqueue only).  newton: only what a
-// Newton step reads.
+// Newton step reads (rh_solve then makes the direction kernel's from it: copies_behind).
 void enqueue_factor_copies(rh_grid* g, cudaStream_t s, bool newton = false) {
     const auto& S = g->S;
     const bool line = g->n_line >= 0;
@@ -566,6 +569,7 @@ rh_status enqueue_factor(rh_grid* g) {
 rh_status assemble_and_factor(rh_grid* g) {
     rh_status st = enqueue_factor(g);
     if (st) return st;
+    g->copies_behind = false;
     return check_err_flag(g);
 }
 
@@ -1411,6 +1415,7 @@ rh_status rh_powerflow(rh_grid* g, const double* x0, double tol, int32_t max_ite
         if (res <= tol) { out = RH_OK; break; }
         if (it >= max_iter || !std::isfinite(res)) break;
         RH_CUDA(cudaGraphLaunch(g->nt_fac_exec, s));
+        g->copies_behind = g->n_line >= 0;
         st = check_err_flag(g);
         if (st) return st;
         RH_CUDA(cudaGraphLaunch(g->nt_step_exec, s));
@@ -1679,7 +1684,10 @@ rh_status rh_batch_powerflow(int32_t n_items, rh_grid* const* grids, const doubl
         st = run(mask, 1);
         if (st) return st;
         for (int i = 0; i < n_items; i++)
-            if (mask & (1u << i)) it[i]++;
+            if (mask & (1u << i)) {
+                it[i]++;
+                grids[i]->copies_behind = grids[i]->n_line >= 0;
+            }
     }
     rh_status worst = RH_OK;
     for (int i = 0; i < n_items; i++) {
@@ -1713,6 +1721,7 @@ rh_status rh_adjoint(rh_grid* g, double* F, double* lambda, double* grad) {
         if (st) return st;
     }
     RH_CUDA(cudaGraphLaunch(g->adj_exec, s));
+    g->copies_behind = false;
     if (lambda) {
         rh::launch_gather_rows(S.n_x, 1, g->xmap, g->lam, 1, g->xbuf, S.n_x, 1.0, S.n_x, s);
         RH_CUDA(cudaMemcpyAsync(lambda, g->xbuf, S.n_x * sizeof(double), cudaMemcpyDeviceToHost, s));
@@ -1775,6 +1784,7 @@ rh_status rh_reduced_hessian(rh_grid* g, double* H, int64_t ldh, double* F, doub
         RH_CUDA(cudaStreamWaitEvent(g->stream, g->ev_user, 0));
     }
     RH_CUDA(cudaGraphLaunch(g->hess_exec, g->stream));
+    g->copies_behind = false;
     if (host)
         RH_CUDA(cudaMemcpy2DAsync(H, ldh * sizeof(double), Hd, lh * sizeof(double), np * sizeof(double), np,
                                   cudaMemcpyDeviceToHost, g->stream));
@@ -2138,6 +2148,13 @@ rh_status rh_solve(rh_grid* g, double* R, int64_t ldr, int32_t nrhs, int32_t tra
                                   S.n_x * sizeof(double), nrhs, cudaMemcpyHostToDevice, s));
         Rd = g->stage_in;
         lr = S.n_x;
+    }
+    // a captured solve may be replayed after any later factorisation: it always brings the copies up
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (g->n_line >= 0) RH_CUDA(cudaStreamIsCapturing(s, &cs));
+    if (g->copies_behind || cs != cudaStreamCaptureStatusNone) {
+        rh::LineCopies o = {g->tail_pos, g->Ad, g->Atd, g->triLd, g->triUd, g->triUtd, g->triLtd};
+        RH_CUDA(rh::launch_copies_from_lines(g->s1(), o, rh::solve1_mode(S.n_x, S.n_x - S.t0) == 2, s));
     }
     rh::launch_scatter_rows(S.n_x, nrhs, g->xmap, Rd, lr, g->V, nrhs, 1.0, S.n_x, s);
     // unit-diagonal factors (J_x = D L'' U'): D^-1 R in, or D^-1 out for the transpose

@@ -1974,6 +1974,47 @@ __global__ void k_line_values(const __grid_constant__ LineGrid g) {
     line_values_body(g, blockIdx.y != 0, blockIdx.y ? g.tline : g.line);
 }
 
+// The factor copies that a Newton step leaves out (see enqueue_factor_copies), from those it
+// makes: entry i of `line` is minus L'' or U' at position map[i], the tail's block is in
+// triLd and triUd, or, where every level is swept (use_tail 0), in `line` too.  Writes what
+// k_transpose_values and k_build_tail write from the same factors (Ad, Atd and the tail's
+// triangles; inside the tail up to the order of two multiplications).  A holds the next
+// Jacobian by then.
+__global__ void k_copies_from_lines(const __grid_constant__ LineGrid g, const __grid_constant__ LineCopies o,
+                                    int use_tail) {
+    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int T = g.T, t0 = g.t0;
+    auto lower = [&](int r, int c) { return c * (T - 1) - c * (c - 1) / 2 + (r - c - 1); };   // r > c
+    auto upper = [&](int r, int c) { return c * (c - 1) / 2 + r; };                           // r < c
+    auto put = [&](int p, double v) {
+        o.Ad[p] = v;
+        o.Atd[g.tpos[p]] = v;
+    };
+    if (i < g.n_line) {
+        const int m = g.map[i];
+        if (m < 0) return;
+        const double v = -g.line[i];
+        put(m, v);
+        const int r = g.arow[m] - t0, c = g.col[m] - t0;
+        if (use_tail || r < 0 || c < 0) return;
+        (r > c ? o.triLd[lower(r, c)] : o.triUd[upper(r, c)]) = v;
+        (r > c ? o.triLtd[upper(c, r)] : o.triUtd[lower(c, r)]) = v;
+        return;
+    }
+    i -= g.n_line;
+    if (i < g.n_x) {
+        put(g.diagpos[i], 1.0);
+        return;
+    }
+    i -= g.n_x;
+    if (!use_tail || i >= (int64_t)T * T) return;
+    const int r = (int)(i / T), c = (int)(i % T), p = o.tail_pos[i];
+    if (r == c) return;
+    const double v = r > c ? g.triLd[lower(r, c)] : g.triUd[upper(r, c)];
+    (r > c ? o.triLtd[upper(c, r)] : o.triUtd[lower(c, r)]) = v;
+    if (p >= 0) put(p, v);
+}
+
 // One right-hand side, one CTA, x held in shared memory for the whole sweep
 // (Newton steps and the first-order adjoint).  Dynamic shared memory holds
 // X[n_x] | a zero | the packed tail triangle (use_tail) | kSolve1Part doubles of scratch
@@ -2692,6 +2733,12 @@ void launch_line_values(const LineGrid& g, bool transposed_too, cudaStream_t st)
     if (g.n_line > 0)
         launch_pdl(true, k_line_values, dim3((unsigned)blocks_for(g.n_line, 256), transposed_too ? 2u : 1u), dim3(256), 0,
                    st, g);
+}
+
+cudaError_t launch_copies_from_lines(const LineGrid& g, const LineCopies& o, bool use_tail, cudaStream_t st) {
+    const int64_t n = (int64_t)g.n_line + g.n_x + (use_tail ? (int64_t)g.T * g.T : 0);
+    if (n > 0) k_copies_from_lines<<<blocks_for(n, 256), 256, 0, st>>>(g, o, use_tail ? 1 : 0);
+    return cudaGetLastError();
 }
 
 void launch_adjoint_rhs(const PfGrid& g, const PfState& s, const AdjData& a, cudaStream_t st) {

@@ -343,6 +343,12 @@ struct LineGrid {
     const double *triLd, *triUd, *triUtd, *triLtd;
 };
 void launch_line_values(const LineGrid& g, bool transposed_too, cudaStream_t st);
+// The direction kernel's unit-diagonal factors from the line values and the tail's triangles
+struct LineCopies {
+    const int* tail_pos;
+    double *Ad, *Atd, *triLd, *triUd, *triUtd, *triLtd;
+};
+cudaError_t launch_copies_from_lines(const LineGrid& g, const LineCopies& o, bool use_tail, cudaStream_t st);
 int line_threads(int n_x);
 cudaError_t launch_solve1(const LineGrid& g, const double* x, double* out, bool trans, bool use_tail, bool chained,
                           cudaStream_t st);          // out may be x
