@@ -344,11 +344,15 @@ rh_status rh_reduced_hessian_times(const rh_grid *grid, float *ms);
  *                the four sweeps (2 nnz(L), 2 (nnz(U) - n_x) each) and the
  *                projection (eq. 13: 8 per incidence and per bus, 4 per
  *                slack-gradient entry, 1 per Pg row)
- *   executed     what the kernels issue for those launches: the forward L
+ *   executed     what the kernels issue for those launches (padding lanes and
+ *                sums of partial sums not counted): no multiplications in SpMul
+ *                (it scatters columns of J_p), the dense tail as a full
+ *                triangle; with more than 2 n_sm directions the forward L
  *                sweep over each CTA's reach only (the rows W = I can make
- *                nonzero for that CTA's directions), the last L^T sweep over
- *                the rows SpMulAdd reads, no multiplications in SpMul (it
- *                scatters columns of J_p), the dense tail as a full triangle
+ *                nonzero for that CTA's directions) and the last L^T sweep over
+ *                the rows SpMulAdd reads.  Up to 2 n_sm, where each direction
+ *                has a CTA and x fits in its shared memory, all rows in every
+ *                sweep
  *   n_sm         SMs of the device (it fixes the CTA split); 0 takes the grid's
  *                device, required > 0 on a symbolic-only grid.
  * Host only, no device work.

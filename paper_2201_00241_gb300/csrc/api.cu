@@ -74,7 +74,7 @@ struct rh_grid {
     int *sbr_ptr = nullptr, *sbr_maxext = nullptr;
     int4* sbr_slot = nullptr;
     int n_sbr = 0;
-    // k_solve1's schedules (LineSched) and line arrays; n_line < 0: its descriptors do not fit
+    // k_solve1's schedules (LineSched) and line arrays; n_line < 0: it has none (line_fits)
     int4 *line_up = nullptr, *line_down = nullptr;
     int *line_col = nullptr, *line_map = nullptr;
     double *line_val = nullptr, *line_tval = nullptr;
@@ -317,18 +317,38 @@ std::vector<int> tree_column_order(const rh::Symbolic& S) {
     return cm;
 }
 
+// Lanes of a row, as a power of two: the two rows of a bus share a warp
+constexpr int line_lg_max(bool two) { return two ? 4 : 5; }
+
+// Whether the single solves and k_dir1 have their schedules: x fits in one CTA's shared
+// memory, and the entries a lane takes of each row (outside the bus, and of the tail's rows
+// outside the tail) fit in a descriptor at the most lanes a row can have.
+bool line_fits(const rh::Symbolic& S) {
+    const int mode = rh::solve1_mode(S.n_x, S.n_x - S.t0);
+    if (mode == 0) return false;
+    for (int k = 0; k < S.n_elim; k++) {
+        const int q = S.q0[k];
+        const bool two = S.nv[k] == 2, tail = mode == 2 && k >= S.tail_bus0;
+        int n = 0;
+        for (int t = S.rowptr[q]; t < S.diagpos[q] && !(tail && S.col[t] >= S.t0); t++) n++;
+        if (!tail) n = std::max(n, S.rowptr[q + 1] - S.diagpos[q] - S.nv[k]);
+        if (n > rh::kLineCntMask << line_lg_max(two)) return false;
+    }
+    return true;
+}
+
 // The steps of a sweep over the levels ptr[l] .. ptr[l + 1] of `slots`, for CTAs of NT
 // threads: the buses of a level by descending number of lanes, side by side (a group
 // starts at a multiple of its size), in rounds of NT, or on one half of the warps and the
 // other in turn where they fit; the level's last round ends in a barrier.  A level's groups are those that cost its busiest sub-partition, or its longest
 // warp, the fewest FP64 instructions (64 cycles each; a shuffle takes as long): at most m
-// entries a lane, for m = 1, 2, 4, ...  False: a row is too long for the descriptors.
+// entries a lane, for m = 1, 2, 4, ...  Every row has to fit (line_fits).
 struct LineHost {
     std::vector<int4> steps;
     std::vector<int> map, col, vt;       // entries' positions in A (-1: a pad) and columns; buses' own entries
     int pad;                             // the pads' column, whose x is 0
 };
-bool line_steps(const std::vector<int>& ptr, const std::vector<int4>& slots, const std::vector<int>& col, bool up,
+void line_steps(const std::vector<int>& ptr, const std::vector<int4>& slots, const std::vector<int>& col, bool up,
                 int flags, int NT, LineHost& L) {
     struct Bus {
         int lg, t;
@@ -345,7 +365,7 @@ bool line_steps(const std::vector<int>& ptr, const std::vector<int4>& slots, con
             for (int t = ptr[l]; t < ptr[l + 1]; t++) {
                 const bool two = slots[t].w >= 0;
                 int lg = 0;
-                while (lg < (two ? 4 : 5) && (m << lg) < slots[t].y) lg++;
+                while (lg < line_lg_max(two) && (m << lg) < slots[t].y) lg++;
                 cur.push_back({lg, t, two});
             }
             std::stable_sort(cur.begin(), cur.end(),
@@ -400,7 +420,6 @@ bool line_steps(const std::vector<int>& ptr, const std::vector<int4>& slots, con
                 cnt = std::max(cnt, (slots[lanes[i].slot].y + (1 << l) - 1) >> l);
                 on = rh::kLineActive;
             }
-            if (cnt > rh::kLineCntMask) return false;
             const int base = (int)L.map.size();
             const int w0 = flags | on | cnt | (lg << rh::kLineWlg) | (k + NT >= lanes.size() ? rh::kLineSync : 0);
             for (int e = 0; e < cnt; e++)
@@ -427,7 +446,6 @@ bool line_steps(const std::vector<int>& ptr, const std::vector<int4>& slots, con
             }
         }
     }
-    return true;
 }
 
 rh_status set_device(const rh_grid* g) {
@@ -1133,16 +1151,15 @@ rh_status rh_grid_create(const rh_grid_desc* d, int32_t device, rh_grid** out) {
             const int mode = rh::solve1_mode(S.n_x, S.n_x - S.t0), NT = rh::line_threads(S.n_x);
             LineHost up, down;
             up.pad = down.pad = S.n_x;
-            bool ok = mode > 0;
-            if (mode == 2) {
-                ok = line_steps(sfp, sfs, S.col, true, 0, NT, up) &&
-                     line_steps(efp, efs, S.col, true, rh::kLineExt, NT, up) &&
-                     line_steps(sbp, sbs, S.col, false, 0, NT, down);
-            } else if (mode == 1) {
-                ok = line_steps(S.flev_ptr, fs, S.col, true, 0, NT, up) &&
-                     line_steps(S.blev_ptr, bs, S.col, false, 0, NT, down);
-            }
-            if (ok) {
+            if (line_fits(S)) {
+                if (mode == 2) {
+                    line_steps(sfp, sfs, S.col, true, 0, NT, up);
+                    line_steps(efp, efs, S.col, true, rh::kLineExt, NT, up);
+                    line_steps(sbp, sbs, S.col, false, 0, NT, down);
+                } else {
+                    line_steps(S.flev_ptr, fs, S.col, true, 0, NT, up);
+                    line_steps(S.blev_ptr, bs, S.col, false, 0, NT, down);
+                }
                 g->n_line_up = (int)(up.steps.size() / NT);
                 g->n_line_down = (int)(down.steps.size() / NT);
                 g->line_off[0] = (int)up.map.size();
@@ -1761,9 +1778,11 @@ rh_status rh_reduced_hessian(rh_grid* g, double* H, int64_t ldh, double* F, doub
     }
     if (!g->hess_exec) {
         // the first launch's reach schedule is built here: the capture cannot allocate
-        rh::ReachSched* rs = nullptr;
-        st = reach_schedule(g, first_launch_ctas(np), &rs);
-        if (st) return st;
+        if (!by_dir1(g, np)) {
+            rh::ReachSched* rs = nullptr;
+            st = reach_schedule(g, first_launch_ctas(np), &rs);
+            if (st) return st;
+        }
         if (!g->stream2) RH_CUDA(cudaStreamCreateWithFlags(&g->stream2, cudaStreamNonBlocking));
         if (!g->ev_fork) RH_CUDA(cudaEventCreateWithFlags(&g->ev_fork, cudaEventDisableTiming));
         if (!g->ev_join) RH_CUDA(cudaEventCreateWithFlags(&g->ev_join, cudaEventDisableTiming));
@@ -1824,7 +1843,11 @@ rh_status rh_reduced_hessian_flops(const rh_grid* g, int32_t n_sm, double* algor
     const int per = (np + slots - 2) / std::max(1, slots - 1);
     const int n_cta2 = rh::dirs_ctas_for(np, slots);
     const int n_cta1 = std::min(n_cta2, std::max(1, (np + std::max(1, per) - 1) / std::max(1, per)));
-    const bool tailed = rh::dirs_tail_fits(T, np, n_cta1) && rh::dirs_tail_fits(T, np, n_cta2);
+    // one direction per CTA (by_dir1): every sweep over all rows, the projection without the
+    // first U'^T level
+    const bool one = np <= slots && line_fits(S);
+    const bool tailed = one ? rh::solve1_mode(S.n_x, T) == 2
+                            : rh::dirs_tail_fits(T, np, n_cta1) && rh::dirs_tail_fits(T, np, n_cta2);
     // FMAs of bus block k in a forward / backward sweep: both rows' parts outside the
     // bus, plus the (v, theta) entry of a PQ bus
     auto fwd_fma = [&](int k) {
@@ -1854,13 +1877,13 @@ rh_status rh_reduced_hessian_flops(const rh_grid* g, int32_t n_sm, double* algor
         if (need[k])
             for (int c : S.colpat[k]) need[c] = 1;
     int64_t l_all = 0, u_all = 0, ut = 0, lt = 0, fold = 0;
-    const bool fold_ut = tailed && S.tail_bus0 > 0;
+    const bool fold_ut = !one && tailed && S.tail_bus0 > 0;
     for (int k = 0; k < sparse_end; k++) {
         l_all += fwd_fma(k);
         u_all += bwd_fma(k);
         if (fold_ut && S.flevel[k] == 0) fold += S.nv[k] == 2 ? 1 : 0;   // done by the projection
         else ut += fwd_fma(k);
-        if (!tailed || need[k]) lt += bwd_fma(k);
+        if (one || !tailed || need[k]) lt += bwd_fma(k);
     }
     // the projection, per direction: 3 + 3 flops per bus, 8 per incidence, 4 per bus next to the
     // slack, 2 n_gref + 1 for the slack term, 1 per Pg row, 2 per PQ bus of level 0 (the folded
@@ -1869,14 +1892,15 @@ rh_status rh_reduced_hessian_flops(const rh_grid* g, int32_t n_sm, double* algor
     const double nnz_jp = (double)S.jp_col.size();
     const double l2 = proj + 2.0 * (ut + ext + 2 * tail + lt) + 2.0 * nnz_jp;
     // launch 1 (identity W): the L sweep over each CTA's reach, the buses of its J_p columns and
-    // their ancestors in the sparse part (all buses without the dense tail), then the tail's
-    // external phase, the two tail solves and the U sweep
+    // their ancestors in the sparse part (all buses without the dense tail or with one
+    // direction per CTA), then the tail's external phase, the two tail solves and the U sweep
     double l1 = 0.0;
     std::vector<int> bpos(S.n_x);
     for (int k = 0; k < S.n_elim; k++)
         for (int t = 0; t < S.nv[k]; t++) bpos[S.q0[k] + t] = k;
     std::vector<char> in(S.n_elim);
-    for (int c = 0; c < n_cta1 && np > 0; c++) {
+    if (one) l1 = (double)np * 2.0 * (l_all + ext + 2 * tail + u_all);
+    for (int c = 0; c < n_cta1 && np > 0 && !one; c++) {
         const int c0 = (int)((int64_t)c * np / n_cta1), c1 = (int)((int64_t)(c + 1) * np / n_cta1);
         int64_t l = l_all;
         if (tailed) {
