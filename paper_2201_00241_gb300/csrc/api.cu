@@ -248,13 +248,14 @@ struct rh_grid {
     }
     rh::LineGrid s1() const {
         rh::LineGrid g;
-        g.n_x = S.n_x; g.t0 = S.t0; g.T = S.n_x - S.t0;
+        g.n_x = S.n_x; g.t0 = S.t0; g.T = S.n_x - S.t0; g.nnz = (int)S.col.size();
         const double *v = line_val, *t = line_tval;
         const int *up = line_col, *down = line_col + line_off[0];
-        g.up = {n_line_up, line_up, up, v, v + line_off[1]};
-        g.down = {n_line_down, line_down, down, v + line_off[0], v + line_off[2]};
-        g.tup = {n_line_up, line_up, up, t, t + line_off[1]};
-        g.tdown = {n_line_down, line_down, down, t + line_off[0], t + line_off[2]};
+        const int eu = line_off[0], ed = line_off[1] - line_off[0], vu = line_off[2] - line_off[1], vd = n_line - line_off[2];
+        g.up = {n_line_up, eu, vu, line_up, up, v, v + line_off[1]};
+        g.down = {n_line_down, ed, vd, line_down, down, v + line_off[0], v + line_off[2]};
+        g.tup = {n_line_up, eu, vu, line_up, up, t, t + line_off[1]};
+        g.tdown = {n_line_down, ed, vd, line_down, down, t + line_off[0], t + line_off[2]};
         g.n_line = n_line; g.map = line_map; g.arow = arow; g.col = col; g.tpos = tpos; g.diagpos = diagpos;
         g.line = line_val; g.tline = line_tval;
         g.A = A; g.invdiag = invdiag;

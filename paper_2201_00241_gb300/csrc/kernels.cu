@@ -1858,17 +1858,17 @@ __device__ __forceinline__ void line_ahead(const LineSched& sc, const int4 d, Li
     const int at = d.y + (threadIdx.x & 31);
 #pragma unroll
     for (int k = 0; k < kLinePre; k++)
-        if (k < cnt) {
+        if (k < cnt && inb(at + 32 * k, sc.n_ent)) {
             p.i[k] = sc.col[at + 32 * k];
             p.u[k] = sc.val[at + 32 * k];
         }
-    if (d.z >= 0) p.vt = sc.vt[d.z];
+    if (d.z >= 0 && inb(d.z, sc.n_vt)) p.vt = sc.vt[d.z];
 }
 
 // x_q = b_q - sum v_qc x_c over the schedule's levels; in a bus of two rows the theta row
-// is solved first (FWD) or the v row.
+// is solved first (FWD) or the v row.  X: n_x rows and the pads' zero.
 template <bool FWD, int NT>
-__device__ void line_sweep(const LineSched& sc, double* X) {
+__device__ void line_sweep(const LineSched& sc, double* X, const int n_x) {
     const int n_steps = sc.n;
     if (n_steps <= 0) return;
     const int4* my = sc.steps + threadIdx.x;
@@ -1889,10 +1889,10 @@ __device__ void line_sweep(const LineSched& sc, double* X) {
             const int q = d.x, lg = (w >> kLineLg) & 7, cnt = w & kLineCntMask, wlg = (w >> kLineWlg) & 7;
             const int G = 1 << lg, row = (w & kLineSplit) && (threadIdx.x & G) ? 1 : 0;
             // the first lane of a row starts from its right-hand side
-            double s = q >= 0 && (threadIdx.x & (G - 1)) == 0 ? X[q + row] : 0.0;
+            double s = q >= 0 && (threadIdx.x & (G - 1)) == 0 && inb(q + row, n_x) ? X[q + row] : 0.0;
             double xv[kLinePre];
 #pragma unroll
-            for (int k = 0; k < kLinePre; k++) xv[k] = k < cnt ? X[p.i[k]] : 0.0;
+            for (int k = 0; k < kLinePre; k++) xv[k] = k < cnt && inb(p.i[k], n_x + 1) ? X[p.i[k]] : 0.0;
             // Jumps, not predicates: a predicated-off FP64 instruction still takes its 64 cycles.
             // Unrolled with `if (k < cnt)`, a level of 16-lane rows cost 2000 cycles for any cnt;
             // so it costs 1700, and the two sweeps of the 9241-bus grid 494 k cycles for 580 k.
@@ -1913,12 +1913,13 @@ __device__ void line_sweep(const LineSched& sc, double* X) {
                 double u[4];
 #pragma unroll
                 for (int m = 0; m < 4; m++) {
-                    c[m] = k + m < cnt ? sc.col[at + 32 * m] : 0;
-                    u[m] = k + m < cnt ? sc.val[at + 32 * m] : 0.0;
+                    const bool in = k + m < cnt && inb(at + 32 * m, sc.n_ent);
+                    c[m] = in ? sc.col[at + 32 * m] : 0;
+                    u[m] = in ? sc.val[at + 32 * m] : 0.0;
                 }
 #pragma unroll
                 for (int m = 0; m < 4; m++)
-                    if (k + m < cnt) s = fma(u[m], X[c[m]], s);
+                    if (k + m < cnt && inb(c[m], n_x + 1)) s = fma(u[m], X[c[m]], s);
             }
             auto halve = [&](int o) {
                 const double t = __shfl_down_sync(0xffffffffu, s, 1 << o);
@@ -1933,7 +1934,8 @@ __device__ void line_sweep(const LineSched& sc, double* X) {
                 default: break;
             }
             const double s1 = __shfl_sync(0xffffffffu, s, (threadIdx.x + G) & 31);
-            if (q >= 0 && (threadIdx.x & ((w & kLineSplit ? 2 * G : G) - 1)) == 0) {
+            if (q >= 0 && (threadIdx.x & ((w & kLineSplit ? 2 * G : G) - 1)) == 0 &&
+                inb(w & kLineSplit ? q + 1 : q, n_x)) {
                 if (!(w & kLineSplit)) {
                     X[q] = s;
                 } else if (w & kLineExt) {
@@ -1961,7 +1963,7 @@ __device__ __forceinline__ void line_values_body(const LineGrid& g, bool trans, 
     if (i >= g.n_line) return;
     const int m = g.map[i];
     double v = 0.0;
-    if (m >= 0) {
+    if (m >= 0 && inb(m, g.nnz) && inb(g.tpos[m], g.nnz)) {
         const int r = g.arow[m], c = g.col[m];
         v = trans ? -(g.A[g.tpos[m]] * unit_scale(g.A, g.diagpos, g.invdiag, c, r))
                   : -(g.A[m] * unit_scale(g.A, g.diagpos, g.invdiag, r, c));
@@ -1987,12 +1989,14 @@ __global__ void k_copies_from_lines(const __grid_constant__ LineGrid g, const __
     auto lower = [&](int r, int c) { return c * (T - 1) - c * (c - 1) / 2 + (r - c - 1); };   // r > c
     auto upper = [&](int r, int c) { return c * (c - 1) / 2 + r; };                           // r < c
     auto put = [&](int p, double v) {
+        if (!inb(p, g.nnz) || !inb(g.tpos[p], g.nnz)) return;
         o.Ad[p] = v;
         o.Atd[g.tpos[p]] = v;
     };
     if (i < g.n_line) {
         const int m = g.map[i];
         if (m < 0) return;
+        if (!inb(m, g.nnz)) return;
         const double v = -g.line[i];
         put(m, v);
         const int r = g.arow[m] - t0, c = g.col[m] - t0;
@@ -2033,12 +2037,12 @@ __device__ __forceinline__ void k_solve1_body(const LineGrid& g, const double* x
     for (int q = threadIdx.x; q < g.n_x; q += NT) X[q] = trans ? x[q] : x[q] * g.invdiag[q];
     if (threadIdx.x == 0) X[g.n_x] = 0.0;                  // the pads' column
     __syncthreads();
-    line_sweep<true, NT>(trans ? g.tup : g.up, X);
+    line_sweep<true, NT>(trans ? g.tup : g.up, X, g.n_x);
     if (use_tail) {
         tail_fwd<false>(g, trans ? g.triUtd : g.triLd, X, 1, 0, 1, part, tri);
         tail_bwd<false>(g, trans ? g.triLtd : g.triUd, X, 1, 0, 1, part, tri);
     }
-    line_sweep<false, NT>(trans ? g.tdown : g.down, X);
+    line_sweep<false, NT>(trans ? g.tdown : g.down, X, g.n_x);
     __syncthreads();
     for (int q = threadIdx.x; q < g.n_x; q += NT) out[q] = trans ? X[q] * g.invdiag[q] : X[q];
 }
@@ -2087,12 +2091,12 @@ __device__ __forceinline__ void dir1_body(const DirGrid& g, const LineGrid& s, c
                 if (inb(g.jpt_row[t], g.n_x)) X[g.jpt_row[t]] = -g.jptvd[t];
         }
         __syncthreads();
-        line_sweep<true, NT>(s.up, X);
+        line_sweep<true, NT>(s.up, X, g.n_x);
         if (use_tail) {
             tail_fwd<false>(s, s.triLd, X, 1, 0, 1, part, tri);
             tail_bwd<false>(s, s.triUd, X, 1, 0, 1, part, tri);
         }
-        line_sweep<false, NT>(s.down, X);
+        line_sweep<false, NT>(s.down, X, g.n_x);
         __syncthreads();
     }
     if (!(L.phases & PH_TPROJ)) {
@@ -2164,12 +2168,12 @@ __device__ __forceinline__ void dir1_body(const DirGrid& g, const LineGrid& s, c
     __syncthreads();
     for (int q = threadIdx.x; q < g.n_x; q += NT) X[q] = Y[q];
     __syncthreads();
-    line_sweep<true, NT>(s.tup, X);
+    line_sweep<true, NT>(s.tup, X, g.n_x);
     if (use_tail) {
         tail_fwd<false>(s, s.triUtd, X, 1, 0, 1, part, tri);
         tail_bwd<false>(s, s.triLtd, X, 1, 0, 1, part, tri);
     }
-    line_sweep<false, NT>(s.tdown, X);
+    line_sweep<false, NT>(s.tdown, X, g.n_x);
     __syncthreads();
     double* HW = L.HW + (int64_t)(id - L.col0) * L.ldhw;
     for (int k = threadIdx.x; k < g.n_p; k += NT) {

@@ -327,14 +327,14 @@ constexpr int kLineSync = 1 << 27;    // barrier after the step (its level ends)
 constexpr int kLineSplit = 1 << 28;   // a bus of two rows: a group of lanes for each, side by side
 constexpr int kLineActive = 1 << 30;  // the warp has a bus in this step
 struct LineSched {
-    int n;                            // steps
+    int n, n_ent, n_vt;               // steps, entries and buses' own entries of the line arrays
     const int4* steps;
     const int* col;                   // line arrays: column of each entry (n_x: a pad),
     const double* val;                //   its value negated (0: a pad), and each bus's own
     const double* vt;                 //   off-diagonal entry negated
 };
 struct LineGrid {
-    int n_x, t0, T;
+    int n_x, t0, T, nnz;              // nnz: positions of the pattern of A (index checks)
     LineSched up, down, tup, tdown;   // with L'', U', and with U'^T, L''^T
     int n_line;                       // entries of the line arrays [up | down | up's vt | down's vt]
     const int *map, *arow, *col, *tpos, *diagpos;   // their positions in A (-1: a pad); A's rows, columns, ...
