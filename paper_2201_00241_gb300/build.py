@@ -21,7 +21,7 @@ INCLUDE = os.path.join(os.path.dirname(HERE), "include")
 
 CU = ["kernels.cu", "dense.cu", "api.cu", "peak.cu"]
 CPP = ["symbolic.cpp"]
-HEADERS = ["rh_internal.h", "rh_kernels.h"]
+HEADERS = ["rh_internal.h", "rh_kernels.h", "batch_plan.h"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 

@@ -821,118 +821,24 @@ __global__ void k_rto_apply(int n_p, int n_bus, const int* info, const double* p
 
 int nblk(int n, int t) { return (n + t - 1) / t; }
 
-// CTAs of each item of a batched launch whose width is left to the library.  A CTA of the
-// batched direction kernel with D directions of a grid takes about
-//   t(D) = kLevelUs x (levels of the four sweeps) + (kRowUs + kFlopUs x D) x (flops of a direction),
-// with the SM's CTA slots occupied: a level's chain, the rows' loads, which the directions
-// share, and their arithmetic (fitted on GB300, D = 1 / 2 / 3: 2196 / 2526 / 3013 us on the
-// 9241-bus grid, 744 / 795 / 1001 on 2869 buses, 360 / 401 / 476 on 1354 buses, 119 / 122 /
-// 130 on 118 buses).  The items run side by side, so the launch ends with its slowest CTA:
-// the least T is taken for which every item, at the most directions per CTA that end by T,
-// gets all its CTAs into the slots at once.  One CTA a direction instead, whatever the
-// batch, puts a batch of many directions through the slots in several waves of the
-// latency-bound sweeps: a round of 15 requests (118 to 9241 buses, 1912 directions) took
-// 5.6 ms, 8 x 64 directions on the 1354-bus grid 0.92 ms.  A CTA with an SM to itself takes
-// kSole x t(D) (one product an SM: 281 us for 360 at 1354 buses, 571 for 744 at 2869), so
-// fewer CTAs of more directions can end sooner: 8 x 64 directions at 1354 buses 488 us in 256
-// CTAs of 2, 479 in 128 of 4.
-//
-// The items on the largest grids may run one direction per CTA with x in shared memory
-// instead (k_dir1_batch, an SM each, t(1) x kAlone), the others filling the SMs it leaves
-// and, once its last CTA has started, those that are done.  Their few directions are the
-// longest chains of a mixed batch: next to CTAs of many directions, which keep an SM's FP64
-// pipes busy, they end it.  Of the sets "the items on grids of at least n rows" the one with
-// the least predicted time is taken: the round of 15 requests takes 3.2 ms with none, 1.9
-// ms with the 9241-bus grid (184 directions), 2.3 with 2869 buses and more, 2.2 with 1354
-// buses and more; 8 x 64 directions on the 1354-bus grid take 488 us with none, 509 with all.
-struct BatchPlan {
-    int G[rh::kMaxBatch];                // CTAs (0: no directions, or one per CTA in k_dir1_batch)
-    bool alone[rh::kMaxBatch];
-};
-void plan_batch(const rh_hv_item* items, int n, int threads, bool may_alone, BatchPlan& P) {
-    constexpr double kLevelUs = 1.1, kRowUs = 0.78e-3, kFlopUs = 0.3e-3, kAlone = 0.36, kSole = 0.77;
-    const int slots = rh::dirs_batch_slots(threads), per_sm = rh::dirs_batch_ctas_per_sm(threads), n_sm = slots / per_sm;
-    std::vector<double> a(n), b(n);
-    std::vector<int> cap(n);
+// The split of items whose width is left to the library (batch_plan.h).  may_alone: in
+// the default configuration.
+void plan_batch(const rh_hv_item* items, int n, int threads, bool may_alone, rh::BatchPlan& P) {
+    const int slots = rh::dirs_batch_slots(threads), per_sm = rh::dirs_batch_ctas_per_sm(threads);
+    rh::BatchItem b[rh::kMaxBatch];
     for (int k = 0; k < n; k++) {
         const auto& S = items[k].grid->S;
         const int T = S.n_x - S.t0;
-        const double flops = 4.0 * (double)S.jp_col.size() + 4.0 * (S.nnz_l + S.nnz_u - S.n_x) +
-                             8.0 * (double)S.yj.size();
-        a[k] = kLevelUs * (2.0 * S.n_flev + 2.0 * S.n_blev) + kRowUs * flops;
-        b[k] = kFlopUs * flops;
+        b[k].levels = 2.0 * S.n_flev + 2.0 * S.n_blev;
+        b[k].flops = 4.0 * (double)S.jp_col.size() + 4.0 * (S.nnz_l + S.nnz_u - S.n_x) + 8.0 * (double)S.yj.size();
+        b[k].N = items[k].N;
         // at most 256 directions, and the dense tail's rows in shared memory
-        cap[k] = T > 1 ? std::max(1, rh::dirs_tail_cap() / T) : 256;
-        cap[k] = std::min(std::min(cap[k], 256), std::max(1, items[k].N));
+        b[k].cap = T > 1 ? std::max(1, rh::dirs_tail_cap() / T) : 256;
+        b[k].cap = std::min(std::min(b[k].cap, 256), std::max(1, items[k].N));
+        b[k].n_x = S.n_x;
+        b[k].line = items[k].grid->n_line >= 0 && rh::line_threads(S.n_x) == 512;
     }
-    // the items outside `alone`: their time on `room` slots at the rates of full SMs, and G
-    auto fill = [&](const bool* alone, int room, int* G) {
-        double lo = 0.0, hi = 0.0;
-        for (int k = 0; k < n; k++) {
-            G[k] = 0;
-            if (alone[k] || items[k].N == 0) continue;
-            lo = std::max(lo, a[k] + b[k]);
-            hi = std::max(hi, a[k] + b[k] * cap[k]);
-        }
-        auto ctas = [&](double t) {
-            int64_t sum = 0;
-            for (int k = 0; k < n; k++) {
-                if (alone[k] || items[k].N == 0) continue;
-                const int D = std::max(1, (int)std::min((double)cap[k], std::floor((t - a[k]) / b[k])));
-                G[k] = (items[k].N + D - 1) / D;         // the fewest CTAs with at most D directions
-                sum += G[k];
-            }
-            return sum;
-        };
-        if (ctas(lo) <= room) return lo;
-        for (int it = 0; it < 40; it++) {
-            const double mid = 0.5 * (lo + hi);
-            (ctas(mid) <= room ? hi : lo) = mid;
-        }
-        // more CTAs than slots even at the caps: further waves
-        const int64_t all = ctas(hi);
-        return hi * (double)((all + room - 1) / room);
-    };
-    // the same, or one CTA an SM where that ends sooner
-    auto spread = [&](const bool* alone, int room, int* G) {
-        int H[rh::kMaxBatch];
-        const double two = fill(alone, room, G), one = room >= per_sm ? kSole * fill(alone, room / per_sm, H) : two;
-        if (one < two) std::copy(H, H + n, G);
-        return std::min(one, two);
-    };
-    std::fill(P.alone, P.alone + n, false);
-    double best = spread(P.alone, slots, P.G);
-    if (!may_alone) return;
-    std::vector<int> order;
-    for (int k = 0; k < n; k++)
-        if (items[k].N > 0) order.push_back(k);
-    std::stable_sort(order.begin(), order.end(), [&](int p, int q) { return items[p].grid->S.n_x > items[q].grid->S.n_x; });
-    BatchPlan Q = P;
-    double sm_us = 0.0, longest = 0.0, shortest = 0.0;
-    int64_t dirs = 0;
-    for (size_t i = 0; i < order.size(); i++) {
-        const int k = order[i];
-        const auto& S = items[k].grid->S;
-        if (items[k].grid->n_line < 0 || rh::line_threads(S.n_x) != 512) break;
-        Q.alone[k] = true;
-        shortest = kAlone * (a[k] + b[k]);
-        longest = std::max(longest, shortest);
-        sm_us += shortest * items[k].N;
-        dirs += items[k].N;
-        if (i + 1 < order.size() && items[order[i + 1]].grid->S.n_x == S.n_x) continue;
-        // SMs that the last wave leaves, and when it starts
-        const int last = (int)((dirs - 1) % n_sm) + 1;
-        const double wave = sm_us / (double)dirs, start = wave * (double)((dirs - 1) / n_sm);
-        const bool rest = i + 1 < order.size();
-        const int room = per_sm * (n_sm - last);
-        double t = std::max(start + wave, longest);
-        if (rest) t = room > 0 ? std::max(t, start + spread(Q.alone, room, Q.G)) : t + spread(Q.alone, slots, Q.G);
-        if (t < best) {
-            best = t;
-            P = Q;
-        }
-        std::fill(Q.G, Q.G + n, 0);
-    }
+    rh::BatchPlanner(b, n, slots / per_sm, per_sm, may_alone).plan(P);
 }
 
 }  // namespace
@@ -2015,7 +1921,7 @@ rh_status rh_batch_hessvec_cfg(int32_t n_items, const rh_hv_item* items, const r
     std::unique_ptr<rh::DirBatch> B(new rh::DirBatch());
     for (int first = 0; first < n_items; first += rh::kMaxBatch) {
         int n = std::min(rh::kMaxBatch, n_items - first);
-        BatchPlan P;
+        rh::BatchPlan P;
         std::fill(P.alone, P.alone + n, false);
         if (width == 0) plan_batch(items + first, n, threads, threads == 384 && ks_cap == 32, P);
         const bool alone = std::find(P.alone, P.alone + n, true) != P.alone + n;

@@ -5,6 +5,8 @@
 
 #include <cuda_runtime.h>
 
+#include "batch_plan.h"
+
 namespace rh {
 
 // Phases of the direction kernel (one bit each, executed in this order).
@@ -124,7 +126,6 @@ struct ReachSched {
 
 // Up to kMaxBatch (grid, W block) items of one batched launch, passed by value as
 // the kernel parameter (about 16 KB).
-constexpr int kMaxBatch = 32;
 struct DirBatch {
     int n_items;
     int cta_ptr[kMaxBatch + 1];
