@@ -341,9 +341,10 @@ bool line_fits(const rh::Symbolic& S) {
 // The steps of a sweep over the levels ptr[l] .. ptr[l + 1] of `slots`, for CTAs of NT
 // threads: the buses of a level by descending number of lanes, side by side (a group
 // starts at a multiple of its size), in rounds of NT, or on one half of the warps and the
-// other in turn where they fit; the level's last round ends in a barrier.  A level's groups are those that cost its busiest sub-partition, or its longest
-// warp, the fewest FP64 instructions (64 cycles each; a shuffle takes as long): at most m
-// entries a lane, for m = 1, 2, 4, ...  Every row has to fit (line_fits).
+// other in turn where they fit; the level's last round ends in a barrier.  A level's groups
+// are those that cost its busiest sub-partition, or its longest warp, the fewest FP64
+// instructions (64 cycles each; a shuffle takes as long): at most m entries a lane, for
+// m = 1, 2, 4, ...  Every row has to fit (line_fits).
 struct LineHost {
     std::vector<int4> steps;
     std::vector<int> map, col, vt;       // entries' positions in A (-1: a pad) and columns; buses' own entries
@@ -355,22 +356,29 @@ void line_steps(const std::vector<int>& ptr, const std::vector<int4>& slots, con
         int lg, t;
         bool two;
     };
-    std::vector<Bus> best, cur;
+    struct Lane {
+        int slot, lg, li, r0;      // slot -1: idle
+        bool lead;
+    };
+    std::vector<Lane> lanes;
+    std::vector<Bus> best, cur, by_size[6];        // by lanes of a bus: 1 << 0 .. 5
     bool half = false;           // the last level took the first half of the warps
     for (size_t l = 0; l + 1 < ptr.size(); l++) {
         if (ptr[l + 1] == ptr[l]) continue;
+        int longest_row = 1;
+        for (int t = ptr[l]; t < ptr[l + 1]; t++) longest_row = std::max(longest_row, slots[t].y);
         double least = 0.0;
         best.clear();
-        for (int m = 1; m <= 64; m *= 2) {
-            cur.clear();
+        for (int m = 1; m <= 64 && m < 2 * longest_row; m *= 2) {      // beyond, a lane a row again
+            for (std::vector<Bus>& v : by_size) v.clear();
             for (int t = ptr[l]; t < ptr[l + 1]; t++) {
                 const bool two = slots[t].w >= 0;
                 int lg = 0;
                 while (lg < line_lg_max(two) && (m << lg) < slots[t].y) lg++;
-                cur.push_back({lg, t, two});
+                by_size[lg + two].push_back({lg, t, two});
             }
-            std::stable_sort(cur.begin(), cur.end(),
-                             [](const Bus& x, const Bus& y) { return x.lg + x.two > y.lg + y.two; });
+            cur.clear();
+            for (int z = 5; z >= 0; z--) cur.insert(cur.end(), by_size[z].begin(), by_size[z].end());
             double pipe[4] = {0, 0, 0, 0}, longest = 0.0;
             int lane = 0, warp = 0, e = 0, lg = 0;
             auto close = [&] {
@@ -395,11 +403,7 @@ void line_steps(const std::vector<int>& ptr, const std::vector<int4>& slots, con
             }
         }
         // lanes of the level: the bus and its row's first position, then the warps' blocks
-        struct Lane {
-            int slot, lg, li, r0;      // slot -1: idle
-            bool lead;
-        };
-        std::vector<Lane> lanes;
+        lanes.clear();
         for (const Bus& b : best) {
             const int4 s = slots[b.t];
             for (int r = 0; r < (b.two ? 2 : 1); r++)
@@ -413,24 +417,29 @@ void line_steps(const std::vector<int>& ptr, const std::vector<int4>& slots, con
         half = lanes.size() <= (size_t)NT / 2;
         while (lanes.size() % NT) lanes.push_back(idle);
         for (size_t k = 0; k < lanes.size(); k += 32) {
-            int lg = 0, cnt = 0, on = 0;
+            const int base = (int)L.map.size(), sync = k + NT >= lanes.size() ? rh::kLineSync : 0;
+            if (lanes[k].slot < 0) {                    // an idle warp: its first lane would be the first in use
+                L.steps.insert(L.steps.end(), 32, make_int4(-1, base, -1, flags | sync));
+                continue;
+            }
+            int lg = 0, cnt = 0;
             for (size_t i = k; i < k + 32; i++) {
                 if (lanes[i].slot < 0) continue;
                 const int l = lanes[i].lg;
                 lg = std::max(lg, l);
                 cnt = std::max(cnt, (slots[lanes[i].slot].y + (1 << l) - 1) >> l);
-                on = rh::kLineActive;
             }
-            const int base = (int)L.map.size();
-            const int w0 = flags | on | cnt | (lg << rh::kLineWlg) | (k + NT >= lanes.size() ? rh::kLineSync : 0);
-            for (int e = 0; e < cnt; e++)
-                for (size_t i = k; i < k + 32; i++) {
-                    const Lane& ln = lanes[i];
-                    const int at = ln.slot < 0 ? 0 : ln.li + (e << ln.lg);
-                    const bool in = ln.slot >= 0 && at < slots[ln.slot].y;
-                    L.map.push_back(in ? ln.r0 + at : -1);
-                    L.col.push_back(in ? col[ln.r0 + at] : L.pad);
+            const int w0 = flags | rh::kLineActive | cnt | (lg << rh::kLineWlg) | sync;
+            L.map.resize(base + 32 * (size_t)cnt, -1);
+            L.col.resize(base + 32 * (size_t)cnt, L.pad);
+            for (size_t i = k; i < k + 32; i++) {
+                const Lane& ln = lanes[i];
+                const int n = ln.slot < 0 ? 0 : slots[ln.slot].y;
+                for (int at = ln.li, o = base + (int)(i - k); at < n; at += 1 << ln.lg, o += 32) {
+                    L.map[o] = ln.r0 + at;
+                    L.col[o] = col[ln.r0 + at];
                 }
+            }
             for (size_t i = k; i < k + 32; i++) {
                 const Lane& ln = lanes[i];
                 int4 d = make_int4(-1, base, -1, w0);
@@ -1075,12 +1084,16 @@ rh_status rh_grid_create(const rh_grid_desc* d, int32_t device, rh_grid** out) {
                 for (const std::vector<int>* v : {&down.map, &up.vt, &down.vt}) up.map.insert(up.map.end(), v->begin(), v->end());
                 up.col.insert(up.col.end(), down.col.begin(), down.col.end());
                 g->n_line = (int)up.map.size();
+                // three device arrays: steps of both sweeps, columns and map, values and their transpose's
+                const size_t n_up = up.steps.size(), n_col = up.col.size();
+                up.steps.insert(up.steps.end(), down.steps.begin(), down.steps.end());
+                up.col.insert(up.col.end(), up.map.begin(), up.map.end());
                 RH_CUDA(g->upload(g->line_up, up.steps));
-                RH_CUDA(g->upload(g->line_down, down.steps));
+                g->line_down = g->line_up + n_up;
                 RH_CUDA(g->upload(g->line_col, up.col));
-                RH_CUDA(g->upload(g->line_map, up.map));
-                RH_CUDA(g->alloc(g->line_val, up.map.size()));
-                RH_CUDA(g->alloc(g->line_tval, up.map.size()));
+                g->line_map = g->line_col + n_col;
+                RH_CUDA(g->alloc(g->line_val, 2 * up.map.size()));
+                g->line_tval = g->line_val + up.map.size();
             }
         }
         RH_CUDA(g->upload(g->ef_ptr, efp));
