@@ -222,12 +222,12 @@ rh_status rh_hessvec(rh_grid *grid, const double *W, int64_t ldw, int32_t N,
 /*
  * Cross-instance batching: several (grid, W block) items, for instance the load
  * scenarios of one topology (each its own rh_grid with its own state) or
- * requests on grids of different sizes, computed by ONE kernel launch on
- * `stream` (asynchronous).  Items are independent; item i gets
- * ceil(N_i / width) CTAs (width = target directions per CTA, the right-hand-
- * side interleave width; 0 spreads the items so that they end together, which may
- * put the items on the largest grids in a launch of their own beside the others').
- * Up to 32 items per launch; larger batches take several launches.
+ * requests on grids of different sizes, computed together on `stream`
+ * (asynchronous).  Items are independent; item i gets
+ * ceil(N_i / width) CTAs of one launch (width = target directions per CTA, the
+ * right-hand-side interleave width; 0 spreads the items so that they end together,
+ * which may put the items on the largest grids in a second launch beside it).
+ * Up to 32 items at a time; larger batches take their turn.
  *   grid    adjoint-ready grid (rh_adjoint for its current state); all items
  *           must be on the same device
  *   W, HW   DEVICE pointers, n_p x N column-major (ldw, ldhw >= n_p of the grid)

@@ -103,7 +103,7 @@ struct rh_grid {
     std::vector<int> colmap;                    // host copy
     std::map<int, rh::ReachSched*> reach_dev;   // device structs, keyed by the launch's CTA count
     int *tp_bus = nullptr, *uth = nullptr, *uv = nullptr, *inc_ptr = nullptr;
-    int* tp_l0 = nullptr;   // per bus: position of (v, theta) in At for a PQ bus of forward level 0, else -1
+    int* tp_l0 = nullptr;   // per bus: position of (v, theta) in Atd for a PQ bus of forward level 0, else -1
     int *inc_uth = nullptr, *inc_uv = nullptr, *gref_row = nullptr, *pg_row = nullptr, *xmap = nullptr;
     uint8_t* has_gref = nullptr;
     int n_inc = 0, n_gref = 0;

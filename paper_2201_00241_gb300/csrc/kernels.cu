@@ -1181,17 +1181,14 @@ __device__ __forceinline__ void split_sum(int ks, bool wtwo, double& s0, double&
 // warp-uniform choice of the two-row path (lanes that left the item loop do not vote)
 __device__ __forceinline__ bool warp_any(bool p) { return __any_sync(__activemask(), p); }
 
-// forward sweep over the L pattern: x_q = (b_q - sum_{c<q} v_qc x_c) [* 1/u_qq]
-template <bool SCALE, bool TWO>
+// forward sweep over the L pattern: x_q = b_q - sum_{c<q} v_qc x_c
+template <bool TWO>
 __device__ __forceinline__ void fwd_finish(const DirGrid& g, const double* __restrict__ vals, double* X, int64_t ld,
                                            int64_t c, int q, bool two, int pos_vt, double a0, double a1) {
-    double x0 = SCALE ? a0 * g.invdiag[q] : a0;
-    stx(X, q, ld, c, x0, g.n_x);
+    stx(X, q, ld, c, a0, g.n_x);
     if constexpr (TWO) {
-        a1 = fma(-vals[pos_vt], x0, a1);
-        const double i1 = (SCALE && two) ? g.invdiag[q + 1] : 1.0;
-        const double x1 = SCALE ? a1 * i1 : a1;
-        if (two) stx(X, q + 1, ld, c, x1, g.n_x);
+        a1 = fma(-vals[pos_vt], a0, a1);
+        if (two) stx(X, q + 1, ld, c, a1, g.n_x);
     }
 }
 
@@ -1216,7 +1213,7 @@ __device__ __forceinline__ void mask_bus(unsigned* m, int enc) {
     mask_set(m, enc >> 1);
     if (enc & 1) mask_set(m, (enc >> 1) + 1);
 }
-template <bool SCALE, bool EXT = false, bool CMASK = false>
+template <bool EXT = false, bool CMASK = false>
 __device__ void sweep_fwd(const DirGrid& g, const LevelSet& ls, const double* __restrict__ vals, double* X,
                           int64_t ld, int c0, int D, double* part, unsigned* mask = nullptr,
                           const unsigned* seed = nullptr, const unsigned* cmask = nullptr) {
@@ -1250,12 +1247,12 @@ __device__ void sweep_fwd(const DirGrid& g, const LevelSet& ls, const double* __
                         stx(X, q, ld, c, a0, g.n_x);
                         if (two) stx(X, q + 1, ld, c, a1, g.n_x);
                     } else {
-                        fwd_finish<SCALE, true>(g, vals, X, ld, c, q, two, rpv + n, a0, a1);
+                        fwd_finish<true>(g, vals, X, ld, c, q, two, rpv + n, a0, a1);
                     }
                 } else {
                     block_sub<false, CMASK>(g.col, vals, rp, rpv, 0, n, X, ld, c, a0, a1, cmask, g.n_x);
                     if (EXT) stx(X, q, ld, c, a0, g.n_x);
-                    else fwd_finish<SCALE, false>(g, vals, X, ld, c, q, two, rpv + n, a0, a1);
+                    else fwd_finish<false>(g, vals, X, ld, c, q, two, rpv + n, a0, a1);
                 }
                 if (mask) mask_bus(mask, g.bparent[q]);
             }
@@ -1289,9 +1286,9 @@ __device__ void sweep_fwd(const DirGrid& g, const LevelSet& ls, const double* __
                     stx(X, q, ld, c, a0, g.n_x);
                     if (two) stx(X, q + 1, ld, c, a1, g.n_x);
                 } else if (two) {
-                    fwd_finish<SCALE, true>(g, vals, X, ld, c, q, two, rpv + n, a0, a1);
+                    fwd_finish<true>(g, vals, X, ld, c, q, two, rpv + n, a0, a1);
                 } else {
-                    fwd_finish<SCALE, false>(g, vals, X, ld, c, q, two, rpv + n, a0, a1);
+                    fwd_finish<false>(g, vals, X, ld, c, q, two, rpv + n, a0, a1);
                 }
                 if (mask) mask_bus(mask, g.bparent[q]);
             }
@@ -1300,21 +1297,18 @@ __device__ void sweep_fwd(const DirGrid& g, const LevelSet& ls, const double* __
     }
 }
 
-// backward sweep over the U pattern: x_q = (b_q - sum_{c>q} v_qc x_c) [* 1/u_qq]
-template <bool SCALE, bool TWO>
+// backward sweep over the U pattern: x_q = b_q - sum_{c>q} v_qc x_c
+template <bool TWO>
 __device__ __forceinline__ void bwd_finish(const DirGrid& g, const double* __restrict__ vals, double* X, int64_t ld,
                                            int64_t c, int q, bool two, int pos_tv, double a0, double a1) {
     if constexpr (TWO) {
-        const double i1 = (SCALE && two) ? g.invdiag[q + 1] : 1.0;
-        const double x1 = SCALE ? a1 * i1 : a1;
-        if (two) stx(X, q + 1, ld, c, x1, g.n_x);
-        a0 = fma(-vals[pos_tv], two ? x1 : 0.0, a0);
+        if (two) stx(X, q + 1, ld, c, a1, g.n_x);
+        a0 = fma(-vals[pos_tv], two ? a1 : 0.0, a0);
     }
-    stx(X, q, ld, c, SCALE ? a0 * g.invdiag[q] : a0, g.n_x);
+    stx(X, q, ld, c, a0, g.n_x);
 }
 
 // rmask (optional): right-hand side rows whose bit is clear are zero and are not read
-template <bool SCALE>
 __device__ void sweep_bwd(const DirGrid& g, const LevelSet& ls, const double* __restrict__ vals, double* X,
                           int64_t ld, int c0, int D, double* part, const unsigned* rmask = nullptr) {
     for (int lev = 0; lev < ls.n_lev; lev++) {
@@ -1341,10 +1335,10 @@ __device__ void sweep_bwd(const DirGrid& g, const LevelSet& ls, const double* __
                 double a1 = (two && has_b && inb(q + 1, g.n_x)) ? X[(int64_t)(q + 1) * ld + c] : 0.0;
                 if (warp_any(two)) {
                     block_sub<true>(g.col, vals, ue0, ue1, 0, n, X, ld, c, a0, a1, nullptr, g.n_x);
-                    bwd_finish<SCALE, true>(g, vals, X, ld, c, q, two, ue0 - 1, a0, a1);
+                    bwd_finish<true>(g, vals, X, ld, c, q, two, ue0 - 1, a0, a1);
                 } else {
                     block_sub<false>(g.col, vals, ue0, ue1, 0, n, X, ld, c, a0, a1, nullptr, g.n_x);
-                    bwd_finish<SCALE, false>(g, vals, X, ld, c, q, two, ue0 - 1, a0, a1);
+                    bwd_finish<false>(g, vals, X, ld, c, q, two, ue0 - 1, a0, a1);
                 }
                 bi = bi2;
             }
@@ -1372,8 +1366,8 @@ __device__ void sweep_bwd(const DirGrid& g, const LevelSet& ls, const double* __
                 else strided_sub<false, false>(g.col, vals, ue0, ue1, sli, n, ks, X, ld, c, s0, s1, nullptr, g.n_x);
                 split_sum(ks, wtwo, s0, s1);
                 if (!fin) continue;
-                if (two) bwd_finish<SCALE, true>(g, vals, X, ld, c, q, two, ue0 - 1, b0 + s0, b1 + s1);
-                else bwd_finish<SCALE, false>(g, vals, X, ld, c, q, two, ue0 - 1, b0 + s0, b1 + s1);
+                if (two) bwd_finish<true>(g, vals, X, ld, c, q, two, ue0 - 1, b0 + s0, b1 + s1);
+                else bwd_finish<false>(g, vals, X, ld, c, q, two, ue0 - 1, b0 + s0, b1 + s1);
             }
         }
         __syncthreads();
@@ -1382,9 +1376,8 @@ __device__ void sweep_bwd(const DirGrid& g, const LevelSet& ls, const double* __
 
 // Dense trailing block [t0, t0 + T) of a sweep, column-oriented in shared memory.
 // xt[i * D + d] holds row t0 + i of the CTA's directions; tri_g is the packed
-// strictly-triangular block (column j contiguous), columns pre-scaled by 1/u_jj
-// for the scaled sweeps, so each column step is y_i -= tri_ij y_j and the
-// result is x_i = y_i [* 1/u_ii].  One barrier per column.  With tri != NULL the
+// strictly-triangular block (column j contiguous); each column step is
+// y_i -= tri_ij y_j.  With tri != NULL the
 // triangle is first staged in shared memory (one CTA per SM); with tri == NULL
 // it is read through L1, where it is shared by all the CTAs of the SM.
 __device__ __forceinline__ int lpack_off(int j, int T) { return j * (T - 1) - j * (j - 1) / 2; }  // rows j+1..T-1
@@ -1400,7 +1393,7 @@ constexpr int kTailB = 16;
 __device__ __forceinline__ double tri_l(const double* src, int T, int i, int j) { return src[lpack_off(j, T) + (i - j - 1)]; }
 __device__ __forceinline__ double tri_u(const double* src, int i, int j) { return src[upack_off(j) + i]; }
 
-template <bool SCALE, class Grid>
+template <class Grid>
 __device__ void tail_fwd(const Grid& g, const double* __restrict__ tri_g, double* X, int64_t ld, int c0, int D,
                          double* xt, double* tri) {
     const int T = g.T, t0 = g.t0;
@@ -1446,13 +1439,12 @@ __device__ void tail_fwd(const Grid& g, const double* __restrict__ tri_g, double
     }
     for (int it = threadIdx.x; it < T * D; it += blockDim.x) {
         int i = it / D, d = it - i * D;
-        double v = xt[it];
-        X[(int64_t)(t0 + i) * ld + c0 + d] = SCALE ? v * g.invdiag[t0 + i] : v;
+        X[(int64_t)(t0 + i) * ld + c0 + d] = xt[it];
     }
     __syncthreads();
 }
 
-template <bool SCALE, class Grid>
+template <class Grid>
 __device__ void tail_bwd(const Grid& g, const double* __restrict__ tri_g, double* X, int64_t ld, int c0, int D,
                          double* xt, double* tri) {
     const int T = g.T, t0 = g.t0;
@@ -1498,8 +1490,7 @@ __device__ void tail_bwd(const Grid& g, const double* __restrict__ tri_g, double
     }
     for (int it = threadIdx.x; it < T * D; it += blockDim.x) {
         int i = it / D, d = it - i * D;
-        double v = xt[it];
-        X[(int64_t)(t0 + i) * ld + c0 + d] = SCALE ? v * g.invdiag[t0 + i] : v;
+        X[(int64_t)(t0 + i) * ld + c0 + d] = xt[it];
     }
     __syncthreads();
 }
@@ -1738,24 +1729,24 @@ __device__ __forceinline__ void dirs_body(const DirGrid& g, const DirLaunch& L, 
                 const ReachSched& R = *L.reach;
                 const int m0 = R.lev0[cta];
                 const LevelSet rs = {R.nlev[cta], R.ptr + m0 + cta, R.slots, R.maxext + m0};
-                sweep_fwd<false, false, true>(g, rs, g.Ad, V, ld, 0, D, part, nullptr, seed, mask);
-                sweep_fwd<false, true, true>(g, g.ef, g.Ad, V, ld, 0, D, part, nullptr, nullptr, mask);
+                sweep_fwd<false, true>(g, rs, g.Ad, V, ld, 0, D, part, nullptr, seed, mask);
+                sweep_fwd<true, true>(g, g.ef, g.Ad, V, ld, 0, D, part, nullptr, nullptr, mask);
             } else if (mask) {
-                sweep_fwd<false, false, true>(g, g.sf, g.Ad, V, ld, 0, D, part, mask, seed, mask);
-                sweep_fwd<false, true, true>(g, g.ef, g.Ad, V, ld, 0, D, part, nullptr, nullptr, mask);
+                sweep_fwd<false, true>(g, g.sf, g.Ad, V, ld, 0, D, part, mask, seed, mask);
+                sweep_fwd<true, true>(g, g.ef, g.Ad, V, ld, 0, D, part, nullptr, nullptr, mask);
             } else {
-                sweep_fwd<false>(g, g.sf, g.Ad, V, ld, 0, D, part);
-                sweep_fwd<false, true>(g, g.ef, g.Ad, V, ld, 0, D, part);
+                sweep_fwd(g, g.sf, g.Ad, V, ld, 0, D, part);
+                sweep_fwd<true>(g, g.ef, g.Ad, V, ld, 0, D, part);
             }
-            tail_fwd<false>(g, g.triLd, V, ld, 0, D, part, nullptr);
+            tail_fwd(g, g.triLd, V, ld, 0, D, part, nullptr);
         }
         if (L.phases & PH_U) {
-            tail_bwd<false>(g, g.triUd, V, ld, 0, D, part, nullptr);
-            sweep_bwd<false>(g, g.sb, g.Ad, V, ld, 0, D, part, mask);
+            tail_bwd(g, g.triUd, V, ld, 0, D, part, nullptr);
+            sweep_bwd(g, g.sb, g.Ad, V, ld, 0, D, part, mask);
         }
     } else {
-        if (L.phases & PH_L) sweep_fwd<false>(g, g.lf, g.Ad, V, ld, 0, D, part);
-        if (L.phases & PH_U) sweep_bwd<false>(g, g.lb, g.Ad, V, ld, 0, D, part);
+        if (L.phases & PH_L) sweep_fwd(g, g.lf, g.Ad, V, ld, 0, D, part);
+        if (L.phases & PH_U) sweep_bwd(g, g.lb, g.Ad, V, ld, 0, D, part);
     }
     const bool fold_ut = (L.phases & PH_TPROJ) && (L.phases & PH_UT) && L.use_tail && g.sf.n_lev > 0;
     if (L.phases & PH_TPROJ) {
@@ -1770,18 +1761,18 @@ __device__ __forceinline__ void dirs_body(const DirGrid& g, const DirLaunch& L, 
                 sf.ptr += 1;
                 sf.maxext += 1;
             }
-            sweep_fwd<false>(g, sf, g.Atd, T, ld, 0, D, part);
-            sweep_fwd<false, true>(g, g.ef, g.Atd, T, ld, 0, D, part);
-            tail_fwd<false>(g, g.triUtd, T, ld, 0, D, part, nullptr);
+            sweep_fwd(g, sf, g.Atd, T, ld, 0, D, part);
+            sweep_fwd<true>(g, g.ef, g.Atd, T, ld, 0, D, part);
+            tail_fwd(g, g.triUtd, T, ld, 0, D, part, nullptr);
         }
         if (L.phases & PH_LT) {
             // psi is only read by SpMulAdd here: rows outside J_p and its ancestors are skipped
-            tail_bwd<false>(g, g.triLtd, T, ld, 0, D, part, nullptr);
-            sweep_bwd<false>(g, (L.phases & PH_MULADD) ? g.sbr : g.sb, g.Atd, T, ld, 0, D, part);
+            tail_bwd(g, g.triLtd, T, ld, 0, D, part, nullptr);
+            sweep_bwd(g, (L.phases & PH_MULADD) ? g.sbr : g.sb, g.Atd, T, ld, 0, D, part);
         }
     } else {
-        if (L.phases & PH_UT) sweep_fwd<false>(g, g.lf, g.Atd, T, ld, 0, D, part);
-        if (L.phases & PH_LT) sweep_bwd<false>(g, g.lb, g.Atd, T, ld, 0, D, part);
+        if (L.phases & PH_UT) sweep_fwd(g, g.lf, g.Atd, T, ld, 0, D, part);
+        if (L.phases & PH_LT) sweep_bwd(g, g.lb, g.Atd, T, ld, 0, D, part);
     }
     if (L.phases & PH_MULADD) {
         for (int k = threadIdx.x; k < g.n_p; k += blockDim.x) {
@@ -2039,8 +2030,8 @@ __device__ __forceinline__ void k_solve1_body(const LineGrid& g, const double* x
     __syncthreads();
     line_sweep<true, NT>(trans ? g.tup : g.up, X, g.n_x);
     if (use_tail) {
-        tail_fwd<false>(g, trans ? g.triUtd : g.triLd, X, 1, 0, 1, part, tri);
-        tail_bwd<false>(g, trans ? g.triLtd : g.triUd, X, 1, 0, 1, part, tri);
+        tail_fwd(g, trans ? g.triUtd : g.triLd, X, 1, 0, 1, part, tri);
+        tail_bwd(g, trans ? g.triLtd : g.triUd, X, 1, 0, 1, part, tri);
     }
     line_sweep<false, NT>(trans ? g.tdown : g.down, X, g.n_x);
     __syncthreads();
@@ -2093,8 +2084,8 @@ __device__ __forceinline__ void dir1_body(const DirGrid& g, const LineGrid& s, c
         __syncthreads();
         line_sweep<true, NT>(s.up, X, g.n_x);
         if (use_tail) {
-            tail_fwd<false>(s, s.triLd, X, 1, 0, 1, part, tri);
-            tail_bwd<false>(s, s.triUd, X, 1, 0, 1, part, tri);
+            tail_fwd(s, s.triLd, X, 1, 0, 1, part, tri);
+            tail_bwd(s, s.triUd, X, 1, 0, 1, part, tri);
         }
         line_sweep<false, NT>(s.down, X, g.n_x);
         __syncthreads();
@@ -2170,8 +2161,8 @@ __device__ __forceinline__ void dir1_body(const DirGrid& g, const LineGrid& s, c
     __syncthreads();
     line_sweep<true, NT>(s.tup, X, g.n_x);
     if (use_tail) {
-        tail_fwd<false>(s, s.triUtd, X, 1, 0, 1, part, tri);
-        tail_bwd<false>(s, s.triLtd, X, 1, 0, 1, part, tri);
+        tail_fwd(s, s.triUtd, X, 1, 0, 1, part, tri);
+        tail_bwd(s, s.triLtd, X, 1, 0, 1, part, tri);
     }
     line_sweep<false, NT>(s.tdown, X, g.n_x);
     __syncthreads();
@@ -2658,7 +2649,7 @@ void launch_transpose_values(int nnz, const int* tpos, const int* arow, const in
 }
 
 // SMs of the current device (1 if the query fails)
-static int num_sms() {
+int num_sms() {
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return 1;
     std::lock_guard<std::mutex> lock(g_dev_mu);

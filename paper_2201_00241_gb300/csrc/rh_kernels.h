@@ -69,7 +69,7 @@ struct DirGrid {
     int n_bus;
     const int *tp_bus;                         // bus processing order (internal order, slack last)
     const int *uth, *uv;                       // rows of theta_b (zero row at the slack) and v_b
-    const int *tp_l0;                          // position of (v, theta) in At for a PQ bus of forward level 0, else -1
+    const int *tp_l0;                          // position of (v, theta) in Atd for a PQ bus of forward level 0, else -1
     const int *inc_ptr, *inc_uth, *inc_uv;     // incident branches: rows of the other end
     const double4_32a *inc_coef;               // (K, -a, b, -c) per incidence (state dependent)
     const double *d2, *asum, *csum;            // per-bus coefficients (state dependent)
@@ -414,7 +414,7 @@ void launch_pf_prep_batch(const PfBatch& B, cudaStream_t st);
 void launch_batch_status(const PfBatch& B, double* out, cudaStream_t st);
 cudaError_t launch_refactor_batch(const RfBatch& B, const int* lev_ptr_host, const int64_t* tgt_lev_ptr_host,
                                   const int* piv_lev_ptr_host, int n_lev, cudaStream_t st);
-// the dense tail's triangles of the single solves (L, and U with columns scaled by 1/u_jj)
+// the dense tail's triangles of the single solves (L'' and U')
 void launch_tail_tri_batch(const TriBatch& B, cudaStream_t st);
 cudaError_t launch_solve1_batch(const Solve1Batch& B, bool use_tail, int n_x, int T, cudaStream_t st);
 void launch_newton_update_batch(const PfBatch& B, bool chained, cudaStream_t st);
@@ -430,6 +430,7 @@ int dirs_cta_slots_for(int n_sm);
 int dirs_ctas_for(int N, int slots);
 // CTAs of k_dirs the device holds at once (CTAs per SM x SMs)
 int dirs_cta_slots();
+int num_sms();             // SMs of the current device (1 if the query fails)
 
 // adjoint helpers
 struct AdjData {

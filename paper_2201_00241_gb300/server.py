@@ -14,10 +14,10 @@ Admission is by memory footprint and size class: the oldest waiting request open
 the next free arena's round, and waiting requests of grids of a comparable size
 (n_x within mix_ratio) join it, in arrival order, while their W, HW and workspace
 fit in it (a request that does not fit waits for a later round; one larger than
-an arena is refused).  A round's requests all complete with its one launch, so a
+an arena is refused).  A round's requests all complete with that one call, so a
 small request never waits there for a grid many times larger.
 A round is then three operations on its stream: one copy of all its W blocks to
-the device, ONE rh_batch_hessvec launch over all its requests (cross-instance
+the device, ONE rh_batch_hessvec call over all its requests (cross-instance
 batching: grids of different sizes and widths in one kernel), and one copy of
 all its HW blocks back.  Rounds on different streams overlap on the device while
 new requests keep arriving (continuous batching, not a queue drained one
