@@ -804,10 +804,6 @@ cudaError_t potrf_tiles(int n, double* A, int64_t lda, int* info, double* y, cud
     return cudaGetLastError();
 }
 
-// A panel launch has (1 + strips) CTAs per right-hand side; strips of 8 rows end sooner,
-// strips of 32 need fewer CTAs.
-constexpr int kSolveCtas = 152;
-
 // Every CTA of a panel launch solves its panel, so the panels lose where right-hand sides
 // already fill the GPU, and for orders of one or two panels.  Measured, tiles -> panels, us
 // for both sweeps: 1019 x 1 403 -> 252, x 3 408 -> 277, x 16 505 -> 405, x 32 511 -> 657;
@@ -818,11 +814,13 @@ bool by_panels(int n, int nrhs) { return n > 128 && nrhs <= 16 && (int64_t)n * n
 template <bool FWD>
 cudaError_t panel_sweep(int n, const double* L, int64_t ldl, double* B, int64_t ldb, int nrhs, double* W, bool pdl,
                         cudaStream_t s) {
-    const int np = (n + kPN - 1) / kPN;
+    const int np = (n + kPN - 1) / kPN, sms = num_sms();
     for (int i = 0; i < np; i++) {
         const int p = FWD ? i : np - 1 - i;
         const int rows = FWD ? (n > (p + 1) * kPN ? n - (p + 1) * kPN : 0) : p * kPN;
-        const bool narrow = (int64_t)(1 + (rows + 7) / 8) * nrhs <= kSolveCtas;
+        // (1 + strips) CTAs per right-hand side: strips of 8 rows end sooner while each CTA has an
+        // SM of its own, strips of 32 need fewer CTAs
+        const bool narrow = (int64_t)(1 + (rows + 7) / 8) * nrhs <= sms;
         const dim3 grid(1 + (narrow ? (rows + 7) / 8 : (rows + 31) / 32), (unsigned)nrhs);
         const cudaError_t e = launch_pdl(pdl, narrow ? k_chol_panel<FWD, 8> : k_chol_panel<FWD, 32>, grid,
                                          dim3(kDenseThreads), 0, s, n, L, ldl, B, ldb, W, p);
