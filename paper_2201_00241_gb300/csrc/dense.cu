@@ -33,11 +33,11 @@
 // elimination, as in Bareiss's fraction-free Gaussian elimination, with an exact
 // power-of-two rescaling in place of Bareiss's exact division).  The trailing
 // block after step j is then s_{j+1} times the ordinary Schur complement, with
-// s_{j+1} = s_j 2^-e_j d_j, within about 2^+-128 (see pivot_shift).  At the
-// end l_rc = a_rc / sqrt(s_c d_c) for r >= c (d_c = a_cc), one reciprocal
-// square root per column, and 1 / l_cc = s_c / sqrt(s_c d_c) and
-// 1 / d_c = s_c / (s_c d_c) follow by multiplications.  A step is one FMA and an
-// exponent update on the critical path instead of a division.  GB300 runs FP64
+// s_{j+1} = s_j 2^-e_j d_j (bounds: see pivot_shift).  At the end
+// l_rc = a_rc / sqrt(s_c d_c) for r >= c (d_c = a_cc), one reciprocal square root
+// per column, and 1 / l_cc = s_c / sqrt(s_c d_c) and 1 / d_c = s_c / (s_c d_c)
+// follow by multiplications.  A step is one FMA on the critical path, and far from
+// 1 an exponent update, instead of a division.  GB300 runs FP64
 // on the CUDA cores (the tensor cores have no fast FP64 mode) at one warp
 // instruction per 64 cycles per SM sub-partition, and a dependent FP64
 // instruction waits those 64 cycles, so every step also keeps its FP64 work on

@@ -185,10 +185,19 @@ __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.lau
 // tail LU, the tracking step's Cholesky) are eliminated by cross-multiplied steps
 // a_rc <- 2^-e (d a_rc - a_rj a_jc), d the current pivot, instead of a reciprocal of
 // every pivot on the critical path.  e is 0 while d lies within 2^+-64 and otherwise the
-// power of two that brings |d| into [1, 2): the values then stay within about 2^+-200 of
-// the tile's own, and most steps do not carry the exponent update (12 dependent integer
-// instructions) in their chain.  A 16 x 16 tile of the tail's LU: 8300 cycles with the
-// update, the own entry and its indexes in every step, 6000 without.
+// power of two that brings |d| into [1, 2): most steps do not carry the exponent update (12
+// dependent integer instructions) in their chain.  A 16 x 16 tile of the tail's LU: 8300
+// cycles with the update, the own entry and its indexes in every step, 6000 without.
+//
+// The trailing block after j steps is s_j times the ordinary one, s_0 = 1 and s_{j+1} =
+// s_j d_j 2^-e with d_j = s_j u_j, u_j the ordinary pivot.  A rescaled step takes |s| up by
+// less than a factor 2; any other leaves |s_{j+1}| = d_j^2 / |u_j| between 2^-128 / max|u|
+// and 2^130 / min|u|.  So |s| < 2^(130 + TB) max(1, 1 / min|u|) in a tile of TB columns, and
+// no product of a step overflows while the entries a of the tile and its Schur complements
+// have max|a| < 2^350 min(1, min|u|) (TB = 32).  An equilibrated Cholesky tile has |a| < 4:
+// pivots down to 2^-348.  The tail's LU tiles are not equilibrated: its pivots are at least
+// 1e-14 max|J_x|, or the factorisation is reported singular, which leaves its entries a
+// growth of 2^300 over a max|J_x| of up to 1.
 // e for a pivot d: 0 also where d is zero, subnormal, infinite or NaN and the
 // factorisation has failed (|e| <= 1022, so 2^-e is normal).
 __device__ __forceinline__ int pivot_shift(double d) {
