@@ -2099,6 +2099,7 @@ rh_status rh_solve(rh_grid* g, double* R, int64_t ldr, int32_t nrhs, int32_t tra
     if (g->copies_behind || cs != cudaStreamCaptureStatusNone) {
         rh::LineCopies o = {g->tail_pos, g->Ad, g->Atd, g->triLd, g->triUd, g->triUtd, g->triLtd};
         RH_CUDA(rh::launch_copies_from_lines(g->s1(), o, rh::solve1_mode(S.n_x, S.n_x - S.t0) == 2, s));
+        if (cs == cudaStreamCaptureStatusNone) g->copies_behind = false;
     }
     rh::launch_scatter_rows(S.n_x, nrhs, g->xmap, Rd, lr, g->V, nrhs, 1.0, S.n_x, s);
     // unit-diagonal factors (J_x = D L'' U'): D^-1 R in, or D^-1 out for the transpose

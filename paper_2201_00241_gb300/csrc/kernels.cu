@@ -1972,7 +1972,9 @@ __global__ void k_line_values(const __grid_constant__ LineGrid g) {
 // triLd and triUd, or, where every level is swept (use_tail 0), in `line` too.  Writes what
 // k_transpose_values and k_build_tail write from the same factors (Ad, Atd and the tail's
 // triangles; inside the tail up to the order of two multiplications).  A holds the next
-// Jacobian by then.
+// Jacobian by then.  One thread an entry, bound by the latency of its loads and scattered
+// stores: 7 us at 118 and 1354 buses, 35 us at 9241 (320 k threads), for the first solve
+// after a power flow instead of in each of its Newton steps.
 __global__ void k_copies_from_lines(const __grid_constant__ LineGrid g, const __grid_constant__ LineCopies o,
                                     int use_tail) {
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
